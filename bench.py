@@ -76,7 +76,7 @@ def peaks():
 # holds only for the kernel built from files with the recorded digest: after
 # any change to them the bench reports null until the kernel is captured again.
 AX_SOURCES = tuple(os.path.join("paper_2107_01243_gb300", "csrc", f) for f in (
-    "ax_df.cu", "df.cuh", "df_tables.cuh", "ax_tile.cuh", "tma.cuh", "reduce.cuh",
+    "ax_df.cu", "df_tile.cuh", "df.cuh", "df_tables.cuh", "ax_tile.cuh", "tma.cuh", "reduce.cuh",
     "cg_state.cuh"))
 
 

@@ -619,6 +619,8 @@ static CGState read_state(const CGState* d, cudaStream_t s, int* dev_err = nullp
   return *pin.p;
 }
 
+constexpr int kResidentIters = 512;     // iterations per launch of the grid-resident CG
+
 template <class T>
 struct PcgArgs {
   const OpData<T>* op;
@@ -764,14 +766,49 @@ static CGState run_pcg_loop(sem_handle* h, CGState* st, const sem_solve_opts& o,
   return hs;
 }
 
+static void ensure(DevBuf<double>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
+static void ensure(DevBuf<float>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
+
+// Whether the grid-resident iterations (resident.cu) run this solve: below
+// about a million local points they win at every order and precision, above
+// it the streaming kernels do (microseconds an iteration, resident / one kernel
+// per stage: 12^3 elements, N = 7, FP64 54.5 / 65.5 and FP32 19.6 / 34.4; 10^3,
+// N = 9, FP64 76.6 / 89.7; 12^3, N = 9, FP64 134.8 / 125.9; 16^3, N = 7, FP64
+// 129.0 / 107.1 and FP32 55.4 / 43.4).
+constexpr int64_t kResidentPoints = 1 << 20;
+
+template <class T>
+static bool resident_ok(const sem_handle* h, const T* h1f) {
+  if (h->nL > kResidentPoints) return false;
+  if (h->mult_replaced) return false;       // its dots count the handle's own copies
+  if (sizeof(T) == 8 && h->f64_kernel == SEM_F64_KERNEL_DOUBLEFLOAT &&
+      !df_ax_supported(h, nullptr, nullptr, h1f))
+    return false;                           // launch_ax reports the unsupported combination
+  return true;
+}
+
 template <class T>
 static CGState run_pcg(sem_handle* h, const PcgArgs<T>& a, const sem_solve_opts& o,
                        cudaStream_t s) {
+  if (resident_ok<T>(h, a.h1f)) {
+    T *vs, *w2;
+    if constexpr (std::is_same<T, double>::value) {
+      ensure(h->res_s, h->nL); ensure(h->res_w2, h->nL);
+      vs = h->res_s.ptr; w2 = h->res_w2.ptr;
+    } else {
+      ensure(h->res_s32, h->nL); ensure(h->res_w232, h->nL);
+      vs = h->res_s32.ptr; w2 = h->res_w232.ptr;
+    }
+    const PcgVecs<T> v{a.x, a.r, a.p, vs, a.w, w2, a.dinv, a.h1f, a.h1, a.h2, a.st};
+    CGState hs;
+    do {
+      launch_resident<T>(h, v, kResidentIters, s);
+      hs = read_state(a.st, s, h->dev_err.ptr);
+    } while (!hs.done);
+    return hs;
+  }
   return run_pcg_loop(h, a.st, o, s, [&](int count) { pcg_iterations<T>(h, a, count, s); });
 }
-
-static void ensure(DevBuf<double>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
-static void ensure(DevBuf<float>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
 
 // Jacobi inverse diagonal for (h1 | h1_field, h2): mask / QQ^T diag(H_L)
 static void ensure_dinv(sem_handle* h, double h1, double h2, const double* h1f, bool need32,
@@ -920,7 +957,9 @@ static void solve_mixed(sem_handle* h, const double* b, double* x, const sem_sol
                         sem_solve_info& info, cudaStream_t s) {
   const int64_t n = h->nL;
   if (!h->f32.G.ptr) throw Error(SEM_ERR_STATE, "mixed solve needs FP32 geometry (SEM_PREC_F32)");
-  const bool glob = h->inner_vectors != SEM_INNER_LOCAL && !o.h1_field && glob_supported(h);
+  // AUTO: small problems iterate grid-resident on L-vectors
+  const bool glob = h->inner_vectors != SEM_INNER_LOCAL && !o.h1_field && glob_supported(h) &&
+                    !(h->inner_vectors == SEM_INNER_AUTO && resident_ok<float>(h, nullptr));
   ensure(h->r, n); ensure(h->w, n);
   if (!glob) {
     ensure(h->r32, n); ensure(h->p32, n); ensure(h->w32, n); ensure(h->x32, n);

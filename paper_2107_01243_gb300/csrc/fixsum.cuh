@@ -1,0 +1,126 @@
+// Order-independent sums of doubles in integer arithmetic, for the latency-bound
+// reductions of resident.cu.  GB300 issues one FP64 instruction of a warp in
+// 64 cycles per scheduler, so a shuffle tree of FP64 adds over a CTA and then
+// over the grid cost 3 to 5 us; here every value becomes a 57-bit integer on
+// the scale of the largest one, warps add with redux.sync, and only the final
+// total is rounded to a double (to nearest).  Values are truncated at 2^-57
+// of the largest of their warp (FP64 addition rounds at 2^-53 of the partial
+// sum), and the result does not depend on the order of the additions.
+#pragma once
+#include <stdint.h>
+
+namespace sem {
+
+__host__ __device__ inline int min_int(int a, int b) { return a < b ? a : b; }
+
+// m 2^(e - 1079), e the biased FP64 exponent of the scale; e = kFxBad: Inf or NaN
+struct FxVal {
+  long long m;
+  int e;
+};
+constexpr int kFxBad = 0x7FF;
+
+// biased exponent of a double (1 for zero and subnormals)
+__host__ __device__ inline int fx_exp(unsigned long long bits) {
+  const int ex = (int)((bits >> 52) & 0x7FF);
+  return ex ? ex : 1;
+}
+
+// the double on the scale e >= its own exponent (finite values), truncated
+__host__ __device__ inline long long fx_mant(unsigned long long bits, int e) {
+  unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
+  const int ex = (int)((bits >> 52) & 0x7FF);
+  if (ex) m |= 1ull << 52;
+  const int sh = e - (ex ? ex : 1);
+  m = sh < 58 ? (m << 4) >> sh : 0ull;
+  return (bits >> 63) ? -(long long)m : (long long)m;
+}
+
+// (hi 2^32 + lo) 2^(e - 1079) as a double, lo >= 0: rounded to nearest from its
+// leading 64 bits
+__host__ __device__ inline double fx_round(long long hi, long long lo, int e) {
+  hi += lo >> 32;
+  unsigned l = (unsigned)lo;
+  const bool neg = hi < 0;
+  if (neg) {
+    l = 0u - l;
+    hi = ~hi + (l == 0u ? 1 : 0);
+  }
+  unsigned long long m = (unsigned long long)hi, bits = neg ? 1ull << 63 : 0ull;
+  if (e >= kFxBad) {
+    bits = 0x7FF8000000000000ull;
+  } else if (m | l) {
+    // the leading 64 bits, bit 63 set; ex: the biased exponent of bit 63
+#ifdef __CUDA_ARCH__
+    const int n = m ? __clzll((long long)m) : 32 + __clz((int)l) + 32;
+#else
+    const int n = m ? __builtin_clzll(m) : 64 + __builtin_clz(l);
+#endif
+    if (m) m = (m << n) | (n >= 32 ? (unsigned long long)l << (n - 32) : (unsigned long long)(l >> (32 - n)) * (n != 0));
+    else m = (unsigned long long)l << (n - 32);
+    int ex = e + 95 - n - 56;
+    int sh = 11;
+    if (ex < 1) {                         // subnormal
+      sh = min_int(11 + 1 - ex, 64);
+      ex = 0;
+    }
+    const unsigned long long half = (m >> (sh - 1)) & 1ull;
+    m = (sh < 64 ? m >> sh : 0ull) + half;   // up to 2^53: the carry moves the exponent
+    if (ex == 0) bits |= m;                  // 2^52: the smallest normal number
+    else if (ex >= kFxBad) bits |= 0x7FF0000000000000ull;
+    else bits |= ((unsigned long long)(ex - 1) << 52) + m;
+  }
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)bits);
+#else
+  double d;
+  __builtin_memcpy(&d, &bits, 8);
+  return d;
+#endif
+}
+
+#ifdef __CUDACC__
+// sum over the warp of 64-bit integers, exact; the result in every lane
+// (three redux.sync on 27-bit pieces: 32 x 2^27 fits 32 bits)
+__device__ __forceinline__ long long fx_warp_add(long long m) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)m & 0x7FFFFFFu);
+  const unsigned mi = __reduce_add_sync(0xffffffffu, (unsigned)(m >> 27) & 0x7FFFFFFu);
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(m >> 54));
+  return ((long long)hi << 54) + ((long long)mi << 27) + (long long)lo;
+}
+
+// sum of v over the warp (in every lane): |m| < 2^62
+__device__ __forceinline__ FxVal fx_warp_sum(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  FxVal r;
+  r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(b));
+  r.m = r.e == kFxBad ? 0 : fx_warp_add(fx_mant(b, r.e));
+  return r;
+}
+
+// running sum of FxVals by one lane, on a common scale e fixed beforehand:
+// the two halves are added separately, so nothing overflows below 2^31 terms
+struct FxAcc {
+  long long hi = 0, lo = 0;
+  __device__ __forceinline__ void add(FxVal v, int e) {
+    const int sh = e - v.e;
+    const long long m = sh < 63 ? v.m >> sh : 0;
+    hi += m >> 32;
+    lo += (long long)(unsigned)m;
+  }
+};
+
+// Sum of the lanes' accumulators (in every lane), |hi| and lo below 2^50.
+__device__ __forceinline__ FxAcc fx_warp_add(const FxAcc& a) {
+  FxAcc t;
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, (unsigned)a.lo & 0x7FFFFFFu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, (unsigned)(a.lo >> 27));
+  const unsigned h0 = __reduce_add_sync(0xffffffffu, (unsigned)a.hi & 0x7FFFFFFu);
+  const int h1 = __reduce_add_sync(0xffffffffu, (int)(a.hi >> 27));
+  t.lo = ((long long)l1 << 27) + (long long)l0;
+  t.hi = ((long long)h1 << 27) + (long long)h0;
+  return t;
+}
+#endif
+
+}  // namespace sem

@@ -151,6 +151,7 @@ extern "C" sem_status sem_scatter_add(sem_handle* h, double* dst_L, const int64_
 extern "C" sem_status sem_set_multiplicity(sem_handle* h, const double* mult_L, void* stream) {
   return guarded("sem_set_multiplicity", [&] {
     SEM_REQUIRE(h && mult_L, "sem_set_multiplicity: null argument");
+    h->mult_replaced = 1;
     k_set_imult<<<part_grid(h->nL), 256, 0, (cudaStream_t)stream>>>(h->nL, mult_L, h->imult.ptr,
                                                                     h->dev_err.ptr);
     SEM_CHECK_LAUNCH();

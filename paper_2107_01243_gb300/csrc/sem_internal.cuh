@@ -153,7 +153,7 @@ template <class T>
 struct OpData {
   DevBuf<T> G;      // [E][6][p^3]
   DevBuf<T> B;      // [E][p^3]
-  DevBuf<T> D;      // [p][p] row-major D[i][l] = l_l'(xi_i)
+  DevBuf<T> D;      // [p][p] row-major D[i][l] = l_l'(xi_i), then the even-odd tables
   DevBuf<T> dinv;   // Jacobi inverse diagonal (mask folded in)
   DevBuf<T> dmi;    // dinv / mult (FP64 only: <r, z> = sum r^2 dinv / mult)
   DevBuf<T> h1f;    // per-point h1 in this precision (mixed solves)
@@ -212,6 +212,12 @@ struct sem_handle {
   sem::DevBuf<double> partials;
   // [4]: outer/FP64, inner/FP32, sem_dot ticket, sem_cg_update ticket
   sem::DevBuf<sem::CGState> state;
+  // grid-resident CG (resident.cu): its grid barrier and reduction partials
+  sem::DevBuf<unsigned> res_bar;
+  sem::DevBuf<double> res_part;
+  sem::DevBuf<double> res_s, res_w2;        // its vectors beside r, p, w
+  sem::DevBuf<float> res_s32, res_w232;
+  int mult_replaced = 0;                    // sem_set_multiplicity was called
   // host staging for sem_apply_host
   sem::DevBuf<double> stage_in, stage_out;
   std::shared_ptr<sem::GmresWork> gmres;    // GMRES workspace, kept between solves
@@ -274,6 +280,23 @@ void launch_dssum(const sem_handle* h, T* w, bool apply_mask, const CGState* sta
 template <class T>
 void launch_dssum_box(const sem_handle* h, T* w, bool apply_mask, const CGState* state,
                       cudaStream_t s);
+
+// ---- resident.cu: up to iters PCG iterations of a small problem in one launch
+// (x, r and the state as k_init leaves them; p, s, w, w2 scratch)
+template <class T>
+struct PcgVecs {
+  T *x, *r, *p, *s, *w, *w2;
+  const T* dinv;
+  const T* h1f;
+  T h1, h2;
+  CGState* st;
+};
+template <class T>
+void launch_resident(sem_handle* h, const PcgVecs<T>& v, int iters, cudaStream_t s);
+template <>
+void launch_resident<double>(sem_handle* h, const PcgVecs<double>& v, int iters, cudaStream_t s);
+template <>
+void launch_resident<float>(sem_handle* h, const PcgVecs<float>& v, int iters, cudaStream_t s);
 
 // ---- cg.cu: pieces of the mixed-precision solve reused by the batched solver
 double inner_target(double inner_tol, double tol, double rel);

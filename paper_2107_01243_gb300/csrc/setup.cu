@@ -11,6 +11,7 @@
 
 #include "sem_internal.cuh"
 #include "df.cuh"
+#include "eo_tile.cuh"
 
 namespace sem {
 
@@ -442,9 +443,12 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     DevBuf<double> dxi, dwq;
     dxi.alloc(P); dxi.upload(h->xi.data(), P, s);
     dwq.alloc(P); dwq.upload(h->wq.data(), P, s);
-    h->f64.D.alloc(P * P); h->f64.D.upload(h->Dh.data(), P * P, s);
-    std::vector<float> D32(h->Dh.begin(), h->Dh.end());
-    h->f32.D.alloc(P * P); h->f32.D.upload(D32.data(), P * P, s);
+    // D, then the even-odd tables of D and D^T (eo_tile.cuh), in one buffer
+    std::vector<double> D64(h->Dh), eo = eo_tables(P, h->Dh);
+    D64.insert(D64.end(), eo.begin(), eo.end());
+    const std::vector<float> D32(D64.begin(), D64.end());
+    h->f64.D.alloc(D64.size()); h->f64.D.upload(D64.data(), D64.size(), s);
+    h->f32.D.alloc(D32.size()); h->f32.D.upload(D32.data(), D32.size(), s);
 
     h->coords.alloc(3 * nL);
     double* X = h->coords.ptr;
