@@ -216,15 +216,16 @@ sem_status sem_ax(sem_handle* h, const void* u_L, void* w_L, double h1, double h
  * result.  An element whose u holds an Inf or a NaN gives NaN at all of its
  * points (the native kernel lets them spread through the element's contractions
  * instead, so some of its points stay finite).
- * SEM_F64_KERNEL_NATIVE forces IEEE FP64 arithmetic (at N = 7 and 9 with the
- * even-odd split of D, about 20% fewer FP64 operations).  Returns SEM_ERR_ARG
+ * SEM_F64_KERNEL_NATIVE forces IEEE FP64 arithmetic (except at N = 1 and 3 with
+ * the even-odd split of D, about a fifth fewer FP64 operations).  Returns SEM_ERR_ARG
  * for an unknown kind.
  */
 sem_status sem_set_f64_kernel(sem_handle* h, int kind);
 
 /* Tile chosen by sem_autotune (times in ms per Ax launch, -1 if not timed). */
 typedef struct {
-  int ax32_kernel;          /* FP32 Ax: 0 bulk-copy (TMA) pipeline, 1 global-load kernel */
+  int ax32_kernel;          /* FP32 Ax: 0 bulk-copy (TMA) pipeline, 1 global-load (line) kernel,
+                               the default */
   int ax32_stages;          /* bulk-copy stages in flight per CTA (1..3) */
   int ax32_elems_per_cta;   /* elements per CTA of the bulk-copy kernel (1 or 2) */
   int f64_stages;           /* double-float FP64 Ax: bulk-copy stages (1 or 2) */
@@ -253,7 +254,7 @@ sem_status sem_set_tuning(sem_handle* h, const sem_tuning* t);
  * sem_apply -- the assembled operator w_L = mask o QQ^T (h1 A_L + h2 B_L) u_L
  * (§2, Eq. 9-10; one CG matvec), the same result as sem_ax followed by
  * sem_dssum with the mask, computed with the gather-scatter split by
- * direction.  The element kernel walks segments of four consecutive
+ * direction.  The element kernel walks segments of consecutive
  * elements per CTA and sums the copies of x-interface points inside a
  * segment itself; short passes then add the x-pairs between segments and
  * the y- and z-pairs.  The copies of a point on several interfaces are summed
@@ -261,9 +262,9 @@ sem_status sem_set_tuning(sem_handle* h, const sem_tuning* t);
  * sem_dssum's increasing-index order in the last bits.
  * phase: SEM_APPLY_FULL, or SEM_APPLY_LOCAL then SEM_APPLY_FINISH (the
  * finish phase must follow a local phase on the same handle, dtype and
- * vectors; splitting lets a caller time or overlap the two).  Orders,
- * dtypes or alignments the fused kernels do not cover (odd N, the native
- * FP64 kernel, a per-point h1 in FP64) run sem_ax and sem_dssum's kernels
+ * vectors; splitting lets a caller time or overlap the two).  Segments hold
+ * four elements (double-float, FP32 bulk copies) or as many as the line kernel
+ * takes per CTA.  FP64 at N = 1 and 3 runs sem_ax and sem_dssum's kernels
  * instead, the local phase being the element operator and the finish phase
  * the whole gather-scatter.  u_L and w_L are distinct L-vectors of the
  * dtype (SEM_F64 or SEM_F32); SEM_ERR_ARG otherwise.

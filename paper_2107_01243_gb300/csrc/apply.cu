@@ -23,6 +23,7 @@
 #include "sem_internal.cuh"
 #include <type_traits>
 
+#include "ax_line.cuh"
 #include "ax_tile.cuh"
 
 namespace sem {
@@ -38,46 +39,43 @@ bool df_ax_supported(const sem_handle* h, const void* u, const void* w, const vo
 namespace {
 
 // x-pairs at the segment starts of the element kernel: the first element
-// e_b = g kFuseSeg of segment g >= 1 pairs its i = 0 face with the i = N face
-// of the element before it, unless it starts an x-row.  One block per segment
-// start.
-template <int P, class T>
-__global__ void __launch_bounds__(P * P)
-k_sx_cut(T* __restrict__ w, int nelx, const CGState* __restrict__ st) {
+// e_b = g SEG of segment g >= 1 pairs its i = 0 face with the i = N face
+// of the element before it, unless it starts an x-row.  Threads run over
+// (j, k, segment start).
+template <int P, int SEG, class T>
+__global__ void __launch_bounds__(256)
+k_sx_cut(T* __restrict__ w, uint32_t total, FastDiv dnx, const CGState* __restrict__ st) {
   if (st && st->done) return;
-  constexpr int P2 = P * P;
+  constexpr uint32_t P2 = P * P;
   constexpr long long P3 = (long long)P2 * P;
-  const long long eb = (long long)(blockIdx.x + 1) * kFuseSeg;
-  if (eb % nelx == 0) return;
-  const int j = threadIdx.x % P, k = threadIdx.x / P;
-  const long long hi = eb * P3 + (long long)k * P2 + j * P;    // (eb, 0, j, k)
-  const long long lo = hi - P3 + (P - 1);                       // (eb - 1, N, j, k)
-  const T sum = w[lo] + w[hi];
-  w[lo] = sum;
-  w[hi] = sum;
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += gridDim.x * blockDim.x) {
+    const uint32_t c = t / P2, jk = t - c * P2, eb = (c + 1) * SEG;
+    if (eb == dnx.div(eb) * dnx.d) continue;
+    const long long hi = (long long)eb * P3 + (long long)jk * P;   // (eb, 0, j, k)
+    const long long lo = hi - P3 + (P - 1);                         // (eb - 1, N, j, k)
+    const T sum = w[lo] + w[hi];
+    w[lo] = sum;
+    w[hi] = sum;
+  }
 }
 
-template <class T>
-struct Vec2;
-template <>
-struct Vec2<float> {
-  using V = float2;
-};
-template <>
-struct Vec2<double> {
-  using V = double2;
+// VW values of T moved together
+template <class T, int VW>
+struct alignas(VW * sizeof(T)) Pack {
+  T v[VW];
 };
 
 // y-pairs: (e, i, N, k) + (e + nelx, i, 0, k) for every element with
-// ey < nely - 1; a thread takes two neighbouring i (P is even), threads run
-// over (i pair, k, element) with the i pair fastest
-template <int P, class T>
+// ey < nely - 1; a thread takes VW neighbouring i (VW divides P, w aligned to
+// VW values), threads run over (i, k, element) with i fastest
+template <int P, int VW, class T>
 __global__ void __launch_bounds__(256)
 k_sy(T* __restrict__ w, int nelx, int nely, uint32_t total, FastDiv dnx, FastDiv dny1,
      const CGState* __restrict__ st) {
   if (st && st->done) return;
-  using V = typename Vec2<T>::V;
-  constexpr int H = P / 2, P2 = P * P, P3 = P2 * P;
+  constexpr int H = P / VW, P2 = P * P, P3 = P2 * P;
+  using V = Pack<T, VW>;
   V* wv = reinterpret_cast<V*>(w);
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += gridDim.x * blockDim.x) {
@@ -88,24 +86,26 @@ k_sy(T* __restrict__ w, int nelx, int nely, uint32_t total, FastDiv dnx, FastDiv
     const uint32_t ez = dny1.div(r2);
     const uint32_t ey = r2 - ez * (uint32_t)(nely - 1);
     const uint32_t e = ex + (uint32_t)nelx * (ey + (uint32_t)nely * ez);
-    const uint32_t lo = (e * P3 + k * P2 + (P - 1) * P) / 2 + ip;
-    const uint32_t hi = ((e + nelx) * P3 + k * P2) / 2 + ip;
-    const V a = wv[lo], b = wv[hi];
-    const V sum = {a.x + b.x, a.y + b.y};
-    wv[lo] = sum;
-    wv[hi] = sum;
+    const uint32_t lo = (e * P3 + k * P2 + (P - 1) * P) / VW + ip;
+    const uint32_t hi = ((e + nelx) * P3 + k * P2) / VW + ip;
+    V a = wv[lo];
+    const V b = wv[hi];
+#pragma unroll
+    for (int c = 0; c < VW; ++c) a.v[c] = a.v[c] + b.v[c];
+    wv[lo] = a;
+    wv[hi] = a;
   }
 }
 
 // z-pairs: (e, i, j, N) + (e + nelx nely, i, j, 0) for every element with
-// ez < nelz - 1 (the first nelx nely (nelz - 1) elements); 16 bytes per thread
-template <int P, class T>
+// ez < nelz - 1 (the first nelx nely (nelz - 1) elements), VW values a thread
+// (VW divides P^2, w aligned to VW values)
+template <int P, int VW, class T>
 __global__ void __launch_bounds__(256)
 k_sz(T* __restrict__ w, uint32_t layer, uint32_t total, const CGState* __restrict__ st) {
   if (st && st->done) return;
-  constexpr int VW = 16 / (int)sizeof(T), P2 = P * P, P3 = P2 * P, Q = P2 / VW;
-  static_assert(P2 % VW == 0, "plane not a whole number of 16-byte vectors");
-  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+  constexpr int P2 = P * P, P3 = P2 * P, Q = P2 / VW;
+  using V = Pack<T, VW>;
   V* wv = reinterpret_cast<V*>(w);
   for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total;
        t += gridDim.x * blockDim.x) {
@@ -114,10 +114,8 @@ k_sz(T* __restrict__ w, uint32_t layer, uint32_t total, const CGState* __restric
     const uint32_t hi = ((e + layer) * P3) / VW + q;
     V a = wv[lo];
     const V b = wv[hi];
-    T* ap = reinterpret_cast<T*>(&a);
-    const T* bp = reinterpret_cast<const T*>(&b);
 #pragma unroll
-    for (int c = 0; c < VW; ++c) ap[c] = ap[c] + bp[c];
+    for (int c = 0; c < VW; ++c) a.v[c] = a.v[c] + b.v[c];
     wv[lo] = a;
     wv[hi] = a;
   }
@@ -127,33 +125,57 @@ int sweep_blocks(long long total) {
   return (int)std::max<long long>(1, std::min<long long>((total + 255) / 256, 16LL * sem_num_sms()));
 }
 
-// the finishing passes on a box of nelx x nely x nelz elements starting at w
-template <int P, class T>
-void finish_box(T* w, int nelx, int nely, int nelz, const CGState* st, cudaStream_t s) {
-  const long long E = (long long)nelx * nely * nelz;
-  const long long nseg = (E + kFuseSeg - 1) / kFuseSeg;
-  if (nseg > 1 && nelx > 1) {
-    k_sx_cut<P, T><<<(unsigned)(nseg - 1), P * P, 0, s>>>(w, nelx, st);
-    SEM_CHECK_LAUNCH();
-  }
-  if (nely > 1) {
-    const long long total = (long long)nelx * (nely - 1) * nelz * P * (P / 2);
-    k_sy<P, T><<<sweep_blocks(total), 256, 0, s>>>(
-        w, nelx, nely, (uint32_t)total, FastDiv((uint32_t)nelx), FastDiv((uint32_t)(nely - 1)),
-        st);
-    SEM_CHECK_LAUNCH();
-  }
-  if (nelz > 1) {
-    const long long layer = (long long)nelx * nely;
-    const long long total = layer * (nelz - 1) * P * P / (16 / (int)sizeof(T));
-    k_sz<P, T><<<sweep_blocks(total), 256, 0, s>>>(w, (uint32_t)layer, (uint32_t)total, st);
-    SEM_CHECK_LAUNCH();
-  }
+// whether w starts on a multiple of VW values (element bases are then too: VW
+// divides P^2)
+template <int VW, class T>
+bool aligned_to(const T* w) {
+  return reinterpret_cast<uintptr_t>(w) % (VW * sizeof(T)) == 0;
 }
 
 template <int P, class T>
-void finish_p(const sem_handle* h, T* w, const CGState* st, cudaStream_t s) {
-  finish_box<P, T>(w, h->nelx, h->nely, h->nelz, st, s);
+void launch_sy(T* w, int nelx, int nely, int nelz, const CGState* st, cudaStream_t s) {
+  auto go = [&](auto vw) {
+    constexpr int VW = decltype(vw)::value;
+    const long long total = (long long)nelx * (nely - 1) * nelz * P * (P / VW);
+    k_sy<P, VW, T><<<sweep_blocks(total), 256, 0, s>>>(w, nelx, nely, (uint32_t)total,
+                                                       FastDiv((uint32_t)nelx),
+                                                       FastDiv((uint32_t)(nely - 1)), st);
+    SEM_CHECK_LAUNCH();
+  };
+  if constexpr (P % 2 == 0)
+    if (aligned_to<2>(w)) return go(std::integral_constant<int, 2>());
+  go(std::integral_constant<int, 1>());
+}
+
+// the z-pairs of nz element layers and the ones above them
+template <int P, class T>
+void launch_sz(T* w, long long layer, int nz, const CGState* st, cudaStream_t s) {
+  auto go = [&](auto vw) {
+    constexpr int VW = decltype(vw)::value;
+    const long long total = layer * nz * P * P / VW;
+    k_sz<P, VW, T><<<sweep_blocks(total), 256, 0, s>>>(w, (uint32_t)layer, (uint32_t)total, st);
+    SEM_CHECK_LAUNCH();
+  };
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (P * P % W == 0)
+    if (aligned_to<W>(w)) return go(std::integral_constant<int, W>());
+  go(std::integral_constant<int, 1>());
+}
+
+// the finishing passes on a box of nelx x nely x nelz elements starting at w,
+// after an element kernel with segments of SEG elements
+template <int P, int SEG, class T>
+void finish_box(T* w, int nelx, int nely, int nelz, const CGState* st, cudaStream_t s) {
+  const long long E = (long long)nelx * nely * nelz;
+  const long long nseg = (E + SEG - 1) / SEG;
+  if (nseg > 1 && nelx > 1) {
+    const long long total = (nseg - 1) * P * P;
+    k_sx_cut<P, SEG, T><<<sweep_blocks(total), 256, 0, s>>>(w, (uint32_t)total,
+                                                            FastDiv((uint32_t)nelx), st);
+    SEM_CHECK_LAUNCH();
+  }
+  if (nely > 1) launch_sy<P, T>(w, nelx, nely, nelz, st, s);
+  if (nelz > 1) launch_sz<P, T>(w, (long long)nelx * nely, nelz - 1, st, s);
 }
 
 // z-pairs between element planes z - 1 and z of the box (one plane of pairs)
@@ -161,10 +183,7 @@ template <int P, class T>
 void zpairs_between(const sem_handle* h, T* w, int z, cudaStream_t s) {
   constexpr long long P3 = (long long)P * P * P;
   const long long layer = (long long)h->nelx * h->nely;
-  const long long total = layer * P * P / (16 / (int)sizeof(T));
-  k_sz<P, T><<<sweep_blocks(total), 256, 0, s>>>(w + (z - 1) * layer * P3, (uint32_t)layer,
-                                                  (uint32_t)total, nullptr);
-  SEM_CHECK_LAUNCH();
+  launch_sz<P, T>(w + (z - 1) * layer * P3, layer, 1, nullptr, s);
 }
 
 // the finishing passes of the slab of element planes [z0, z1), then (z0 > 0)
@@ -172,19 +191,33 @@ void zpairs_between(const sem_handle* h, T* w, int z, cudaStream_t s) {
 template <int P>
 void finish_slab(const sem_handle* h, double* w, int z0, int z1, cudaStream_t s) {
   constexpr long long P3 = (long long)P * P * P;
-  finish_box<P, double>(w + (long long)z0 * h->nelx * h->nely * P3, h->nelx, h->nely, z1 - z0,
+  finish_box<P, kFuseSeg, double>(w + (long long)z0 * h->nelx * h->nely * P3, h->nelx, h->nely, z1 - z0,
                         nullptr, s);
   if (z0 > 0) zpairs_between<P, double>(h, w, z0, s);
 }
 
+// line: the element kernel was the line kernel (its own segment length)
+template <int P, class T>
+void finish_p(const sem_handle* h, T* w, bool line, const CGState* st, cudaStream_t s) {
+  if (line)
+    finish_box<P, line_elems(P, sizeof(T) == 8), T>(w, h->nelx, h->nely, h->nelz, st, s);
+  else if constexpr (P % 2 == 0)
+    finish_box<P, kFuseSeg, T>(w, h->nelx, h->nely, h->nelz, st, s);
+}
+
 template <class T>
-void finish(const sem_handle* h, T* w, const CGState* st, cudaStream_t s) {
+void finish(const sem_handle* h, T* w, bool line, const CGState* st, cudaStream_t s) {
   switch (h->P) {
-    case 2: finish_p<2, T>(h, w, st, s); break;
-    case 4: finish_p<4, T>(h, w, st, s); break;
-    case 6: finish_p<6, T>(h, w, st, s); break;
-    case 8: finish_p<8, T>(h, w, st, s); break;
-    case 10: finish_p<10, T>(h, w, st, s); break;
+    case 2: finish_p<2, T>(h, w, line, st, s); break;
+    case 3: finish_p<3, T>(h, w, line, st, s); break;
+    case 4: finish_p<4, T>(h, w, line, st, s); break;
+    case 5: finish_p<5, T>(h, w, line, st, s); break;
+    case 6: finish_p<6, T>(h, w, line, st, s); break;
+    case 7: finish_p<7, T>(h, w, line, st, s); break;
+    case 8: finish_p<8, T>(h, w, line, st, s); break;
+    case 9: finish_p<9, T>(h, w, line, st, s); break;
+    case 10: finish_p<10, T>(h, w, line, st, s); break;
+    case 11: finish_p<11, T>(h, w, line, st, s); break;
     default: throw Error(SEM_ERR_ARG, "apply: unsupported order");
   }
 }
@@ -207,10 +240,21 @@ bool apply_fused_supported<double>(const sem_handle* h, const void* u, const voi
 template <class T>
 bool launch_apply(sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2, const T* h1f,
                   const CGState* st, int phase, cudaStream_t s, CGState* pwst) {
-  if (!apply_fused_supported<T>(h, u, w, h1f)) {
-    // element kernel and the gather-scatter kernel, in the full phase
-    if (phase & SEM_APPLY_LOCAL) launch_ax<T>(h, op, u, w, h1, h2, h1f, st, s);
-    if (phase & SEM_APPLY_FINISH) launch_dssum<T>(h, w, true, st, s);
+  // the streaming kernels (double-float; FP32 bulk copies where they are tuned,
+  // or asked for <p, H p>), else the line kernel, else element kernel and
+  // gather-scatter (the FP64 orders and errors of launch_ax)
+  bool stream = apply_fused_supported<T>(h, u, w, h1f);
+  if (sizeof(T) == 4) stream = stream && (!h->tune.ax32_ldg || (pwst && h->P == 8));
+  if (!stream) {
+    const bool line = line_ax_supported<T>(h) && h->nL < (1LL << 31);
+    if (phase & SEM_APPLY_LOCAL) {
+      if (line) launch_ax_line<T>(h, op, u, w, h1, h2, h1f, true, st, s);
+      else launch_ax<T>(h, op, u, w, h1, h2, h1f, st, s);
+    }
+    if (phase & SEM_APPLY_FINISH) {
+      if (line) finish<T>(h, w, true, st, s);
+      else launch_dssum<T>(h, w, true, st, s);
+    }
     return false;
   }
   bool pw = false;
@@ -220,7 +264,7 @@ bool launch_apply(sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T 
     else
       pw = launch_ax_df_fused(h, u, w, h1, h2, st, pwst, s);
   }
-  if (phase & SEM_APPLY_FINISH) finish<T>(h, w, st, s);
+  if (phase & SEM_APPLY_FINISH) finish<T>(h, w, false, st, s);
   return pw;
 }
 

@@ -1,0 +1,183 @@
+// The line kernels' element body (L-vectors: ax_line.cu; global vectors:
+// global.cu and batch_glob.cuh): K consecutive elements a CTA, thread (i, j) of
+// an element owning its k-column.
+#pragma once
+#include "sem_internal.cuh"
+#include "ax_tile.cuh"
+#include "eo_tile.cuh"
+
+namespace sem {
+
+// Elements per CTA: the most that fit 256 threads among the counts whose K P^2
+// threads fill their warps best.  FP64 at P = 10 takes three (300 of 320 lanes
+// instead of 200 of 224: the FP64 pipe is its bound, and pays for idle lanes:
+// 818 against 856 us on 8 M points); FP32 there holds 60 G values a thread, and
+// two elements fit the registers twice an SM (59 against 64 us).
+constexpr int line_elems(int P, bool f64) {
+  const int P2 = P * P, most = f64 && P == 10 ? 320 : 256;
+  int best = 1;
+  for (int k = 1; k * P2 <= most; ++k) {
+    const int lanes = (k * P2 + 31) / 32 * 32, bl = (best * P2 + 31) / 32 * 32;
+    if ((long long)k * bl >= (long long)best * lanes) best = k;
+  }
+  return best;
+}
+
+template <int P, class T>
+struct LineCfg {
+  static constexpr int P2 = P * P, P3 = P2 * P, K = line_elems(P, sizeof(T) == 8);
+  static constexpr int THREADS = (K * P2 + 31) / 32 * 32;
+  static constexpr int RS = P | 1, PL = P * RS, VOL = P * PL;   // rows of odd length
+  static constexpr int TS = sizeof(T) == 8 ? 2 * EoTab<P>::SIZE : 0;
+  static constexpr size_t SMEM = (3 * (size_t)K * VOL + TS) * sizeof(T);
+  // CTAs per SM the registers are bounded for (FP64, P = 10: two of 320 threads;
+  // FP32, P = 8: three instead of two, sem_apply on 16.8 M points 120 against 134 us)
+  static constexpr int MINB = sizeof(T) == 4 ? (P >= 10 ? 2 : P == 8 ? 3 : 1) : (P <= 8 ? 4 : P == 10 ? 2 : 3);
+};
+
+// y = D x or D^T x for a line in registers
+template <int P, class T, bool TRANS, class PUT>
+__device__ __forceinline__ void line_dots(const T (&x)[P], const DMat<P, T>& D, const T* tab,
+                                          PUT put) {
+  if constexpr (sizeof(T) == 8) {
+    eo_dots<P, T>(x, tab + (TRANS ? EoTab<P>::SIZE : 0), put);
+  } else {
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+      T y = (TRANS ? D.d[i] : D.d[i * P]) * x[0];
+#pragma unroll
+      for (int l = 1; l < P; ++l) y = fma(TRANS ? D.d[l * P + i] : D.d[i * P + l], x[l], y);
+      put(i, y);
+    }
+  }
+}
+
+// This thread's place in its element and the element's shared-memory arrays
+template <int P, class T>
+struct LineThread {
+  using C = LineCfg<P, T>;
+  int el, lam, i, j, col, ln_r, ln_s;
+  T *tab, *U, *R, *S;
+  __device__ __forceinline__ void init(unsigned char* smem) {
+    const int tid = threadIdx.x;
+    el = tid / C::P2;
+    lam = tid - el * C::P2;
+    i = lam % P;
+    j = lam / P;
+    col = j * C::RS + i;                 // (i, j, 0)
+    ln_r = lam * C::RS;                  // r-line (j, k) = (lam % P, lam / P)
+    ln_s = j * C::PL + i;                // s-line (i, k) = (lam % P, lam / P)
+    tab = reinterpret_cast<T*>(smem);
+    U = tab + C::TS + (el < C::K ? el : 0) * C::VOL;
+    R = U + C::K * C::VOL;
+    S = R + C::K * C::VOL;
+  }
+};
+
+// out = (h1 D^T G D + h2 B) u at the k-column: uc the column of u, g, b, h1f the
+// element's G, B and h1 at this thread's (i, j, 0) (h1f may be NULL).  All
+// threads of the CTA call it (act: the thread has an element); U is free once
+// the second barrier is behind.
+template <int P, class T>
+__device__ __forceinline__ void line_element(const LineThread<P, T>& t, bool act,
+                                             const DMat<P, T>& D, const T (&uc)[P], const T* g,
+                                             const T* b, const T* h1f, T h1, T h2, T (&out)[P]) {
+  using C = LineCfg<P, T>;
+  constexpr int P2 = C::P2, P3 = C::P3, RS = C::RS, PL = C::PL;
+  constexpr bool PRE = sizeof(T) == 4;       // G prefetched to registers
+  T gr[PRE ? P : 1][6];
+  if (act) {
+    if constexpr (PRE) {
+#pragma unroll
+      for (int k = 0; k < P; ++k)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) gr[k][c] = __ldcs(g + c * P3 + k * P2);
+    }
+#pragma unroll
+    for (int k = 0; k < P; ++k) t.U[k * PL + t.col] = uc[k];
+  }
+  __syncthreads();
+  if (act) {
+    T x[P];
+#pragma unroll
+    for (int l = 0; l < P; ++l) x[l] = t.U[t.ln_r + l];
+    line_dots<P, T, false>(x, D, t.tab, [&](int a, T y) { t.R[t.ln_r + a] = y; });
+#pragma unroll
+    for (int l = 0; l < P; ++l) x[l] = t.U[t.ln_s + l * RS];
+    line_dots<P, T, false>(x, D, t.tab, [&](int a, T y) { t.S[t.ln_s + a * RS] = y; });
+  }
+  __syncthreads();
+  T wt[P];
+  if (act) {
+    T ut[P];
+    line_dots<P, T, false>(uc, D, t.tab, [&](int a, T y) { ut[a] = y; });
+    const bool scale = h1f || h1 != T(1);
+#pragma unroll
+    for (int k = 0; k < P; ++k) {
+      const T ur = t.R[k * PL + t.col], us = t.S[k * PL + t.col];
+      T g11, g22, g33, g12, g13, g23;
+      if constexpr (PRE) {
+        g11 = gr[k][0]; g22 = gr[k][1]; g33 = gr[k][2];
+        g12 = gr[k][3]; g13 = gr[k][4]; g23 = gr[k][5];
+      } else {
+        g11 = __ldcs(g + k * P2); g22 = __ldcs(g + P3 + k * P2); g33 = __ldcs(g + 2 * P3 + k * P2);
+        g12 = __ldcs(g + 3 * P3 + k * P2); g13 = __ldcs(g + 4 * P3 + k * P2);
+        g23 = __ldcs(g + 5 * P3 + k * P2);
+      }
+      T wr = fma(g13, ut[k], fma(g12, us, g11 * ur));
+      T ws = fma(g23, ut[k], fma(g22, us, g12 * ur));
+      T wk = fma(g33, ut[k], fma(g23, us, g13 * ur));
+      if (scale) {
+        const T c = h1f ? __ldcs(h1f + k * P2) : h1;
+        wr *= c;
+        ws *= c;
+        wk *= c;
+      }
+      t.R[k * PL + t.col] = wr;
+      t.S[k * PL + t.col] = ws;
+      wt[k] = wk;
+    }
+  }
+  __syncthreads();
+  if (act) {
+    T x[P];
+#pragma unroll
+    for (int l = 0; l < P; ++l) x[l] = t.R[t.ln_r + l];
+    line_dots<P, T, true>(x, D, t.tab, [&](int a, T y) { t.R[t.ln_r + a] = y; });
+#pragma unroll
+    for (int l = 0; l < P; ++l) x[l] = t.S[t.ln_s + l * RS];
+    line_dots<P, T, true>(x, D, t.tab, [&](int a, T y) { t.S[t.ln_s + a * RS] = y; });
+    line_dots<P, T, true>(wt, D, t.tab, [&](int a, T y) { out[a] = y; });
+  }
+  __syncthreads();
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < P; ++k) out[k] += t.R[k * PL + t.col] + t.S[k * PL + t.col];
+    if (h2 != T(0)) {
+#pragma unroll
+      for (int k = 0; k < P; ++k) out[k] = fma(h2 * __ldcs(b + k * P2), uc[k], out[k]);
+    }
+  }
+}
+
+// Whether the line kernel is this precision's element kernel.  FP32: always
+// (8 M points, us, against the kernel it took the place of: N = 2 58 / 79, N = 4
+// 50 / 76, N = 6 49 / 99, N = 8 52 / 91; against the bulk-copy kernel, which
+// stays for large meshes at N = 7 and 9 and for tuned handles: N = 1 58 / 209,
+// N = 3 46 / 52, N = 5 45 / 56, N = 7 42 / 42, N = 9 59 / 61).  FP64: not at P = 2 and 4, where the split saves next to
+// nothing and the column kernel keeps the FP64 pipe busier (N = 1 447 / 367, N = 3
+// 585 / 528; N = 2 431 / 452, N = 4 603 / 637, N = 6 670 / 810, N = 8 805 / 1037,
+// N = 10 814 / 1072, and against the one-element even-odd kernel N = 7 681 / 783,
+// N = 9 818 / 923); nor where a handle insists on the double-float kernel.
+template <class T>
+inline bool line_ax_supported(const sem_handle* h) {
+  return sizeof(T) == 4 || (h->P != 2 && h->P != 4 && h->f64_kernel != SEM_F64_KERNEL_DOUBLEFLOAT);
+}
+
+// w = (h1 A + h2 B) u on L-vectors; fuse: masked points zero, x-pairs inside
+// segments of line_elems(P, T) elements summed.  st may be null.
+template <class T>
+void launch_ax_line(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2,
+                    const T* h1f, bool fuse, const CGState* st, cudaStream_t s);
+
+}  // namespace sem

@@ -22,22 +22,20 @@ struct EoTab {
   static constexpr int SIZE = M + ODD * H;
 };
 
-// y = M x along one line: x at in[off[.]], y at out[off[.]] (in may equal
-// out); tab in shared memory (one broadcast read per use: the compiler would
-// otherwise keep the whole table in registers across the element loop)
-template <int P, class T>
-__device__ __forceinline__ void eo_line(const T* in, T* out, const int (&off)[P], const T* tab) {
+// y = M x for a line in registers; put(i, y_i) receives the outputs.  tab in
+// shared memory (one broadcast read per use: the compiler would otherwise
+// keep the whole table in registers across the element loop)
+template <int P, class T, class PUT>
+__device__ __forceinline__ void eo_dots(const T (&x)[P], const T* tab, PUT put) {
   using E = EoTab<P>;
   constexpr int H = E::H, HS = E::HS, N = P - 1;
   T e[HS], o[H];
 #pragma unroll
   for (int l = 0; l < H; ++l) {
-    const T a = in[off[l]], b = in[off[N - l]];
-    e[l] = a + b;
-    o[l] = a - b;
+    e[l] = x[l] + x[N - l];
+    o[l] = x[l] - x[N - l];
   }
-  if constexpr (E::ODD) e[H] = in[off[H]];
-  // every input of the line is in registers: outputs may go out in place
+  if constexpr (E::ODD) e[H] = x[H];
 #pragma unroll
   for (int i = 0; i < H; ++i) {
     T a = tab[E::A + i * H] * o[0];
@@ -47,15 +45,24 @@ __device__ __forceinline__ void eo_line(const T* in, T* out, const int (&off)[P]
       if (l < H) a = fma(tab[E::A + i * H + l], o[l], a);
       s = fma(tab[E::S + i * HS + l], e[l], s);
     }
-    out[off[i]] = a + s;
-    out[off[N - i]] = a - s;
+    put(i, a + s);
+    put(N - i, a - s);
   }
   if constexpr (E::ODD) {
     T a = tab[E::M] * o[0];
 #pragma unroll
     for (int l = 1; l < H; ++l) a = fma(tab[E::M + l], o[l], a);
-    out[off[H]] = a;
+    put(H, a);
   }
+}
+
+// the same with x at in[off[.]] and y at out[off[.]] (in may equal out)
+template <int P, class T>
+__device__ __forceinline__ void eo_line(const T* in, T* out, const int (&off)[P], const T* tab) {
+  T x[P];
+#pragma unroll
+  for (int l = 0; l < P; ++l) x[l] = in[off[l]];
+  eo_dots<P, T>(x, tab, [&](int i, T y) { out[off[i]] = y; });
 }
 
 // host: the tables of D and D^T, one after the other (2 EoTab<P>::SIZE values)

@@ -181,7 +181,7 @@ struct sem_handle {
   sem::DevBuf<int> escale;                  // per element: exponents sG | sB << 16 of gdf, bdf
   int f64_kernel = SEM_F64_KERNEL_AUTO;     // which FP64 Ax kernel runs
   struct Tune {
-    int ax32_ldg = 0;          // 1: FP32 Ax by the global-load kernel instead of bulk copies
+    int ax32_ldg = 1;          // 1: FP32 Ax by the line kernel (global loads), 0: bulk copies
     int ax32_variant = 1;      // bulk-copy variant: (stages, elements per CTA), see ax_tma.cu
     int df_variant = 0;        // double-float Ax: 0 = one stage, 1 = two stages
     int tuned = 0;
@@ -262,7 +262,6 @@ void launch_ax_tma(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T
 // FP64-accurate double-float variant (even P in {6, 8, 10}, constant h1)
 bool df_ax_supported(const sem_handle* h, const void* u, const void* w, const void* h1f);
 void df_prepare(const sem_handle* h);          // once-per-process setup, run by sem_setup
-void eo_prepare(const sem_handle* h);          // the same for the IEEE FP64 even-order kernel
 void noalloc_prepare();                        // resolves sem_dot_noalloc's static array
 void launch_ax_df(const sem_handle* h, const double* u, double* w, double h1, double h2,
                   const CGState* state, cudaStream_t s);

@@ -426,6 +426,10 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     h->prec_flags = precision_flags | SEM_PREC_F64;   // FP64 geometry is always kept
     h->faces = mesh->dirichlet_faces & SEM_FACE_ALL;
     for (int d = 0; d < 3; ++d) h->len[d] = mesh->len[d];
+    // until tuned: the line kernel, but bulk copies on large meshes at P = 8 and
+    // 10 (sem_apply, us, line / bulk: N = 9 4 M points 51 / 56, 17.6 M 167 / 166
+    // and with a mass term 187 / 169; N = 7 4 M 42 / 46, 16.8 M 120 / 119)
+    h->tune.ax32_ldg = h->P >= 8 && h->P % 2 == 0 && h->nL > (1 << 23) ? 0 : 1;
     h->tune.ax32_variant = h->P <= 4 ? 2 : 1;     // 3 stages for small elements, else 2
     gll_host(N, h->xi, h->wq, h->Dh);
 
@@ -496,7 +500,6 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
       SEM_CHECK_LAUNCH();
       df_prepare(h.get());
     }
-    if (h->f64.G.ptr) eo_prepare(h.get());
     noalloc_prepare();
     h->dev_err.alloc(1);
     SEM_CUDA(cudaMemsetAsync(h->dev_err.ptr, 0, sizeof(int), s));
