@@ -162,20 +162,141 @@ void launch_sz(T* w, long long layer, int nz, const CGState* st, cudaStream_t s)
   go(std::integral_constant<int, 1>());
 }
 
+// All the pairs the element kernel left, in one pass: every point on a z-face
+// between elements (Z), on a y-face but no such z-face (Y), on an x-face between
+// segments but neither (X).  A thread owns all the copies of its
+// point (the lowest copy's place tells it) and sums them pair by pair along x,
+// y, z; the x-pairs inside a segment already agree, so one of the two is read
+// and both are written.  Threads run over (i, j) or
+// (i, k) of an element, i fastest.
+template <int P, int SEG, class T>
+__global__ void __launch_bounds__(256)
+k_finish(T* __restrict__ w, int nelx, int nely, int nelz, uint32_t nZ, uint32_t nY, uint32_t nX,
+         FastDiv dnx, FastDiv dny, FastDiv dny1, const CGState* __restrict__ st) {
+  if (st && st->done) return;
+  constexpr int N = P - 1, P2 = P * P, P3 = P2 * P;
+  const uint32_t total = nZ + nY + nX;
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < total;
+       t += gridDim.x * blockDim.x) {
+    uint32_t e;
+    int i, j, k, ex, ey, ez;
+    if (t < nZ) {
+      e = t / P2;
+      const int q = (int)(t - e * P2);
+      i = q % P;
+      j = q / P;
+      k = N;
+      const uint32_t r = dnx.div(e);
+      ex = (int)(e - r * (uint32_t)nelx);
+      ez = (int)dny.div(r);
+      ey = (int)r - ez * nely;
+      if (j == 0 && ey > 0) continue;                       // its row j = N below owns it
+    } else if (t < nZ + nY) {
+      const uint32_t m = (t - nZ) / P2;                     // elements with ey < nely - 1
+      const int q = (int)((t - nZ) - m * P2);
+      i = q % P;
+      j = N;
+      k = q / P;
+      const uint32_t r = dnx.div(m);
+      ex = (int)(m - r * (uint32_t)nelx);
+      ez = (int)dny1.div(r);
+      ey = (int)r - ez * (nely - 1);
+      e = (uint32_t)(ex + nelx * (ey + nely * ez));
+      if ((k == 0 && ez > 0) || (k == N && ez < nelz - 1)) continue;   // on a z-face
+    } else {
+      const uint32_t c = (t - nZ - nY) / P2;
+      const int q = (int)((t - nZ - nY) - c * P2);
+      e = (c + 1) * SEG - 1;                                // last of its segment
+      i = N;
+      j = q % P;
+      k = q / P;
+      const uint32_t r = dnx.div(e);
+      ex = (int)(e - r * (uint32_t)nelx);
+      ez = (int)dny.div(r);
+      ey = (int)r - ez * nely;
+      if (ex == nelx - 1 || (j == 0 && ey > 0) || (j == N && ey < nely - 1) ||
+          (k == 0 && ez > 0) || (k == N && ez < nelz - 1))
+        continue;
+    }
+    if (i == 0 && ex > 0) continue;                         // e - 1's column i = N owns it
+    const bool fx = i == N && ex < nelx - 1, fy = j == N && ey < nely - 1,
+               fz = k == N && ez < nelz - 1;
+    const int ox = P3 - N, oy = nelx * P3 - N * P, oz = nelx * nely * P3 - N * P2;
+    T* const b = w + ((size_t)e * P3 + (k * P + j) * P + i);
+    // FP64: adds that no lane of the warp needs are skipped (a warp's FP64 add
+    // takes 64 cycles of a scheduler, predicated or not)
+    bool anyy = fy, anyz = fz;
+    if constexpr (sizeof(T) == 8) {
+      const unsigned am = __activemask();
+      anyy = __any_sync(am, fy);
+      anyz = __any_sync(am, fz);
+    }
+    // the (y, z) copies; at a segment end the x-partner's value is still apart
+    T c[4], x[4];
+    bool cut[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const bool in = (!(m & 1) || fy) && (!(m & 2) || fz);
+      const int o = ((m & 1) ? oy : 0) + ((m & 2) ? oz : 0);
+      const uint32_t em = e + ((m & 1) ? (uint32_t)nelx : 0u) + ((m & 2) ? (uint32_t)(nelx * nely) : 0u);
+      cut[m] = in && fx && (em + 1) % SEG == 0;
+      c[m] = in ? b[o] : T(0);
+      x[m] = cut[m] ? b[o + ox] : T(0);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      bool any = cut[m];
+      if constexpr (sizeof(T) == 8) any = __any_sync(__activemask(), cut[m]);
+      if (any) c[m] += x[m];               // x = 0 where there is no cut
+    }
+    T s = c[0];
+    if (anyy) s += c[1];                   // 0 where there is no copy
+    if (anyz) {
+      T s2 = c[2];
+      if (anyy) s2 += c[3];
+      s += s2;
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+      if ((!(m & 1) || fy) && (!(m & 2) || fz)) {
+        const int o = ((m & 1) ? oy : 0) + ((m & 2) ? oz : 0);
+        b[o] = s;
+        if (fx) b[o + ox] = s;
+      }
+  }
+}
+
+// Below this many bytes of w one pass over the shared points takes the place of
+// the three: it saves two launches, but its copies across an x-face are
+// scattered writes that cost more than the launches once w no longer sits in
+// the caches (finish alone, us, one pass / three: FP32 N = 7, 0.9 M points 11 / 14,
+// 4.1 M 11 / 15, 16.8 M 30 / 24; FP64 N = 7, 0.9 M 9.5 / 14, 4.1 M 19 / 15, 16.8 M
+// 67 / 38).
+constexpr long long kOnePassBytes = 1 << 24;
+
 // the finishing passes on a box of nelx x nely x nelz elements starting at w,
 // after an element kernel with segments of SEG elements
 template <int P, int SEG, class T>
 void finish_box(T* w, int nelx, int nely, int nelz, const CGState* st, cudaStream_t s) {
-  const long long E = (long long)nelx * nely * nelz;
-  const long long nseg = (E + SEG - 1) / SEG;
-  if (nseg > 1 && nelx > 1) {
-    const long long total = (nseg - 1) * P * P;
-    k_sx_cut<P, SEG, T><<<sweep_blocks(total), 256, 0, s>>>(w, (uint32_t)total,
-                                                            FastDiv((uint32_t)nelx), st);
+  const long long layer = (long long)nelx * nely, E = layer * nelz, P2 = P * P;
+  const long long nX = nelx > 1 ? ((E + SEG - 1) / SEG - 1) * P2 : 0;
+  if (E * P2 * P * (long long)sizeof(T) <= kOnePassBytes) {
+    const long long nZ = layer * (nelz - 1) * P2, nY = (long long)nelx * (nely - 1) * nelz * P2;
+    if (nZ + nY + nX == 0) return;
+    const int blocks = (int)std::min<long long>((nZ + nY + nX + 255) / 256, 64LL * sem_num_sms());
+    k_finish<P, SEG, T><<<blocks, 256, 0, s>>>(
+        w, nelx, nely, nelz, (uint32_t)nZ, (uint32_t)nY, (uint32_t)nX, FastDiv((uint32_t)nelx),
+        FastDiv((uint32_t)nely), FastDiv((uint32_t)std::max(1, nely - 1)), st);
+    SEM_CHECK_LAUNCH();
+    return;
+  }
+  if (nX > 0) {
+    k_sx_cut<P, SEG, T><<<sweep_blocks(nX), 256, 0, s>>>(w, (uint32_t)nX, FastDiv((uint32_t)nelx),
+                                                         st);
     SEM_CHECK_LAUNCH();
   }
   if (nely > 1) launch_sy<P, T>(w, nelx, nely, nelz, st, s);
-  if (nelz > 1) launch_sz<P, T>(w, (long long)nelx * nely, nelz - 1, st, s);
+  if (nelz > 1) launch_sz<P, T>(w, layer, nelz - 1, st, s);
 }
 
 // z-pairs between element planes z - 1 and z of the box (one plane of pairs)

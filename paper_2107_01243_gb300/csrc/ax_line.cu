@@ -49,7 +49,7 @@ ax_line_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__
 #pragma unroll
     for (int k = 0; k < P; ++k) uc[k] = u[base + k * P2];
   }
-  line_element<P, T>(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
+  line_element(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
                      h1f ? h1f + base : nullptr, h1, h2, out);
   if constexpr (FUSE) {
     // masked points, then the x-pairs of neighbours in this CTA: the faces

@@ -8,13 +8,13 @@
 
 namespace sem {
 
-// Elements per CTA: the most that fit 256 threads among the counts whose K P^2
+// Elements per CTA: the most that fit the threads among the counts whose K P^2
 // threads fill their warps best.  FP64 at P = 10 takes three (300 of 320 lanes
 // instead of 200 of 224: the FP64 pipe is its bound, and pays for idle lanes:
 // 818 against 856 us on 8 M points); FP32 there holds 60 G values a thread, and
 // two elements fit the registers twice an SM (59 against 64 us).
-constexpr int line_elems(int P, bool f64) {
-  const int P2 = P * P, most = f64 && P == 10 ? 320 : 256;
+constexpr int line_elems(int P, bool f64, int threads = 256) {
+  const int P2 = P * P, most = f64 && P == 10 ? 320 : threads;
   int best = 1;
   for (int k = 1; k * P2 <= most; ++k) {
     const int lanes = (k * P2 + 31) / 32 * 32, bl = (best * P2 + 31) / 32 * 32;
@@ -23,16 +23,22 @@ constexpr int line_elems(int P, bool f64) {
   return best;
 }
 
-template <int P, class T>
+// threads of the global-vector kernels' CTAs: two elements at N = 7, one at N = 9
+// (256 threads, twice the elements: 108 against 100 us and 154 against 147 us on
+// 17 M points)
+constexpr int kGlobThreads = 128;
+
+template <int P, class T, int MOST = 256>
 struct LineCfg {
-  static constexpr int P2 = P * P, P3 = P2 * P, K = line_elems(P, sizeof(T) == 8);
+  static constexpr int P2 = P * P, P3 = P2 * P, K = line_elems(P, sizeof(T) == 8, MOST);
   static constexpr int THREADS = (K * P2 + 31) / 32 * 32;
   static constexpr int RS = P | 1, PL = P * RS, VOL = P * PL;   // rows of odd length
   static constexpr int TS = sizeof(T) == 8 ? 2 * EoTab<P>::SIZE : 0;
   static constexpr size_t SMEM = (3 * (size_t)K * VOL + TS) * sizeof(T);
   // CTAs per SM the registers are bounded for (FP64, P = 10: two of 320 threads;
   // FP32, P = 8: three instead of two, sem_apply on 16.8 M points 120 against 134 us)
-  static constexpr int MINB = sizeof(T) == 4 ? (P >= 10 ? 2 : P == 8 ? 3 : 1) : (P <= 8 ? 4 : P == 10 ? 2 : 3);
+  static constexpr int MINB =
+      sizeof(T) == 4 ? (P >= 10 ? 512 : P == 8 ? 768 : MOST) / MOST : (P <= 8 ? 4 : P == 10 ? 2 : 3);
 };
 
 // y = D x or D^T x for a line in registers
@@ -53,9 +59,9 @@ __device__ __forceinline__ void line_dots(const T (&x)[P], const DMat<P, T>& D, 
 }
 
 // This thread's place in its element and the element's shared-memory arrays
-template <int P, class T>
+template <int P, class T, int MOST = 256>
 struct LineThread {
-  using C = LineCfg<P, T>;
+  using C = LineCfg<P, T, MOST>;
   int el, lam, i, j, col, ln_r, ln_s;
   T *tab, *U, *R, *S;
   __device__ __forceinline__ void init(unsigned char* smem) {
@@ -78,11 +84,11 @@ struct LineThread {
 // element's G, B and h1 at this thread's (i, j, 0) (h1f may be NULL).  All
 // threads of the CTA call it (act: the thread has an element); U is free once
 // the second barrier is behind.
-template <int P, class T>
-__device__ __forceinline__ void line_element(const LineThread<P, T>& t, bool act,
+template <int P, class T, int MOST>
+__device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bool act,
                                              const DMat<P, T>& D, const T (&uc)[P], const T* g,
                                              const T* b, const T* h1f, T h1, T h2, T (&out)[P]) {
-  using C = LineCfg<P, T>;
+  using C = LineCfg<P, T, MOST>;
   constexpr int P2 = C::P2, P3 = C::P3, RS = C::RS, PL = C::PL;
   constexpr bool PRE = sizeof(T) == 4;       // G prefetched to registers
   T gr[PRE ? P : 1][6];
@@ -138,6 +144,11 @@ __device__ __forceinline__ void line_element(const LineThread<P, T>& t, bool act
       wt[k] = wk;
     }
   }
+  T bk[PRE ? P : 1];                         // on its way while the backward lines run
+  if (PRE && act && h2 != T(0)) {
+#pragma unroll
+    for (int k = 0; k < P; ++k) bk[PRE ? k : 0] = __ldcs(b + k * P2);
+  }
   __syncthreads();
   if (act) {
     T x[P];
@@ -155,7 +166,8 @@ __device__ __forceinline__ void line_element(const LineThread<P, T>& t, bool act
     for (int k = 0; k < P; ++k) out[k] += t.R[k * PL + t.col] + t.S[k * PL + t.col];
     if (h2 != T(0)) {
 #pragma unroll
-      for (int k = 0; k < P; ++k) out[k] = fma(h2 * __ldcs(b + k * P2), uc[k], out[k]);
+      for (int k = 0; k < P; ++k)
+        out[k] = fma(h2 * (PRE ? bk[PRE ? k : 0] : __ldcs(b + k * P2)), uc[k], out[k]);
     }
   }
 }

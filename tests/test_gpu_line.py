@@ -66,3 +66,23 @@ def test_infinities_and_nan_stay_in_their_element(N):
         sem.sem_ax(h, u, w)
         finite = torch.isfinite(w).view(5, -1).all(1).cpu().tolist()
         assert finite == [True, True, False, True, True]
+
+
+@pytest.mark.parametrize("nel,N", [((7, 5, 6), 7), ((9, 4, 5), 6), ((5, 5, 5), 9), ((11, 3, 4), 4),
+                                   ((3, 9, 2), 2), ((1, 5, 4), 8), ((6, 1, 5), 5), ((13, 2, 1), 3)])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_apply_one_finishing_pass(nel, N, dtype):
+    """Boxes whose segments end at different columns of neighbouring rows: the
+    single finishing pass leaves every copy of a point with the same value."""
+    faces = sem.SEM_FACE_YMIN | sem.SEM_FACE_XMAX
+    h = sem.sem_setup(nel, N, length=(TWO_PI,) * 3, deform=0.1, faces=faces)
+    o = OracleProblem(nel, N, length=(TWO_PI,) * 3, deform=0.1, faces=faces)
+    u = si.uniform(o.shape, 66).astype(np.float32).astype(np.float64)
+    ud = torch.from_numpy(u).to(DEV, dtype).view(-1)
+    w = torch.empty_like(ud)
+    sem.sem_apply(h, ud, w, 0.9, 0.4)
+    got = w.double().cpu().numpy().reshape(o.shape)
+    assert rel_inf(got, o.matvec(u, 0.9, 0.4)) < TOL[dtype]
+    first = np.zeros(int(o.gid.max()) + 1)
+    first[o.gid.reshape(-1)] = got.reshape(-1)
+    np.testing.assert_array_equal(first[o.gid], got)
