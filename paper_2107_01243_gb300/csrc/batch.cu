@@ -4,10 +4,10 @@
 // batch).  Every stage of an inner CG iteration is one launch over all
 // problems (per order class for the element kernels).  By default (every
 // handle allows global vectors) the inner PCG runs on global vectors:
-//   bglob   per order class, a persistent element kernel that gathers u from
-//           each problem's lattice and adds face values to its w by L2
-//           reductions (batch_glob.cuh), forming <p, H p> at P = 8
-//   bginit, bgpw, bgupdate, bgpupd  per-problem-chunk vector kernels
+//   bglob   per order class, an element kernel that gathers u from each
+//           problem's lattice and adds face values to its w by L2 reductions
+//           (batch_glob.cuh), forming <p, H p>
+//   bginit, bgupdate, bgpupd  per-problem-chunk vector kernels
 // On L-vectors (SEM_INNER_LOCAL on a handle) the stages are:
 //   bax     persistent bulk-copy (TMA) Ax over all elements of the problems of
 //           one order (one launch per order present, each with the tile and
@@ -34,13 +34,16 @@
 #include "tma.cuh"
 #include "reduce.cuh"
 #include "cg_state.cuh"
-#include "ax_tile.cuh"
+#include "ax_line.cuh"
+#include "fixsum.cuh"
 
 namespace sem {
 
 constexpr int kMaxBatch = 256;
 constexpr int kChunk = 65536;          // points per vector work item
 constexpr int kGChunk = 16384;         // values per global-vector work item
+constexpr int kBatchSlots = 256;       // accumulators of a problem's <p, H p>, one per thread of
+                                       // bgupdate (FP64 additions to one address take 40 ns each)
 
 // batched Ax tile per order: K elements of P^2 threads each per work item
 template <int P>
@@ -96,8 +99,7 @@ struct BProb {
   long long nGp;
   int g_off, g_cnt;
   FastDiv dnx, dny;
-  double* pwacc;         // <p, H p> accumulated by the element kernel (fused_pw)
-  int fused_pw;          // P = 8: the element kernel forms <p, H p>
+  double* pwacc;         // <p, H p> accumulated by the element kernel (kBatchSlots)
 };
 
 __device__ __forceinline__ int find_prob(const long long* off, int n, long long g) {
@@ -582,9 +584,7 @@ struct sem_batch {
   // inner solves on global vectors (every handle allows it): per class the
   // element offsets of its problems, the global vector items
   bool glob = false;
-  DevBuf<long long> cls_eoff[kMaxP + 1];
-  long long Ecls[kMaxP + 1] = {};
-  int bglob_grid[kMaxP + 1] = {};
+  DevBuf<int2> cls_groups[kMaxP + 1];       // (problem, first element) of every CTA
   DevBuf<int> gitem_prob;
   DevBuf<double> pwacc;                  // per problem
   int ngitems = 0;
@@ -650,23 +650,22 @@ static int bapply_occupancy(int ncls) {
 }
 
 template <int P>
-static int bglob_occupancy(int ncls) {
-  using C = BGlobCfg<P>;
-  auto kern = bglob_kernel<P>;
-  SEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)C::smem(kMaxBatch)));
-  int occ = 0;
-  SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, C::THREADS,
-                                                         C::smem(ncls)));
-  return occ;
-}
-
-template <int P>
 static void launch_bglob(sem_batch* bt, cudaStream_t s) {
-  using C = BGlobCfg<P>;
-  bglob_kernel<P><<<bt->bglob_grid[P], C::THREADS, C::smem(bt->ncls[P]), s>>>(
-      bt->probs.ptr, bt->cls_prob[P].ptr, bt->cls_eoff[P].ptr, bt->ncls[P], bt->Ecls[P],
-      bt->hs[0]->dev_err.ptr, kWaitTimeoutNs);
+  using C = LineCfg<P, float, kGlobThreads>;
+  static bool configured = false;
+  if (!configured) {
+    SEM_CUDA(cudaFuncSetAttribute(bglob_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)C::SMEM));
+    configured = true;
+  }
+  DMat<P, float> D;
+  for (const sem_handle* h : bt->hs)
+    if (h->P == P) {
+      for (int a = 0; a < P * P; ++a) D.d[a] = (float)h->Dh[a];
+      break;
+    }
+  bglob_kernel<P><<<(unsigned)bt->cls_groups[P].n, C::THREADS, C::SMEM, s>>>(
+      bt->probs.ptr, bt->cls_groups[P].ptr, D);
   SEM_CHECK_LAUNCH();
 }
 
@@ -743,9 +742,6 @@ static void batch_iteration(sem_batch* bt, cudaStream_t s) {
       }
     });
     const int gblocks = std::min(bt->ngitems, 8 * sem_num_sms());
-    bgpw_kernel<<<gblocks, 256, 0, s>>>(bt->probs.ptr, bt->gitem_prob.ptr, n, bt->ngitems,
-                                        bt->partials.ptr, bt->tickets.ptr);
-    SEM_CHECK_LAUNCH();
     bgupdate_kernel<<<gblocks, 256, 0, s>>>(bt->probs.ptr, bt->gitem_prob.ptr, n, bt->ngitems,
                                             bt->partials.ptr, bt->tickets.ptr);
     SEM_CHECK_LAUNCH();
@@ -932,31 +928,22 @@ extern "C" sem_status sem_batch_create(sem_handle* const* handles, int n, sem_ba
         goff += b.g_cnt;
         b.dnx = FastDiv((uint32_t)b.nelx);
         b.dny = FastDiv((uint32_t)b.nely);
-        b.fused_pw = (b.P * b.P) % 32 == 0 ? 1 : 0;
       }
-      bt->pwacc.alloc(n);
-      SEM_CUDA(cudaMemset(bt->pwacc.ptr, 0, n * sizeof(double)));
-      for (int p = 0; p < n; ++p) bt->hp[p].pwacc = bt->pwacc.ptr + p;
+      bt->pwacc.alloc((size_t)n * kBatchSlots);
+      SEM_CUDA(cudaMemset(bt->pwacc.ptr, 0, n * kBatchSlots * sizeof(double)));
+      for (int p = 0; p < n; ++p) bt->hp[p].pwacc = bt->pwacc.ptr + p * kBatchSlots;
       bt->ngitems = goff;
       bt->gitem_prob.alloc(gitem_prob.size());
       bt->gitem_prob.upload(gitem_prob.data(), gitem_prob.size(), nullptr);
       for (int P = 2; P <= kMaxP; P += 2) {
         if (!bt->ncls[P]) continue;
-        std::vector<long long> eoff;
-        long long Ec = 0;
+        const int K = line_elems(P, false, kGlobThreads);
+        std::vector<int2> groups;
         for (int p = 0; p < n; ++p)
-          if (bt->hp[p].P == P) {
-            eoff.push_back(Ec);
-            Ec += bt->hp[p].E;
-          }
-        bt->Ecls[P] = Ec;
-        bt->cls_eoff[P].alloc(eoff.size());
-        bt->cls_eoff[P].upload(eoff.data(), eoff.size(), nullptr);
-        const int ncl = bt->ncls[P];
-        const int occ = P == 2 ? bglob_occupancy<2>(ncl) : P == 4 ? bglob_occupancy<4>(ncl)
-                      : P == 6 ? bglob_occupancy<6>(ncl) : P == 8 ? bglob_occupancy<8>(ncl)
-                      : bglob_occupancy<10>(ncl);
-        bt->bglob_grid[P] = (int)std::min<long long>(Ec, (long long)std::max(1, occ) * nsm);
+          if (bt->hp[p].P == P)
+            for (int e = 0; e < bt->hp[p].E; e += K) groups.push_back(make_int2(p, e));
+        bt->cls_groups[P].alloc(groups.size());
+        bt->cls_groups[P].upload(groups.data(), groups.size(), nullptr);
       }
     }
     bt->d_off.alloc(n);

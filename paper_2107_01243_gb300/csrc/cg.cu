@@ -24,6 +24,7 @@
 #include "sem_internal.cuh"
 #include "reduce.cuh"
 #include "cg_state.cuh"
+#include "fixsum.cuh"
 #include "df.cuh"
 
 namespace sem {
@@ -97,60 +98,77 @@ k_pw_v(int64_t nv, const typename Vec<T>::V* __restrict__ p, const typename Vec<
 
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-k_update_v(int64_t nv, typename Vec<T>::V* __restrict__ x, typename Vec<T>::V* __restrict__ r,
-           const typename Vec<T>::V* __restrict__ p, const typename Vec<T>::V* __restrict__ w,
-           const typename Vec<T>::V* __restrict__ dinv, const typename Vec<T>::M* __restrict__ imult,
+k_update_v(int64_t nv, typename Vec<T>::V* __restrict__ r,
+           const typename Vec<T>::V* __restrict__ w, const typename Vec<T>::V* __restrict__ dinv, const typename Vec<T>::M* __restrict__ imult,
            CGState* __restrict__ st, double* __restrict__ partials) {
   using VT = Vec<T>;
-  if (st->done) return;
+  if (st_update_skips(st)) return;
   const T alpha = (T)st->alpha;
   Acc<T> a0, a1;
 #pragma unroll 2
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
        q += (int64_t)gridDim.x * blockDim.x) {
-    typename VT::V xq = x[q], rq = r[q];
-    const typename VT::V pq = p[q], wq = w[q], dq = dinv[q];
+    typename VT::V rq = r[q];
+    const typename VT::V wq = w[q], dq = dinv[q];
     const typename VT::M mq = imult[q];
-    T* xe = reinterpret_cast<T*>(&xq);
     T* re = reinterpret_cast<T*>(&rq);
-    const T* pe = reinterpret_cast<const T*>(&pq);
     const T* we = reinterpret_cast<const T*>(&wq);
     const T* de = reinterpret_cast<const T*>(&dq);
     const float* me = reinterpret_cast<const float*>(&mq);
 #pragma unroll
     for (int l = 0; l < VT::L; ++l) {
-      xe[l] += alpha * pe[l];
       re[l] = re[l] - alpha * we[l];
       const T z = de[l] * re[l];
       a0.add(re[l], z, me[l]);
       a1.add(re[l], re[l], me[l]);
     }
-    x[q] = xq;
     r[q] = rq;
   }
   double v[2] = {a0.value(), a1.value()};
   double tot[2];
-  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_update(st, tot);
+  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0)
+    st_after_update(st, tot, kXPending);
 }
 
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-k_pupd_v(int64_t nv, typename Vec<T>::V* __restrict__ p, const typename Vec<T>::V* __restrict__ r,
-         const typename Vec<T>::V* __restrict__ dinv, const CGState* __restrict__ st) {
+k_pupd_v(int64_t nv, typename Vec<T>::V* __restrict__ p, typename Vec<T>::V* __restrict__ x,
+         const typename Vec<T>::V* __restrict__ r, const typename Vec<T>::V* __restrict__ dinv,
+         const CGState* __restrict__ st) {
   using VT = Vec<T>;
-  if (st->done) return;
+  const int done = st->done;
+  if (done == 1) return;
+  const T alpha = (T)st->alpha;
+  if (done == kXPending) {                 // the last x; no further direction
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
+         q += (int64_t)gridDim.x * blockDim.x) {
+      typename VT::V xq = x[q];
+      const typename VT::V pq = p[q];
+      T* xe = reinterpret_cast<T*>(&xq);
+      const T* pe = reinterpret_cast<const T*>(&pq);
+#pragma unroll
+      for (int l = 0; l < VT::L; ++l) xe[l] += alpha * pe[l];
+      x[q] = xq;
+    }
+    return;
+  }
   const T beta = (T)st->beta;
 #pragma unroll 4
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
        q += (int64_t)gridDim.x * blockDim.x) {
-    typename VT::V pq = p[q];
+    typename VT::V pq = p[q], xq = x[q];
     const typename VT::V rq = r[q], dq = dinv[q];
     T* pe = reinterpret_cast<T*>(&pq);
+    T* xe = reinterpret_cast<T*>(&xq);
     const T* re = reinterpret_cast<const T*>(&rq);
     const T* de = reinterpret_cast<const T*>(&dq);
 #pragma unroll
-    for (int l = 0; l < VT::L; ++l) pe[l] = de[l] * re[l] + beta * pe[l];
+    for (int l = 0; l < VT::L; ++l) {
+      xe[l] += alpha * pe[l];
+      pe[l] = de[l] * re[l] + beta * pe[l];
+    }
     p[q] = pq;
+    x[q] = xq;
   }
 }
 
@@ -199,30 +217,44 @@ k_gpw(int64_t nv, const float4* __restrict__ p, const float4* __restrict__ w,
   if (grid_sum<1>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_pw(st, tot[0]);
 }
 
+// slots (may be NULL: alpha from the state): the operator's accumulators of
+// <p, H p>, summed by every block and cleared by the last
 __global__ void __launch_bounds__(kRedThreads)
-k_gupdate(int64_t nv, float4* __restrict__ x, float4* __restrict__ r, const float4* __restrict__ p,
-          float4* __restrict__ w, const float4* __restrict__ dinv, CGState* __restrict__ st,
+k_gupdate(int64_t nv, float4* __restrict__ r, float4* __restrict__ w,
+          const float4* __restrict__ dinv, CGState* __restrict__ st, double* __restrict__ slots,
           double* __restrict__ partials) {
-  if (st->done) return;
-  const float alpha = (float)st->alpha;
+  if (st_update_skips(st)) return;
+  double pw = 0.0, a64 = st->alpha;
+  if (slots) {
+    __shared__ FxVal sw[kRedThreads / 32];
+    for (int q = threadIdx.x; q < kPwSlots; q += kRedThreads) pw += __ldcg(slots + q);
+    pw = fx_block_total<kRedThreads / 32>(pw, sw);
+    a64 = st->rz / pw;
+  }
+  const float alpha = (float)a64;
   const float4 zero = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   Acc<float> a0, a1;
 #pragma unroll 2
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
        q += (int64_t)gridDim.x * blockDim.x) {
-    float4 xq = x[q], rq = r[q];
-    const float4 pq = p[q], wq = w[q], dq = dinv[q];
-    xq.x += alpha * pq.x; xq.y += alpha * pq.y; xq.z += alpha * pq.z; xq.w += alpha * pq.w;
+    float4 rq = r[q];
+    const float4 wq = w[q], dq = dinv[q];
     rq.x -= alpha * wq.x; rq.y -= alpha * wq.y; rq.z -= alpha * wq.z; rq.w -= alpha * wq.w;
     const float4 z = make_float4(dq.x * rq.x, dq.y * rq.y, dq.z * rq.z, dq.w * rq.w);
     rz_rr4(rq, z, a0, a1);
-    x[q] = xq;
     r[q] = rq;
     w[q] = zero;
   }
   double v[2] = {a0.value(), a1.value()};
   double tot[2];
-  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_update(st, tot);
+  if (grid_sum<2>(v, partials, &st->counter, tot)) {
+    if (slots)
+      for (int q = threadIdx.x; q < kPwSlots; q += kRedThreads) slots[q] = 0.0;
+    if (threadIdx.x == 0) {
+      if (slots) st_after_pw(st, pw);      // breakdown when <p, H p> <= 0
+      if (!st->done) st_after_update(st, tot, kXPending);
+    }
+  }
 }
 
 // grid of the padded-vector CG kernels: a thread per float4 up to kRedBlocks
@@ -246,18 +278,17 @@ void vcg_pw(int64_t nv4, const float* p, const float* w, CGState* st, double* pa
   SEM_CHECK_LAUNCH();
 }
 
-void vcg_update(int64_t nv4, float* x, float* r, const float* p, float* w, const float* dinv,
-                CGState* st, double* partials, cudaStream_t s) {
-  k_gupdate<<<vcg_grid(nv4), kRedThreads, 0, s>>>(nv4, (float4*)x, (float4*)r,
-                                                  (const float4*)p, (float4*)w,
-                                                  (const float4*)dinv, st, partials);
+void vcg_update(int64_t nv4, float* r, float* w, const float* dinv, CGState* st, double* slots,
+                double* partials, cudaStream_t s) {
+  k_gupdate<<<vcg_grid(nv4), kRedThreads, 0, s>>>(nv4, (float4*)r, (float4*)w,
+                                                  (const float4*)dinv, st, slots, partials);
   SEM_CHECK_LAUNCH();
 }
 
-void vcg_pupd(int64_t nv4, float* p, const float* r, const float* dinv, const CGState* st,
-              cudaStream_t s) {
-  k_pupd_v<float><<<vcg_grid(nv4), kRedThreads, 0, s>>>(nv4, (float4*)p, (const float4*)r,
-                                                        (const float4*)dinv, st);
+void vcg_pupd(int64_t nv4, float* p, float* x, const float* r, const float* dinv,
+              const CGState* st, cudaStream_t s) {
+  k_pupd_v<float><<<vcg_grid(nv4), kRedThreads, 0, s>>>(nv4, (float4*)p, (float4*)x,
+                                                        (const float4*)r, (const float4*)dinv, st);
   SEM_CHECK_LAUNCH();
 }
 
@@ -291,21 +322,18 @@ k_pw_v64(int64_t nv, const double2* __restrict__ p, const double2* __restrict__ 
 }
 
 __global__ void __launch_bounds__(kRedThreads)
-k_update_v64(int64_t nv, double2* __restrict__ x, double2* __restrict__ r,
-             const double2* __restrict__ p, const double2* __restrict__ w,
+k_update_v64(int64_t nv, double2* __restrict__ r, const double2* __restrict__ w,
              const double2* __restrict__ dmi, const float2* __restrict__ imult,
              CGState* __restrict__ st, double* __restrict__ partials) {
-  if (st->done) return;
+  if (st_update_skips(st)) return;
   const double alpha = st->alpha;
   double rz = 0.0, rr = 0.0;
 #pragma unroll 2
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
        q += (int64_t)gridDim.x * blockDim.x) {
-    double2 xq = x[q], rq = r[q];
-    const double2 pq = p[q], wq = w[q], dq = dmi[q];
+    double2 rq = r[q];
+    const double2 wq = w[q], dq = dmi[q];
     const float2 mq = imult[q];
-    xq.x = fma(alpha, pq.x, xq.x);
-    xq.y = fma(alpha, pq.y, xq.y);
     rq.x = fma(-alpha, wq.x, rq.x);
     rq.y = fma(-alpha, wq.y, rq.y);
     const double sx = rq.x * rq.x, sy = rq.y * rq.y;
@@ -313,12 +341,12 @@ k_update_v64(int64_t nv, double2* __restrict__ x, double2* __restrict__ r,
     rz = fma(sy, dq.y, rz);
     rr = fma(sx, pow2_widen(mq.x), rr);
     rr = fma(sy, pow2_widen(mq.y), rr);
-    x[q] = xq;
     r[q] = rq;
   }
   double v[2] = {rz, rr};
   double tot[2];
-  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_update(st, tot);
+  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0)
+    st_after_update(st, tot, kXPending);
 }
 
 template <class T>
@@ -360,15 +388,14 @@ k_pw(int64_t n, const T* __restrict__ p, const T* __restrict__ w, const float* _
 
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-k_update(int64_t n, T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
-         const T* __restrict__ w, const T* __restrict__ dinv, const float* __restrict__ imult,
-         CGState* __restrict__ st, double* __restrict__ partials) {
-  if (st->done) return;
+k_update(int64_t n, T* __restrict__ r, const T* __restrict__ w, const T* __restrict__ dinv,
+         const float* __restrict__ imult, CGState* __restrict__ st,
+         double* __restrict__ partials) {
+  if (st_update_skips(st)) return;
   const T alpha = (T)st->alpha;
   Acc<T> a0, a1;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
-    x[q] += alpha * p[q];
     T rq = r[q] - alpha * w[q];
     r[q] = rq;
     T z = dinv[q] * rq;
@@ -378,18 +405,23 @@ k_update(int64_t n, T* __restrict__ x, T* __restrict__ r, const T* __restrict__ 
   }
   double v[2] = {a0.value(), a1.value()};
   double tot[2];
-  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_update(st, tot);
+  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0)
+    st_after_update(st, tot, kXPending);
 }
 
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-k_pupd(int64_t n, T* __restrict__ p, const T* __restrict__ r, const T* __restrict__ dinv,
-       const CGState* __restrict__ st) {
-  if (st->done) return;
-  const T beta = (T)st->beta;
+k_pupd(int64_t n, T* __restrict__ p, T* __restrict__ x, const T* __restrict__ r,
+       const T* __restrict__ dinv, const CGState* __restrict__ st) {
+  const int done = st->done;
+  if (done == 1) return;
+  const T alpha = (T)st->alpha, beta = (T)st->beta;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
-       q += (int64_t)gridDim.x * blockDim.x)
-    p[q] = dinv[q] * r[q] + beta * p[q];
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const T pq = p[q];
+    x[q] += alpha * pq;
+    if (done == 0) p[q] = dinv[q] * r[q] + beta * pq;
+  }
 }
 
 // r64 = b - w64 (FP64 residual), optional FP32 copy of rscale r64, <r,r> into st->rr
@@ -655,10 +687,11 @@ static void launch_vec64(sem_handle* h, const PcgArgs<double>& a, bool pw_done, 
     SEM_CHECK_LAUNCH();
   }
   k_update_v64<<<kRedBlocks, kRedThreads, 0, s>>>(
-      nv, (double2*)a.x, (double2*)a.r, (const double2*)a.p, (const double2*)a.w,
-      (const double2*)a.dmi, (const float2*)h->imult.ptr, a.st, h->partials.ptr);
+      nv, (double2*)a.r, (const double2*)a.w, (const double2*)a.dmi,
+      (const float2*)h->imult.ptr, a.st, h->partials.ptr);
   SEM_CHECK_LAUNCH();
-  k_pupd_v<double><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (double2*)a.p, (const double2*)a.r,
+  k_pupd_v<double><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (double2*)a.p, (double2*)a.x,
+                                                      (const double2*)a.r,
                                                       (const double2*)a.dinv, a.st);
   SEM_CHECK_LAUNCH();
 }
@@ -689,12 +722,12 @@ static void pcg_iterations(sem_handle* h, const PcgArgs<T>& a, int count, cudaSt
                                                      h->partials.ptr);
         SEM_CHECK_LAUNCH();
       }
-      k_update_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.x, (V*)a.r, (const V*)a.p,
-                                                       (const V*)a.w, (const V*)a.dinv,
+      k_update_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.r, (const V*)a.w,
+                                                       (const V*)a.dinv,
                                                        (const M*)h->imult.ptr, a.st,
                                                        h->partials.ptr);
       SEM_CHECK_LAUNCH();
-      k_pupd_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.p, (const V*)a.r,
+      k_pupd_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.p, (V*)a.x, (const V*)a.r,
                                                      (const V*)a.dinv, a.st);
       SEM_CHECK_LAUNCH();
     } else {
@@ -703,10 +736,10 @@ static void pcg_iterations(sem_handle* h, const PcgArgs<T>& a, int count, cudaSt
                                                    h->partials.ptr);
         SEM_CHECK_LAUNCH();
       }
-      k_update<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.x, a.r, a.p, a.w, a.dinv, h->imult.ptr,
-                                                     a.st, h->partials.ptr);
+      k_update<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.r, a.w, a.dinv, h->imult.ptr, a.st,
+                                                     h->partials.ptr);
       SEM_CHECK_LAUNCH();
-      k_pupd<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.p, a.r, a.dinv, a.st);
+      k_pupd<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.p, a.x, a.r, a.dinv, a.st);
       SEM_CHECK_LAUNCH();
     }
   }
@@ -717,11 +750,9 @@ static void glob_iterations(sem_handle* h, CGState* st, float h1, float h2, int 
                             cudaStream_t s) {
   const int64_t nv4 = glob_padded(h) / 4;
   for (int c = 0; c < count; ++c) {
-    const bool pw_done = launch_apply_global(h, h->pg.ptr, h->wg.ptr, h1, h2, st, st, s);
-    if (!pw_done) vcg_pw(nv4, h->pg.ptr, h->wg.ptr, st, h->partials.ptr, s);
-    vcg_update(nv4, h->xg.ptr, h->rg.ptr, h->pg.ptr, h->wg.ptr, h->dinvg.ptr, st,
-               h->partials.ptr, s);
-    vcg_pupd(nv4, h->pg.ptr, h->rg.ptr, h->dinvg.ptr, st, s);
+    launch_apply_global(h, h->pg.ptr, h->wg.ptr, h1, h2, st, true, s);
+    vcg_update(nv4, h->rg.ptr, h->wg.ptr, h->dinvg.ptr, st, pw_slots(h), h->partials.ptr, s);
+    vcg_pupd(nv4, h->pg.ptr, h->xg.ptr, h->rg.ptr, h->dinvg.ptr, st, s);
   }
 }
 
@@ -951,6 +982,7 @@ void glob_prepare(sem_handle* h, cudaStream_t s) {
     }
   }
   to_global<float>(h, h->f32.dinv.ptr, h->dinvg.ptr, s);
+  SEM_CUDA(cudaMemsetAsync(pw_slots(h), 0, kPwSlots * sizeof(double), s));
 }
 
 static void solve_mixed(sem_handle* h, const double* b, double* x, const sem_solve_opts& o,

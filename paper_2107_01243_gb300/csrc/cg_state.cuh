@@ -33,22 +33,33 @@ __device__ __forceinline__ void st_after_pw(CGState* st, double pw) {
   }
 }
 
-// after the x, r update (tot = {<r, z>, <r, r>}): stop test, beta
-__device__ __forceinline__ void st_after_update(CGState* st, const double (&tot)[2]) {
+// after the r update (tot = {<r, z>, <r, r>}): stop test, beta.  fin: the value
+// of done when the solve ends here: 2 where x is advanced by the direction
+// kernel that follows (kXPending; the next update kernel turns it into 1)
+constexpr int kXPending = 2;
+__device__ __forceinline__ void st_after_update(CGState* st, const double (&tot)[2], int fin = 1) {
   st->iter += 1;
   st->rr = tot[1];
   if (!(tot[1] == tot[1]) || !(tot[0] == tot[0])) {
     st->status = SEM_ERR_BREAKDOWN;
-    st->done = 1;
+    st->done = fin;
   } else if (tot[1] <= st->tol2) {
-    st->done = 1;
+    st->done = fin;
   } else if (st->iter >= st->maxit) {
     st->status = SEM_ERR_NOCONV;
-    st->done = 1;
+    st->done = fin;
   } else {
     st->beta = tot[0] / st->rz;
     st->rz = tot[0];
   }
+}
+
+// an update kernel's entry: whether the solve is over (a pending x has been
+// advanced by now)
+__device__ __forceinline__ bool st_update_skips(CGState* st) {
+  const int done = st->done;
+  if (done == kXPending && blockIdx.x == 0 && threadIdx.x == 0) st->done = 1;
+  return done != 0;
 }
 
 }  // namespace sem

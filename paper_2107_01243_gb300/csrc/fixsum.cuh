@@ -121,6 +121,22 @@ __device__ __forceinline__ FxAcc fx_warp_add(const FxAcc& a) {
   t.hi = ((long long)h1 << 27) + (long long)h0;
   return t;
 }
+// sum of v over a CTA of NW warps, in every thread (two barriers; sw: NW entries
+// of shared memory)
+template <int NW>
+__device__ __forceinline__ double fx_block_total(double v, FxVal* sw) {
+  const int lane = threadIdx.x & 31;
+  const FxVal f = fx_warp_sum(v);
+  __syncthreads();
+  if (lane == 0) sw[threadIdx.x >> 5] = f;
+  __syncthreads();
+  const FxVal f0 = lane < NW ? sw[lane] : FxVal{0, 1};
+  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f0.e);
+  FxAcc acc;
+  if (e < kFxBad) acc.add(f0, e);
+  acc = fx_warp_add(acc);
+  return fx_round(acc.hi, acc.lo, e);
+}
 #endif
 
 }  // namespace sem

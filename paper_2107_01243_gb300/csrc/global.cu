@@ -19,7 +19,8 @@
 
 #include "sem_internal.cuh"
 #include "tma.cuh"
-#include "ax_tile.cuh"
+#include "ax_line.cuh"
+#include "fixsum.cuh"
 #include "reduce.cuh"
 #include "cg_state.cuh"
 
@@ -54,150 +55,77 @@ __device__ __forceinline__ unsigned dirichlet_bits(const GBox& b, int ex, int ey
          ((b.faces & SEM_FACE_ZMAX) && ez == b.nelz - 1 ? 128u : 0u);
 }
 
-// A persistent CTA of P x P threads walks elements blockIdx.x + m gridDim.x.
-// Thread 0 keeps STAGES elements' geometric factors (and B) in flight by bulk
-// copies on mbarriers (a stage is refilled once the forward phase is done); every thread gathers its own k-column of the next
-// element's u into a second shared buffer by cp.async while the current one
-// is computed.  w must hold zeros at every unmasked point on element faces.
-// pwst (P = 8): <p, H p> and alpha from the local products, p = u (the sum
-// over local points of u_L (H_L u_L), equal to the global product because u
-// is zero on Dirichlet points).
-template <int P, int STAGES>
-__global__ void __launch_bounds__(P * P)
+// A CTA takes K consecutive elements (ax_line.cuh): every thread
+// gathers its own k-column of u from the lattice (rows of P consecutive floats;
+// what neighbours share comes from L2) and scatters its column of outputs.
+// With the clearing of w, on 17 M points: N = 3 102 us, N = 5 115, N = 7 101, N = 9
+// 147 (Poisson; with a mass term 112, 131, 106, 150).  The kernel it took the
+// place of staged G by bulk copies and read a row and a column of shared memory
+// for every point: 149, 146, 113, 150 (154, 150, 128, 153).  w
+// must hold zeros at every unmasked point on element faces.
+// PW: <p, H p> from the local products, p = u (the sum over local
+// points of u_L (H_L u_L), equal to the global product because u is zero on
+// Dirichlet points), every warp's sum added to one of kPwSlots accumulators (in
+// no fixed order, as the face sums of w).
+// No loop over elements: with one the compiler keeps D in registers.
+template <int P, bool PW>
+__global__ void __launch_bounds__(LineCfg<P, float, kGlobThreads>::THREADS, LineCfg<P, float, kGlobThreads>::MINB)
 ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* __restrict__ G,
-               const float* __restrict__ B, float h1, float h2, DMat<P, float> D, int E, GBox bx,
-               const CGState* __restrict__ st, CGState* __restrict__ pwst,
-               double* __restrict__ partials, int* __restrict__ err, uint64_t timeout_ns) {
-  constexpr int P2 = P * P, P3 = P2 * P, N = P - 1;
-  constexpr uint32_t FB = P3 * sizeof(float);
+               const float* __restrict__ B, float h1, float h2,
+               const __grid_constant__ DMat<P, float> D, int E, GBox bx,
+               const CGState* __restrict__ st, double* __restrict__ slots) {
+  using C = LineCfg<P, float, kGlobThreads>;
+  constexpr int P3 = C::P3, K = C::K, N = P - 1;
   if (st && st->done) return;
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw);
-  float* stage0 = reinterpret_cast<float*>(smem_raw + 128);
-  const bool helm = h2 != 0.0f;
-  const int nf = 6 + (helm ? 1 : 0);
-  const int SE = nf * P3;
-  float* su = stage0 + STAGES * SE;        // [2][P3]: gathered u, double-buffered
-  float* sT = su + 2 * P3;
-  float* swr = su + 3 * P3;
-  float* swsT = su + 4 * P3;
-  const int tid = threadIdx.x;
-  auto Dm = [&](int r, int c) { return D.d[r * P + c]; };
-  TileThread<P, float> t;
-  t.init(tid, Dm);
-  const long long toff = t.i + (long long)bx.gx * t.j;    // this thread's (i, j, 0)
-  auto gather = [&](int e, float* dst) {
-    int ex, ey, ez;
-    const float* src = u + elem_origin(e, bx, N, ex, ey, ez) + toff;
-#pragma unroll
-    for (int k = 0; k < P; ++k) cp_async4(dst + k * P2 + t.lt, src + bx.sk * k);
-  };
-  auto issue = [&](int e, int s) {
-    float* dst = stage0 + s * SE;
-    const uint64_t pol = l2_policy_evict_first();   // G and B are read once
-    mbar_arrive_expect_tx(&bar[s], (uint32_t)nf * FB);
-    bulk_g2s_hint(dst, G + (size_t)e * 6 * P3, 6 * FB, &bar[s], pol);
-    if (helm) bulk_g2s_hint(dst + 6 * P3, B + (size_t)e * P3, FB, &bar[s], pol);
-  };
-  if (tid == 0) {
-#pragma unroll
-    for (int s = 0; s < STAGES; ++s) mbar_init(&bar[s], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  const int Gs = gridDim.x;
-  int issued = 0;
-  if (tid == 0) {
-#pragma unroll
-    for (int s = 0; s < STAGES; ++s) {
-      const int e = blockIdx.x + s * Gs;
-      if (e < E) {
-        issue(e, s);
-        ++issued;
-      }
-    }
-  }
-  if (blockIdx.x < E) gather(blockIdx.x, su);
-  cp_async_commit();
-  float pw_s = 0.0f, pw_c = 0.0f;          // Kahan-compensated <p, H p>
-  const bool fi = t.i == 0 || t.i == N, fj = t.j == 0 || t.j == N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  LineThread<P, float, kGlobThreads> t;
+  t.init(smem_raw);
+  const int toff = t.i + bx.gx * t.j, sk = (int)bx.sk;      // n_G < 2^31
+  const bool fij = t.i == 0 || t.i == N || t.j == 0 || t.j == N;
   const unsigned pij = (t.i == 0 ? 4u : 0u) | (t.i == N ? 8u : 0u) | (t.j == 0 ? 16u : 0u) |
                        (t.j == N ? 32u : 0u);
-  int n = 0;
-  for (int e = blockIdx.x; e < E; e += Gs, ++n) {
-    const int s = n % STAGES;
-    const bool ok = mbar_wait_bounded(&bar[s], (uint32_t)(n / STAGES) & 1u, err, timeout_ns);
-    // the other buffer was last read before the previous iteration's second barrier
-    const float* cu = su + (n & 1) * P3;
-    if (e + Gs < E) gather(e + Gs, su + ((n + 1) & 1) * P3);
-    cp_async_commit();
-    cp_async_wait<1>();                    // this thread's copies of element e landed
-    float uc[P], bk[P], ck[P], wt[P];
-    const float* sg = stage0 + s * SE;
+  const int e = blockIdx.x * K + t.el;
+  const bool act = t.el < K && e < E;
+  int ex, ey, ez;
+  const int org = (int)elem_origin(act ? e : 0, bx, N, ex, ey, ez) + toff;
+  float uc[P], out[P];
+  if (act) {
+#pragma unroll
+    for (int k = 0; k < P; ++k) uc[k] = __ldg(u + (org + sk * k));
+  }
+  const size_t base = (size_t)(act ? e : 0) * P3 + t.lam;
+  line_element(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
+               (const float*)nullptr, h1, h2, out);
+  float pw = 0.0f;
+  if (act) {
+    int dst0 = org;                        // the column's addresses are made anew:
+    asm volatile("" : "+r"(dst0));         // kept since the gather they would spill
+    const unsigned fl = dirichlet_bits(bx, ex, ey, ez);
+    float pw_c = 0.0f;                     // Kahan-compensated <p, H p>
 #pragma unroll
     for (int k = 0; k < P; ++k) {
-      uc[k] = cu[k * P2 + t.lt];
-      sT[k * P2 + t.tpos] = uc[k];
-      ck[k] = h1;
-      bk[k] = helm ? sg[6 * P3 + k * P2 + t.lt] : 0.0f;
-    }
-    if (__syncthreads_or(!ok)) {
-      // a copy never completed: wait (bounded) for what is in flight, then leave
-      cp_async_wait<0>();
-      if (tid == 0)
-        for (int nn = n; nn < issued; ++nn)
-          mbar_wait_bounded(&bar[nn % STAGES], (uint32_t)(nn / STAGES) & 1u, err, timeout_ns);
-      break;                               // the reduction below still counts this CTA
-    }
-    tile_forward<P, float>(t, cu, sT, sg, uc, ck, swr, swsT, wt, Dm);
-    __syncthreads();
-    if (tid == 0) {                        // stage s consumed
-      const int en = e + STAGES * Gs;
-      if (en < E) {
-        fence_proxy_async_smem();
-        issue(en, s);
-        ++issued;
-      }
-    }
-    int ex, ey, ez;
-    float* we = w + elem_origin(e, bx, N, ex, ey, ez) + toff;
-    const unsigned fl = dirichlet_bits(bx, ex, ey, ez);
-    tile_backward<P, float>(t, swr, swsT, wt, uc, bk, h2, helm, Dm, [&](int k, float v) {
-      if (pwst) {
-        const float y = __fsub_rn(__fmul_rn(uc[k], v), pw_c);
-        const float tt = __fadd_rn(pw_s, y);
-        pw_c = __fsub_rn(__fsub_rn(tt, pw_s), y);
-        pw_s = tt;
+      if (PW) {
+        const float y = __fsub_rn(__fmul_rn(uc[k], out[k]), pw_c);
+        const float tt = __fadd_rn(pw, y);
+        pw_c = __fsub_rn(__fsub_rn(tt, pw), y);
+        pw = tt;
       }
       const unsigned pf = pij | (k == 0 ? 64u : 0u) | (k == N ? 128u : 0u);
-      if (pf & fl) return;                 // Dirichlet point: stays zero
-      float* dst = we + bx.sk * k;
-      if (fi || fj || k == 0 || k == N)
-        red_add(dst, v);                   // shared with neighbours
+      if (pf & fl) continue;               // Dirichlet point: stays zero
+      float* dst = w + (dst0 + sk * k);
+      if (fij || k == 0 || k == N)
+        red_add(dst, out[k]);              // shared with neighbours
       else
-        *dst = v;                          // interior: this element's alone
-    });
-  }
-  cp_async_wait<0>();
-  if constexpr (P2 % 32 == 0) {
-    if (pwst) {
-      double v[1] = {(double)pw_s - (double)pw_c};
-      double tot[1];
-      if (grid_sum<1>(v, partials, &pwst->counter, tot) && threadIdx.x == 0) {
-        st_after_pw(pwst, tot[0]);
-      }
+        *dst = out[k];                     // interior: this element's alone
     }
   }
-}
-
-// one stage of geometric factors: 24.7 KB of shared memory at P = 8, eight
-// CTAs per SM (two stages: six CTAs, 16% slower at 48^3 elements, N = 7)
-constexpr int kGlobStages = 1;
-
-template <int P>
-static size_t glob_smem_bytes(bool helm) {
-  const size_t P3 = (size_t)P * P * P;
-  return 128 + (kGlobStages * (6 + (helm ? 1 : 0)) + 5) * P3 * sizeof(float);
+  if constexpr (PW) {
+    constexpr int NW = C::THREADS / 32;
+    const FxVal f = fx_warp_sum((double)pw);
+    if ((threadIdx.x & 31) == 0)
+      atomicAdd(slots + (blockIdx.x * NW + (threadIdx.x >> 5)) % kPwSlots,
+                fx_round(f.m >> 32, (long long)(unsigned)f.m, f.e));
+  }
 }
 
 static GBox make_gbox(const sem_handle* h) {
@@ -213,33 +141,26 @@ static GBox make_gbox(const sem_handle* h) {
   return b;
 }
 
-template <int P>
+double* pw_slots(const sem_handle* h) {
+  return h->partials.ptr + 6 * kRedBlocks + kFusedPartials;
+}
+
+template <int P, bool PW>
 static void launch_glob_p(const sem_handle* h, const float* u, float* w, float h1, float h2,
-                          const CGState* st, CGState* pwst, cudaStream_t s) {
-  const bool helm = h2 != 0.0f;
-  auto kern = ax_glob_kernel<P, kGlobStages>;
+                          const CGState* st, cudaStream_t s) {
+  using C = LineCfg<P, float, kGlobThreads>;
+  auto kern = ax_glob_kernel<P, PW>;
   static bool configured = false;
-  static int occ[2] = {0, 0};
   if (!configured) {
     SEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)glob_smem_bytes<P>(true)));
+                                  (int)C::SMEM));
     configured = true;
-  }
-  const size_t smem = glob_smem_bytes<P>(helm);
-  int& o = occ[helm ? 1 : 0];
-  if (!o) {
-    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, P * P, smem));
-    if (o < 1) o = 1;
   }
   DMat<P, float> D;
   for (int a = 0; a < P * P; ++a) D.d[a] = (float)h->Dh[a];
   const int E = (int)h->E;
-  int grid = (int)std::min<int64_t>(E, (int64_t)o * sem_num_sms());
-  if (pwst) grid = std::min(grid, kFusedPartials);
-  if (grid < 1) grid = 1;
-  kern<<<grid, P * P, smem, s>>>(u, w, h->f32.G.ptr, h->f32.B.ptr, h1, h2, D, E, make_gbox(h), st,
-                                 pwst, h->partials.ptr + 4 * kRedBlocks, h->dev_err.ptr,
-                                 kWaitTimeoutNs);
+  kern<<<(E + C::K - 1) / C::K, C::THREADS, C::SMEM, s>>>(u, w, h->f32.G.ptr, h->f32.B.ptr, h1, h2,
+                                                          D, E, make_gbox(h), st, pw_slots(h));
   SEM_CHECK_LAUNCH();
 }
 
@@ -251,14 +172,21 @@ bool glob_supported(const sem_handle* h) {
 
 int64_t glob_padded(const sem_handle* h) { return (h->nG + 3) / 4 * 4; }
 
-bool launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,
-                         const CGState* st, CGState* pwst, cudaStream_t s) {
+template <int P>
+static void launch_glob_any(const sem_handle* h, const float* u, float* w, float h1, float h2,
+                            const CGState* st, bool pw, cudaStream_t s) {
+  if (pw) launch_glob_p<P, true>(h, u, w, h1, h2, st, s);
+  else launch_glob_p<P, false>(h, u, w, h1, h2, st, s);
+}
+
+void launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,
+                         const CGState* st, bool pw, cudaStream_t s) {
   switch (h->P) {
-    case 2: launch_glob_p<2>(h, u, w, h1, h2, st, nullptr, s); return false;
-    case 4: launch_glob_p<4>(h, u, w, h1, h2, st, nullptr, s); return false;
-    case 6: launch_glob_p<6>(h, u, w, h1, h2, st, nullptr, s); return false;
-    case 8: launch_glob_p<8>(h, u, w, h1, h2, st, pwst, s); return pwst != nullptr;
-    case 10: launch_glob_p<10>(h, u, w, h1, h2, st, nullptr, s); return false;
+    case 2: launch_glob_any<2>(h, u, w, h1, h2, st, pw, s); break;
+    case 4: launch_glob_any<4>(h, u, w, h1, h2, st, pw, s); break;
+    case 6: launch_glob_any<6>(h, u, w, h1, h2, st, pw, s); break;
+    case 8: launch_glob_any<8>(h, u, w, h1, h2, st, pw, s); break;
+    case 10: launch_glob_any<10>(h, u, w, h1, h2, st, pw, s); break;
     default: throw Error(SEM_ERR_ARG, "apply_global: unsupported order");
   }
 }
@@ -348,7 +276,7 @@ extern "C" sem_status sem_apply_global(sem_handle* h, const void* u_g, void* w_g
                                    "and fewer than 2^31 local points");
     const cudaStream_t s = (cudaStream_t)stream;
     SEM_CUDA(cudaMemsetAsync(w_g, 0, h->nG * sizeof(float), s));
-    launch_apply_global(h, (const float*)u_g, (float*)w_g, (float)h1, (float)h2, nullptr, nullptr,
+    launch_apply_global(h, (const float*)u_g, (float*)w_g, (float)h1, (float)h2, nullptr, false,
                         s);
   });
 }

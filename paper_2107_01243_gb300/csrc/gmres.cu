@@ -518,7 +518,7 @@ void gmres_solve_mixed(sem_handle* h, const double* b, double* x, const sem_solv
         SEM_CUDA(cudaMemcpyAsync(g.r.ptr, r_in, gbytes, cudaMemcpyDeviceToDevice, s));
       } else {
         SEM_CUDA(cudaMemsetAsync(g.w.ptr, 0, gbytes, s));
-        launch_apply_global(h, g.d.ptr, g.w.ptr, (float)o.h1, (float)o.h2, nullptr, nullptr, s);
+        launch_apply_global(h, g.d.ptr, g.w.ptr, (float)o.h1, (float)o.h2, nullptr, false, s);
         k_subf<<<lin_grid(n4), 256, 0, s>>>(n4, r_in, g.w.ptr, g.r.ptr);
         SEM_CHECK_LAUNCH();
       }
@@ -533,7 +533,7 @@ void gmres_solve_mixed(sem_handle* h, const double* b, double* x, const sem_solv
       for (int j = 0; j < m; ++j) {
         schwarz_apply_global(M, g.V[j]->ptr, g.Z[j]->ptr, s);
         SEM_CUDA(cudaMemsetAsync(g.w.ptr, 0, gbytes, s));
-        launch_apply_global(h, g.Z[j]->ptr, g.w.ptr, (float)o.h1, (float)o.h2, nullptr, nullptr,
+        launch_apply_global(h, g.Z[j]->ptr, g.w.ptr, (float)o.h1, (float)o.h2, nullptr, false,
                             s);
         const int cnt = j + 1;
         const dim3 dgrid(kRedBlocks, (cnt + kGsChunk - 1) / kGsChunk);

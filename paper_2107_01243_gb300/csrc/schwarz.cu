@@ -621,9 +621,8 @@ const float* schwarz_levels(sem_schwarz* sw, const float* rg, float* zg, cudaStr
                                                       sw->wc.ptr, h->nelx, h->nely, dnx, dny);
       SEM_CHECK_LAUNCH();
       vcg_pw(sw->nv4, sw->pc.ptr, sw->wc.ptr, st, sw->partials.ptr, s);
-      vcg_update(sw->nv4, sw->xc.ptr, sw->rc.ptr, sw->pc.ptr, sw->wc.ptr, sw->cdinv.ptr, st,
-                 sw->partials.ptr, s);
-      vcg_pupd(sw->nv4, sw->pc.ptr, sw->rc.ptr, sw->cdinv.ptr, st, s);
+      vcg_update(sw->nv4, sw->rc.ptr, sw->wc.ptr, sw->cdinv.ptr, st, nullptr, sw->partials.ptr, s);
+      vcg_pupd(sw->nv4, sw->pc.ptr, sw->xc.ptr, sw->rc.ptr, sw->cdinv.ptr, st, s);
     }
   }
   return coarse ? sw->xc.ptr : nullptr;

@@ -27,6 +27,10 @@ constexpr int kMaxP = kMaxN + 1;
 // product, are then the same on any device.
 constexpr int kRedBlocks = 608;
 constexpr int kRedThreads = 256;
+// accumulators of the global operator's <p, H p>: one address takes an FP64
+// addition every 40 ns or so (32 of them cost 100 us on 32^3 elements, 65,000
+// warps), 1024 hide them
+constexpr int kPwSlots = 1024;
 constexpr int kFusedPartials = 2048;   // partials of the element kernels' fused <p, Hp>
 constexpr uint64_t kWaitTimeoutNs = 2000000000ull;   // bounded device waits give up after 2 s
 
@@ -141,7 +145,7 @@ struct CGState {
   double alpha, beta;
   double tol2;      // (tol)^2 * <b,b>: convergence threshold on <r,r>
   int iter;         // completed iterations
-  int done;         // 1 once converged or failed
+  int done;         // nonzero once converged or failed (2: x not advanced yet, cg_state.cuh)
   int status;       // SEM_OK / SEM_ERR_BREAKDOWN
   int maxit;
   unsigned int counter;   // last-block-done ticket for the reductions
@@ -208,7 +212,8 @@ struct sem_handle {
   int cg_variant = SEM_CG_STANDARD;         // sem_set_cg_variant
   sem::DevBuf<double> pipe_u, pipe_z, pipe_q, pipe_s, pipe_m, pipe_n;   // pipelined CG
   // reduction partials (B = kRedBlocks): [0,2B) solves, [2B,3B) sem_dot,
-  // [4B,4B+F) the element kernels' fused <p, Hp>, [4B+F,6B+F) sem_cg_update
+  // [4B,4B+F) the element kernels' fused <p, Hp>, [4B+F,6B+F) sem_cg_update,
+  // then the global operator's kPwSlots accumulators (zero between launches)
   sem::DevBuf<double> partials;
   // [4]: outer/FP64, inner/FP32, sem_dot ticket, sem_cg_update ticket
   sem::DevBuf<sem::CGState> state;
@@ -314,11 +319,13 @@ void outer_residual_global(sem_handle* h, const double* b, const double* x,
 CGState state_to_host(const CGState* d, cudaStream_t s, int* dev_err);
 
 // ---- global.cu: the FP32 operator on global vectors, w_g = mask Q^T H_L Q u_g
-// (w_g must hold zeros at unmasked element-face points); pwst as launch_apply
+// (w_g must hold zeros at unmasked element-face points); pw: u is a CG direction,
+// whose <u, H u> is added to pw_slots(h) (kPwSlots doubles, zero before)
 bool glob_supported(const sem_handle* h);
 int64_t glob_padded(const sem_handle* h);          // n_G rounded up to a multiple of 4
-bool launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,
-                         const CGState* st, CGState* pwst, cudaStream_t s);
+void launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,
+                         const CGState* st, bool pw, cudaStream_t s);
+double* pw_slots(const sem_handle* h);
 template <class Tin>
 void to_global(const sem_handle* h, const Tin* in, float* out, cudaStream_t s,
                double scale = 1.0);                                    // owner copies x scale
@@ -338,10 +345,12 @@ void vcg_init(int64_t nv4, const float* r, const float* dinv, float* p, float* x
               CGState* st, double* partials, double tol, int maxit, cudaStream_t s);
 void vcg_pw(int64_t nv4, const float* p, const float* w, CGState* st, double* partials,
             cudaStream_t s);
-void vcg_update(int64_t nv4, float* x, float* r, const float* p, float* w, const float* dinv,
-                CGState* st, double* partials, cudaStream_t s);
-void vcg_pupd(int64_t nv4, float* p, const float* r, const float* dinv, const CGState* st,
-              cudaStream_t s);
+// slots (may be NULL): <p, H p> comes from the operator's accumulators
+void vcg_update(int64_t nv4, float* r, float* w, const float* dinv, CGState* st, double* slots,
+                double* partials, cudaStream_t s);
+// x += alpha p, then the next direction
+void vcg_pupd(int64_t nv4, float* p, float* x, const float* r, const float* dinv,
+              const CGState* st, cudaStream_t s);
 // Jacobi inverse diagonal of (h1, h2) for the FP64 operator (L-vector, masked)
 const double* jacobi_dinv64(sem_handle* h, double h1, double h2, cudaStream_t s);
 // w = mask o QQ^T H x, r = b - w and <r, r> into st->rr (FP64 L-vectors)

@@ -505,7 +505,8 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     SEM_CUDA(cudaMemsetAsync(h->dev_err.ptr, 0, sizeof(int), s));
     h->state.alloc(4);
     SEM_CUDA(cudaMemsetAsync(h->state.ptr, 0, 4 * sizeof(CGState), s));
-    h->partials.alloc(6 * kRedBlocks + kFusedPartials);
+    h->partials.alloc(6 * kRedBlocks + kFusedPartials + kPwSlots);
+    SEM_CUDA(cudaMemsetAsync(h->partials.ptr, 0, h->partials.n * sizeof(double), s));
     SEM_CUDA(cudaStreamSynchronize(s));
     *out = h.release();
   });
