@@ -24,6 +24,7 @@
 
 #include "sem_internal.cuh"
 #include "reduce.cuh"
+#include "fixsum.cuh"
 #include "krylov.cuh"
 
 namespace sem {
@@ -194,42 +195,110 @@ struct KahanAcc {
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
-// out[i] = <V_i, w>, i < cnt (blockIdx.y: chunk of kGsChunk vectors)
-__global__ void __launch_bounds__(kRedThreads)
-k_gsf_dots(int64_t n4, const float* const* __restrict__ V, int cnt, const float* __restrict__ w,
-           double* __restrict__ out, double* __restrict__ partials,
-           unsigned* __restrict__ counters) {
-  const int i0 = blockIdx.y * kGsChunk;
-  const int c = min(kGsChunk, cnt - i0);
-  const float4* v[kGsChunk];
+// The grid's sums of v[q] into out[q], q < cnt, by the last block to finish
+// (integer sums, fixsum.cuh: eight FP64 shuffle trees a block took as long as
+// reading two vectors).  partials: NV gridDim.x entries, in the fixed order of
+// the blocks; counter resets itself.
+template <int NV>
+__device__ __forceinline__ void grid_sum_fx(const double (&v)[NV], int cnt, double* out,
+                                            longlong2* partials, unsigned* counter) {
+  constexpr int NW = kRedThreads / 32;
+  __shared__ FxVal sw[NV][NW];
+  __shared__ bool am_last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = gridDim.x;
 #pragma unroll
-  for (int i = 0; i < kGsChunk; ++i)
-    v[i] = i < c ? reinterpret_cast<const float4*>(V[i0 + i]) : nullptr;
-  const float4* w4 = reinterpret_cast<const float4*>(w);
-  KahanAcc acc[kGsChunk];
+  for (int q = 0; q < NV; ++q) {
+    const FxVal f = fx_warp_sum(v[q]);
+    if (lane == 0) sw[q][warp] = f;
+  }
+  __syncthreads();
+  for (int q = warp; q < cnt; q += NW) {
+    const FxVal f = lane < NW ? sw[q][lane] : FxVal{0, 1};
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f.e);
+    FxAcc acc;
+    if (e < kFxBad) acc.add(f, e);
+    acc = fx_warp_add(acc);
+    if (lane == 0) {
+      __stcg(partials + q * nb + blockIdx.x, make_longlong2((acc.hi << 28) + (acc.lo >> 4), e + 4));
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    am_last = atomicInc(counter, (unsigned)nb - 1u) == (unsigned)nb - 1u;
+  }
+  __syncthreads();
+  if (!am_last) return;
+  __threadfence();
+  for (int q = warp; q < cnt; q += NW) {
+    unsigned e = 1u;
+    for (int l = lane; l < nb; l += 32) e = max(e, (unsigned)__ldcg(partials + q * nb + l).y);
+    e = __reduce_max_sync(0xffffffffu, e);
+    FxAcc acc;
+    if (e < kFxBad)
+      for (int l = lane; l < nb; l += 32) {
+        const longlong2 t = __ldcg(partials + q * nb + l);
+        acc.add(FxVal{t.x, (int)t.y}, (int)e);
+      }
+    acc = fx_warp_add(acc);
+    if (lane == 0) out[q] = fx_round(acc.hi, acc.lo, (int)e);
+  }
+}
+
+// out[i] = <V_i, w>, i < cnt (blockIdx.y: chunk of kGsChunk vectors); UPD: first
+// w -= sum_i c_i V_i, stored, and the dots are those of the new w (one reading
+// of V for the first pass's update and the second's dots; one chunk, cnt <= NV)
+template <int NV, bool UPD>
+__global__ void __launch_bounds__(kRedThreads, NV <= 8 ? 3 : 2)
+k_gsf_dots(int64_t n4, const float* const* __restrict__ V, int cnt, const double* __restrict__ c,
+           float* __restrict__ w, double* __restrict__ out, longlong2* __restrict__ partials,
+           unsigned* __restrict__ counters) {
+  const int i0 = blockIdx.y * NV;
+  const int m = min(NV, cnt - i0);
+  const float4* v[NV];
+  float cf[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    v[i] = i < m ? reinterpret_cast<const float4*>(V[i0 + i]) : nullptr;
+    cf[i] = UPD && i < m ? -(float)c[i0 + i] : 0.0f;
+  }
+  float4* w4 = reinterpret_cast<float4*>(w);
+  KahanAcc acc[NV];
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n4;
        q += (int64_t)gridDim.x * blockDim.x) {
-    const float4 wq = w4[q];
+    float4 wq = w4[q];
+    float4 a[NV];
 #pragma unroll
-    for (int i = 0; i < kGsChunk; ++i)
-      if (i < c) {
-        const float4 a = v[i][q];
-        acc[i].add(fmaf(a.x, wq.x, fmaf(a.y, wq.y, __fmul_rn(a.z, wq.z))) + a.w * wq.w);
-      }
+    for (int i = 0; i < NV; ++i)
+      if (i < m) a[i] = v[i][q];
+    if constexpr (UPD) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        if (i < m) {
+          wq.x = fmaf(cf[i], a[i].x, wq.x);
+          wq.y = fmaf(cf[i], a[i].y, wq.y);
+          wq.z = fmaf(cf[i], a[i].z, wq.z);
+          wq.w = fmaf(cf[i], a[i].w, wq.w);
+        }
+      w4[q] = wq;
+    }
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+      if (i < m)
+        acc[i].add(fmaf(a[i].x, wq.x, fmaf(a[i].y, wq.y, __fmul_rn(a[i].z, wq.z))) + a[i].w * wq.w);
   }
-  double tv[kGsChunk], tot[kGsChunk];
+  double tv[NV];
 #pragma unroll
-  for (int i = 0; i < kGsChunk; ++i) tv[i] = acc[i].value();
-  if (grid_sum<kGsChunk>(tv, partials + (size_t)blockIdx.y * kGsChunk * gridDim.x,
-                         counters + blockIdx.y, tot) &&
-      threadIdx.x == 0)
-    for (int i = 0; i < c; ++i) out[i0 + i] = tot[i];
+  for (int i = 0; i < NV; ++i) tv[i] = acc[i].value();
+  grid_sum_fx<NV>(tv, m, out + i0, partials + (size_t)blockIdx.y * NV * gridDim.x,
+                  counters + blockIdx.y);
 }
 
 // w -= sum_{i < cnt} c_i V_i (FP32); with out, also out[0] = <w, w>
 __global__ void __launch_bounds__(kRedThreads)
 k_gsf_update(int64_t n4, const float* const* __restrict__ V, int cnt, const double* __restrict__ c,
-             float* __restrict__ w, double* __restrict__ out, double* __restrict__ partials,
+             float* __restrict__ w, double* __restrict__ out, longlong2* __restrict__ partials,
              unsigned* __restrict__ counter) {
   __shared__ const float4* sv[kGsMax];
   __shared__ float sc[kGsMax];
@@ -256,8 +325,8 @@ k_gsf_update(int64_t n4, const float* const* __restrict__ V, int cnt, const doub
     if (out) acc.add(fmaf(wq.x, wq.x, fmaf(wq.y, wq.y, __fmul_rn(wq.z, wq.z))) + wq.w * wq.w);
   }
   if (out) {
-    double v[1] = {acc.value()}, tot[1];
-    if (grid_sum<1>(v, partials, counter, tot) && threadIdx.x == 0) out[0] = tot[0];
+    const double v[1] = {acc.value()};
+    grid_sum_fx<1>(v, 1, out, partials, counter);
   }
 }
 
@@ -295,7 +364,8 @@ struct GmresWorkF {
   std::vector<std::unique_ptr<DevBuf<float>>> V, Z;
   DevBuf<float> w, r, d;                   // scratch, the inner residual, the correction
   DevBuf<const float*> vptr, zptr;
-  DevBuf<double> coef, coef2, hcol, dots, partials;
+  DevBuf<double> coef, coef2, hcol, dots;
+  DevBuf<longlong2> partials;
   DevBuf<unsigned> counter;
   double* pin = nullptr;
   GmresWorkF(sem_handle* hh, int mm, cudaStream_t s) : h(hh), m(mm) {
@@ -537,15 +607,28 @@ void gmres_solve_mixed(sem_handle* h, const double* b, double* x, const sem_solv
                             s);
         const int cnt = j + 1;
         const dim3 dgrid(kRedBlocks, (cnt + kGsChunk - 1) / kGsChunk);
-        k_gsf_dots<<<dgrid, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.w.ptr, g.coef.ptr,
-                                                 g.partials.ptr, g.counter.ptr);
+        const dim3 dgrid3(3 * kRedBlocks / 4, dgrid.y);     // three blocks an SM, as they fit
+        k_gsf_dots<kGsChunk, false><<<dgrid3, kRedThreads, 0, s>>>(
+            n4, g.vptr.ptr, cnt, nullptr, g.w.ptr, g.coef.ptr, g.partials.ptr, g.counter.ptr);
         SEM_CHECK_LAUNCH();
-        k_gsf_update<<<kRedBlocks, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.coef.ptr, g.w.ptr,
-                                                        nullptr, nullptr, nullptr);
-        SEM_CHECK_LAUNCH();
-        k_gsf_dots<<<dgrid, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.w.ptr, g.coef2.ptr,
-                                                 g.partials.ptr, g.counter.ptr);
-        SEM_CHECK_LAUNCH();
+        if (cnt <= 8) {
+          k_gsf_dots<8, true><<<dgrid3.x, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.coef.ptr,
+                                                               g.w.ptr, g.coef2.ptr,
+                                                               g.partials.ptr, g.counter.ptr);
+          SEM_CHECK_LAUNCH();
+        } else if (cnt <= 12) {
+          k_gsf_dots<12, true><<<kRedBlocks / 2, kRedThreads, 0, s>>>(
+              n4, g.vptr.ptr, cnt, g.coef.ptr, g.w.ptr, g.coef2.ptr, g.partials.ptr,
+              g.counter.ptr);
+          SEM_CHECK_LAUNCH();
+        } else {
+          k_gsf_update<<<kRedBlocks, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.coef.ptr,
+                                                          g.w.ptr, nullptr, nullptr, nullptr);
+          SEM_CHECK_LAUNCH();
+          k_gsf_dots<kGsChunk, false><<<dgrid3, kRedThreads, 0, s>>>(
+              n4, g.vptr.ptr, cnt, nullptr, g.w.ptr, g.coef2.ptr, g.partials.ptr, g.counter.ptr);
+          SEM_CHECK_LAUNCH();
+        }
         k_gsf_update<<<kRedBlocks, kRedThreads, 0, s>>>(n4, g.vptr.ptr, cnt, g.coef2.ptr, g.w.ptr,
                                                         g.dots.ptr, g.partials.ptr,
                                                         g.counter.ptr + kGsMax / kGsChunk);

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "sem_internal.cuh"
+#include "grid_dots.cuh"
 #include "reduce.cuh"
 #include "tma.cuh"
 
@@ -35,7 +36,7 @@ namespace {
 template <int PE>
 struct SwCfg {
   static constexpr int THREADS = PE * PE <= 128 ? 128 : (PE * PE + 31) / 32 * 32;
-  static constexpr int MINB = PE * PE <= 128 ? 4 : 2;
+  static constexpr int MINB = PE * PE <= 128 ? 6 : 4;
 };
 constexpr int kNbr = 0, kDir = 1, kFree = 2;
 
@@ -137,7 +138,8 @@ template <int PE>
 struct SwLayout {
   static constexpr int R = (PE + 3) / 4 * 4;
   static constexpr int TAB = 2 * PE * R + R;         // one (d, v) table
-  static constexpr int ALL = 12 * TAB;
+  static constexpr int ALL = 12 * TAB;               // then 1 / (h1 (lx + ly + lz) + h2) of
+                                                     // the interior element, [c][b][a]
 };
 
 struct SwParams {
@@ -164,155 +166,195 @@ __device__ __forceinline__ float dot_row(const float* __restrict__ row, const fl
   return acc;
 }
 
-// One element at a time per CTA.  Thread (a, b) < PE^2 owns the z-column of
-// the grown box: it gathers the column, applies S^T along z in registers and
-// writes box[c][b][a] (rows padded to R); the x- and y-directions run as line
-// tasks through shared memory (S^T along x; along y S^T, the diagonal scaling
-// and S; S along x); the thread then reads its column back, applies S along
-// z in registers and adds the kept points to z.  Factors along different
-// directions commute, so this order gives the same A~^-1 as x, y, z first.
-// The coarse restriction is taken from the gathered columns of the element's
-// own points (a, b, c in 1 .. P).
+// S of the interior elements (kind 0) per direction, [a][a'], in the kernel
+// parameters: constant-bank operands of the line tasks
+template <int PE>
+struct SwConst {
+  float S[3][PE * PE];
+};
+
+// y = S^T x (TRANS) or S x along direction DIR; interior kinds from the constant
+// bank, the others from the table tb of SwLayout in shared memory
+template <int PE, int DIR, bool TRANS, class PUT>
+__device__ __forceinline__ void sw_line(const SwConst<PE>& k, bool interior, const float* tb,
+                                        const float (&x)[SwLayout<PE>::R], PUT put) {
+  constexpr int R = SwLayout<PE>::R;
+  if (interior) {
+#pragma unroll
+    for (int i = 0; i < PE; ++i) {
+      float y = (TRANS ? k.S[DIR][i] : k.S[DIR][i * PE]) * x[0];
+#pragma unroll
+      for (int l = 1; l < PE; ++l)
+        y = fmaf(TRANS ? k.S[DIR][l * PE + i] : k.S[DIR][i * PE + l], x[l], y);
+      put(i, y);
+    }
+  } else {
+    const float* t = tb + (TRANS ? 0 : PE * R);
+#pragma unroll
+    for (int i = 0; i < PE; ++i) put(i, dot_row<R>(t + i * R, x, PE));
+  }
+}
+
+// One element per CTA.  Thread (a, b) < PE^2 owns the z-column of the grown box:
+// it gathers the column, applies S^T along z in registers and writes
+// box[c][b][a] (rows padded to R, moved as 16-byte vectors); the x- and
+// y-directions run as line tasks through shared memory (S^T along x; along y
+// S^T, the diagonal scaling and S; S along x); the thread then reads its column
+// back, applies S along z in registers and adds the kept points to z.  Factors
+// along different directions commute, so this order gives the same A~^-1 as x,
+// y, z first.  The coarse restriction is taken from the gathered columns of the
+// element's own points (a, b, c in 1 .. P): z-weighted sums per column, then
+// the last warp, which has the fewest lines, adds them up.
+// The kernel is bound by issue and by the latency of its line phases: S as
+// constant operands (an interior direction reads no table: the persistent form
+// with all tables in shared memory spent three 16-byte reads on every output),
+// the interior scaling as a table of reciprocals, and one element a CTA, so
+// that tables that are not used are not loaded and the registers allow twice
+// the CTAs.  13,824 elements, N = 7: LOCALUS.
 template <int PE>
 __global__ void __launch_bounds__(SwCfg<PE>::THREADS, SwCfg<PE>::MINB)
 schwarz_local_kernel(const float* __restrict__ rg, float* __restrict__ zg,
-                     float* __restrict__ rc, const float* __restrict__ tab_g, SwParams prm,
-                     int E) {
+                     float* __restrict__ rc, const float* __restrict__ tab_g,
+                     const __grid_constant__ SwParams prm,
+                     const __grid_constant__ SwConst<PE> kst) {
   using L = SwLayout<PE>;
-  constexpr int R = L::R, P = PE - 2, N = PE - 3;
-  __shared__ __align__(16) float tab[L::ALL];
-  __shared__ __align__(16) float box[PE * PE * R];
-  constexpr int NW = SwCfg<PE>::THREADS / 32;
-  __shared__ float red[8][NW];
-  for (int q = threadIdx.x; q < L::ALL; q += blockDim.x) tab[q] = tab_g[q];
-  __syncthreads();
-  const int tid = threadIdx.x;
-  const bool owner = tid < PE * PE;
+  constexpr int R = L::R, P = PE - 2, N = PE - 3, T = SwCfg<PE>::THREADS, PE2 = PE * PE;
+  static_assert(PE2 <= T, "a line per thread");
+  __shared__ __align__(16) float tab[3][L::TAB];
+  __shared__ __align__(16) float box[PE2 * R];
+  __shared__ float cs[2][PE2];
+  const int tid = threadIdx.x, e = blockIdx.x;
+  const bool owner = tid < PE2;
   const int ca = tid % PE, cb = tid / PE;          // this thread's column (a, b)
-  for (int e = blockIdx.x; e < E; e += gridDim.x) {
-    const uint32_t r1 = prm.dnx.div((uint32_t)e);
-    const int ex = e - (int)r1 * prm.nelx;
-    const uint32_t q1 = prm.dny.div(r1);
-    const int ey = (int)(r1 - q1 * (uint32_t)prm.nely), ez = (int)q1;
-    const int vx = (ex == 0 ? 1 : 0) | (ex == prm.nelx - 1 ? 2 : 0);
-    const int vy = (ey == 0 ? 1 : 0) | (ey == prm.nely - 1 ? 2 : 0);
-    const int vz = (ez == 0 ? 1 : 0) | (ez == prm.nelz - 1 ? 2 : 0);
-    const unsigned kx = prm.keep[0][vx], ky = prm.keep[1][vy], kz = prm.keep[2][vz];
-    const float* tx = tab + (0 * 4 + vx) * L::TAB;
-    const float* ty = tab + (1 * 4 + vy) * L::TAB;
-    const float* tz = tab + (2 * 4 + vz) * L::TAB;
-    const bool colkeep = owner && ((kx >> ca) & 1u) && ((ky >> cb) & 1u);
-    // lattice index of (a, b, 0) of this thread's column
-    const long long cbase = (long long)(N * ex - 1 + ca) + (long long)prm.gx * (N * ey - 1 + cb) +
-                            prm.sk * (long long)(N * ez - 1);
-    float col[R];
+  const uint32_t r1 = prm.dnx.div((uint32_t)e);
+  const int ex = e - (int)r1 * prm.nelx;
+  const uint32_t q1 = prm.dny.div(r1);
+  const int ey = (int)(r1 - q1 * (uint32_t)prm.nely), ez = (int)q1;
+  const int vk[3] = {(ex == 0 ? 1 : 0) | (ex == prm.nelx - 1 ? 2 : 0),
+                     (ey == 0 ? 1 : 0) | (ey == prm.nely - 1 ? 2 : 0),
+                     (ez == 0 ? 1 : 0) | (ez == prm.nelz - 1 ? 2 : 0)};
+  const unsigned kx = prm.keep[0][vk[0]], ky = prm.keep[1][vk[1]], kz = prm.keep[2][vk[2]];
+  const bool colkeep = owner && ((kx >> ca) & 1u) && ((ky >> cb) & 1u);
+  // lattice index of (a, b, 0) of this thread's column
+  const long long cbase = (long long)(N * ex - 1 + ca) + (long long)prm.gx * (N * ey - 1 + cb) +
+                          prm.sk * (long long)(N * ez - 1);
+  float col[R];
 #pragma unroll
-    for (int c = 0; c < R; ++c)
-      col[c] = (c < PE && colkeep && ((kz >> c) & 1u)) ? rg[cbase + prm.sk * c] : 0.0f;
-    if (prm.do_coarse) {
-      // restriction: sum over own points of phi_v r / mult
-      float acc[8];
+  for (int c = 0; c < R; ++c)
+    col[c] = (c < PE && colkeep && ((kz >> c) & 1u)) ? __ldg(rg + cbase + prm.sk * c) : 0.0f;
+  // the tables of the directions that are not interior; the eigenvalues unless
+  // the whole element is interior (then the reciprocals serve)
+  const bool inner = (vk[0] | vk[1] | vk[2]) == 0;
+  if (!inner) {
 #pragma unroll
-      for (int v = 0; v < 8; ++v) acc[v] = 0.0f;
-      if (owner && ca >= 1 && ca <= P && cb >= 1 && cb <= P) {
-        const int i = ca - 1, j = cb - 1;
-        const float mij = ((i == 0 && ex > 0) || (i == N && ex < prm.nelx - 1) ? 0.5f : 1.0f) *
-                          ((j == 0 && ey > 0) || (j == N && ey < prm.nely - 1) ? 0.5f : 1.0f);
-        float s0 = 0.0f, s1 = 0.0f;
+    for (int d = 0; d < 3; ++d) {
+      const float* src = tab_g + (d * 4 + vk[d]) * L::TAB;
+      for (int q = tid + (vk[d] ? 0 : 2 * PE * R); q < L::TAB; q += T) tab[d][q] = __ldg(src + q);
+    }
+  }
+  if (prm.do_coarse && owner) {
+    float s0 = 0.0f, s1 = 0.0f;
+    if (ca >= 1 && ca <= P && cb >= 1 && cb <= P) {
+      const int i = ca - 1, j = cb - 1;
+      const float mij = ((i == 0 && ex > 0) || (i == N && ex < prm.nelx - 1) ? 0.5f : 1.0f) *
+                        ((j == 0 && ey > 0) || (j == N && ey < prm.nely - 1) ? 0.5f : 1.0f);
 #pragma unroll
-        for (int k = 0; k < P; ++k) {
-          const float mk = (k == 0 && ez > 0) || (k == N && ez < prm.nelz - 1) ? 0.5f : 1.0f;
-          const float rv = mk * col[k + 1];
-          s0 = fmaf(prm.phi[0][k], rv, s0);
-          s1 = fmaf(prm.phi[1][k], rv, s1);
-        }
-#pragma unroll
-        for (int v = 0; v < 8; ++v)
-          acc[v] = mij * prm.phi[v & 1][i] * prm.phi[(v >> 1) & 1][j] * ((v >> 2) ? s1 : s0);
+      for (int k = 0; k < P; ++k) {
+        const float mk = (k == 0 && ez > 0) || (k == N && ez < prm.nelz - 1) ? 0.5f : 1.0f;
+        const float rv = mk * col[k + 1];
+        s0 = fmaf(prm.phi[0][k], rv, s0);
+        s1 = fmaf(prm.phi[1][k], rv, s1);
       }
+      s0 *= mij;
+      s1 *= mij;
+    }
+    cs[0][tid] = s0;
+    cs[1][tid] = s1;
+  }
+  __syncthreads();
+  if (prm.do_local && owner)               // S^T along z in registers, to the box
+    sw_line<PE, 2, true>(kst, vk[2] == 0, tab[2], col,
+                         [&](int c, float y) { box[(c * PE + cb) * R + ca] = y; });
+  if (prm.do_coarse && tid >= T - 32) {    // the eight vertex sums of this element
+    const int lane = tid & 31;
+    float acc[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) acc[v] = 0.0f;
+    for (int q = lane; q < P * P; q += 32) {
+      const int i = q % P, j = q / P, at = (j + 1) * PE + i + 1;
+      const float s0 = cs[0][at], s1 = cs[1][at];
 #pragma unroll
       for (int v = 0; v < 8; ++v)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[v] += __shfl_down_sync(0xffffffffu, acc[v], o);
-      if ((tid & 31) == 0)
-#pragma unroll
-        for (int v = 0; v < 8; ++v) red[v][tid >> 5] = acc[v];
-      __syncthreads();
-      if (tid < 8) {
-        float t = 0.0f;
-        for (int w = 0; w < NW; ++w) t += red[tid][w];
-        const int v = tid;
-        const long long vi = (long long)(ex + (v & 1)) +
-                             (long long)(prm.nelx + 1) *
-                                 ((ey + ((v >> 1) & 1)) + (long long)(prm.nely + 1) * (ez + (v >> 2)));
-        red_add(rc + vi, t);
-      }
+        acc[v] = fmaf(prm.phi[v & 1][i] * prm.phi[(v >> 1) & 1][j], (v >> 2) ? s1 : s0, acc[v]);
     }
-    if (prm.do_local) {
-      // S^T along z in registers, to the box
-      if (owner) {
-#pragma unroll 2
-        for (int c = 0; c < PE; ++c) box[(c * PE + cb) * R + ca] = dot_row<R>(tz + c * R, col, PE);
-      }
-      __syncthreads();
-      // S^T along x on lines (b, c)
-      for (int ln = tid; ln < PE * PE; ln += blockDim.x) {
-        float* row = box + ln * R;
-        float x[R];
 #pragma unroll
-        for (int a = 0; a < R; a += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(row + a);
-          x[a] = v.x; x[a + 1] = v.y; x[a + 2] = v.z; x[a + 3] = v.w;
-        }
-#pragma unroll 2
-        for (int a = 0; a < PE; ++a) row[a] = dot_row<R>(tx + a * R, x, PE);
-      }
-      __syncthreads();
-      // along y on lines (a, c): S^T, the diagonal scaling, S
-      for (int ln = tid; ln < PE * PE; ln += blockDim.x) {
-        const int a = ln % PE, c = ln / PE;
-        float* yl = box + c * PE * R + a;
-        float x[R];
+    for (int v = 0; v < 8; ++v)
 #pragma unroll
-        for (int b = 0; b < R; ++b) x[b] = b < PE ? yl[b * R] : 0.0f;
-        const float lac = tx[2 * PE * R + a] + tz[2 * PE * R + c];
-        float t[R];
+      for (int o = 16; o > 0; o >>= 1) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+    float mine = acc[0];
 #pragma unroll
-        for (int b = 0; b < R; ++b) {
-          if (b < PE) {
-            const float d = prm.h1 * (lac + ty[2 * PE * R + b]) + prm.h2;
-            t[b] = dot_row<R>(ty + b * R, x, PE) / d;
-          } else {
-            t[b] = 0.0f;
-          }
-        }
-#pragma unroll 2
-        for (int b = 0; b < PE; ++b) yl[b * R] = dot_row<R>(ty + PE * R + b * R, t, PE);
-      }
-      __syncthreads();
-      // S along x
-      for (int ln = tid; ln < PE * PE; ln += blockDim.x) {
-        float* row = box + ln * R;
-        float x[R];
-#pragma unroll
-        for (int a = 0; a < R; a += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(row + a);
-          x[a] = v.x; x[a + 1] = v.y; x[a + 2] = v.z; x[a + 3] = v.w;
-        }
-#pragma unroll 2
-        for (int a = 0; a < PE; ++a) row[a] = dot_row<R>(tx + PE * R + a * R, x, PE);
-      }
-      __syncthreads();
-      // S along z in registers, add the kept points
-      if (colkeep) {
-#pragma unroll
-        for (int c = 0; c < R; ++c) col[c] = c < PE ? box[(c * PE + cb) * R + ca] : 0.0f;
-#pragma unroll 2
-        for (int c = 0; c < PE; ++c)
-          if ((kz >> c) & 1u) red_add(zg + cbase + prm.sk * c, dot_row<R>(tz + PE * R + c * R, col, PE));
-      }
+    for (int v = 1; v < 8; ++v) mine = lane == v ? acc[v] : mine;
+    if (lane < 8) {
+      const long long vi = (long long)(ex + (lane & 1)) +
+                           (long long)(prm.nelx + 1) *
+                               ((ey + ((lane >> 1) & 1)) + (long long)(prm.nely + 1) * (ez + (lane >> 2)));
+      red_add(rc + vi, mine);
     }
-    __syncthreads();                         // box and red are reused by the next element
+  }
+  if (!prm.do_local) return;
+  __syncthreads();
+  float x[R], y[R];
+  float4* row = reinterpret_cast<float4*>(box + tid * R);
+  auto row_in = [&]() {
+#pragma unroll
+    for (int a = 0; a < R; a += 4) {
+      const float4 v = row[a / 4];
+      x[a] = v.x; x[a + 1] = v.y; x[a + 2] = v.z; x[a + 3] = v.w;
+    }
+  };
+  auto row_out = [&]() {
+#pragma unroll
+    for (int a = 0; a < R; a += 4) row[a / 4] = make_float4(y[a], y[a + 1], y[a + 2], y[a + 3]);
+  };
+#pragma unroll
+  for (int a = 0; a < R; ++a) y[a] = 0.0f;
+  if (owner) {                             // S^T along x on line (b, c)
+    row_in();
+    sw_line<PE, 0, true>(kst, vk[0] == 0, tab[0], x, [&](int a, float v) { y[a] = v; });
+    row_out();
+  }
+  __syncthreads();
+  if (owner) {                             // along y on line (a, c): S^T, scaling, S
+    float* yl = box + cb * PE * R + ca;    // (a, c) = (tid % PE, tid / PE)
+#pragma unroll
+    for (int b = 0; b < R; ++b) x[b] = b < PE ? yl[b * R] : 0.0f;
+    sw_line<PE, 1, true>(kst, vk[1] == 0, tab[1], x, [&](int b, float v) { y[b] = v; });
+    if (inner) {
+      const float* inv = tab_g + L::ALL + cb * PE2 + ca;     // 1 / (h1 (lx + ly + lz) + h2)
+#pragma unroll
+      for (int b = 0; b < PE; ++b) y[b] *= __ldg(inv + b * PE);
+    } else {
+      const float lac = tab[0][2 * PE * R + ca] + tab[2][2 * PE * R + cb];
+#pragma unroll
+      for (int b = 0; b < PE; ++b) y[b] /= prm.h1 * (lac + tab[1][2 * PE * R + b]) + prm.h2;
+    }
+    sw_line<PE, 1, false>(kst, vk[1] == 0, tab[1], y, [&](int b, float v) { yl[b * R] = v; });
+  }
+  __syncthreads();
+  if (owner) {                             // S along x
+    row_in();
+#pragma unroll
+    for (int a = 0; a < R; ++a) y[a] = 0.0f;
+    sw_line<PE, 0, false>(kst, vk[0] == 0, tab[0], x, [&](int a, float v) { y[a] = v; });
+    row_out();
+  }
+  __syncthreads();
+  if (colkeep) {                           // S along z in registers, add the kept points
+#pragma unroll
+    for (int c = 0; c < R; ++c) x[c] = c < PE ? box[(c * PE + cb) * R + ca] : 0.0f;
+    sw_line<PE, 2, false>(kst, vk[2] == 0, tab[2], x, [&](int c, float v) {
+      if ((kz >> c) & 1u) red_add(zg + cbase + prm.sk * c, v);
+    });
   }
 }
 
@@ -344,6 +386,138 @@ __global__ void k_coarse_matvec(int E, const float* __restrict__ K, const float*
       red_add(w + vi[r], acc);
     }
   }
+}
+
+// ------------------------------------------------------------------ coarse CG in one launch
+// A_0 as a 27-point stencil on the vertices: st[o][v] = sum of the entries of
+// the elements that hold both v and its neighbour o (dx, dy, dz in {-1, 0, 1},
+// o = (dx + 1) + 3 (dy + 1) + 9 (dz + 1)); neighbours outside the box get 0.
+__global__ void k_coarse_stencil(int nelx, int nely, int nelz, const float* __restrict__ K,
+                                 float* __restrict__ st, int nv) {
+  const int nvx = nelx + 1, nvy = nely + 1;
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
+    const int x = v % nvx, y = (v / nvx) % nvy, z = v / (nvx * nvy);
+    for (int o = 0; o < 27; ++o) {
+      const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+      double acc = 0.0;
+      for (int c = 0; c < 8; ++c) {            // v is corner c of the element at (ex, ey, ez)
+        const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
+        const int ex = x - cx, ey = y - cy, ez = z - cz;
+        const int bx = cx + dx, by = cy + dy, bz = cz + dz;   // the neighbour's corner
+        if (ex < 0 || ex >= nelx || ey < 0 || ey >= nely || ez < 0 || ez >= nelz) continue;
+        if (bx < 0 || bx > 1 || by < 0 || by > 1 || bz < 0 || bz > 1) continue;
+        const int b = bx + 2 * by + 4 * bz;
+        const size_t e = (size_t)ex + (size_t)nelx * (ey + (size_t)nely * ez);
+        acc += (double)K[e * 36 + (c <= b ? pk(c, b) : pk(b, c))];
+      }
+      st[(size_t)o * nv + v] = (float)acc;
+    }
+  }
+}
+
+constexpr int kCoarseThreads = 256;
+constexpr int kCoarseBlocks = 608;   // the most CTAs (their sums fit the shared memory)
+
+struct CoarseArgs {
+  const float *st, *dinv, *r;       // stencil, Jacobi inverse (0: masked), right-hand side
+  float *x, *p0, *p1, *z;           // solution; directions (two buffers), residual scaled
+  longlong2* partials;              // 2 gridDim.x values, taken in turn
+  unsigned* bar;                    // zero at launch
+  int* err;
+  uint64_t timeout_ns;
+  int nvx, nvy, nvz, iters;
+};
+
+// iters Jacobi-CG iterations from zero, a thread per vertex with its stencil
+// row, x, r and dinv in registers (a cooperative launch; two grid barriers an
+// iteration).  A thread forms its neighbours' p = z + beta p_old itself, so that
+// the barrier that gives beta needs none after it.  Ten iterations on 25^3
+// vertices took 240 us as 40 launches of a few microseconds each.
+__global__ void __launch_bounds__(kCoarseThreads)
+k_coarse_cg(const __grid_constant__ CoarseArgs a) {
+  constexpr int NW = kCoarseThreads / 32;
+  extern __shared__ longlong2 sp[];
+  __shared__ FxVal s_w[2][16];
+  __shared__ double s_tot[2], s_rz;
+  __shared__ float s_alpha, s_beta;
+  __shared__ int s_bad, s_stop;
+  const int nv = a.nvx * a.nvy * a.nvz;
+  const int v = blockIdx.x * kCoarseThreads + threadIdx.x;
+  const bool act = v < nv;
+  const int x0 = act ? v % a.nvx : 0, y0 = act ? (v / a.nvx) % a.nvy : 0,
+            z0 = act ? v / (a.nvx * a.nvy) : 0;
+  float c[27];
+#pragma unroll
+  for (int o = 0; o < 27; ++o) c[o] = act ? __ldg(a.st + (size_t)o * nv + v) : 0.0f;
+  const float d = act ? a.dinv[v] : 0.0f;
+  float r = act ? a.r[v] : 0.0f, x = 0.0f, z = d * r, p = 0.0f;
+  if (act) {
+    __stcg(a.z + v, z);
+    __stcg(a.p0 + v, 0.0f);
+  }
+  if (threadIdx.x == 0) {
+    s_bad = 0;
+    s_stop = 0;
+  }
+  unsigned met = 0;
+  float *pold = a.p0, *pnew = a.p1;
+  {
+    const double v0[1] = {(double)r * (double)z};
+    met += gridDim.x;
+    if (!grid_dots<1, NW>(v0, s_w, sp, s_tot, a.partials + gridDim.x, a.bar, met, a.err, a.timeout_ns, &s_bad,
+                          [&] {
+                            s_rz = s_tot[0];
+                            s_beta = 0.0f;
+                            s_stop = dbits(s_tot[0]) <= 0 || is_nan(s_tot[0]);
+                          }))
+      return;
+  }
+  for (int it = 0; it < a.iters && !s_stop; ++it) {
+    const float beta = s_beta;
+    float w = 0.0f;
+    p = fmaf(beta, p, z);
+    if (act) {
+      __stcg(pnew + v, p);
+#pragma unroll
+      for (int o = 0; o < 27; ++o) {
+        const int dx = o % 3 - 1, dy = (o / 3) % 3 - 1, dz = o / 9 - 1;
+        if (o == 13) {
+          w = fmaf(c[13], p, w);
+        } else if (x0 + dx >= 0 && x0 + dx < a.nvx && y0 + dy >= 0 && y0 + dy < a.nvy &&
+                   z0 + dz >= 0 && z0 + dz < a.nvz) {
+          const int n = v + dx + a.nvx * (dy + a.nvy * dz);
+          w = fmaf(c[o], fmaf(beta, __ldcg(pold + n), __ldcg(a.z + n)), w);
+        }
+      }
+    }
+    const double v1[1] = {(double)p * (double)w};
+    met += gridDim.x;
+    if (!grid_dots<1, NW>(v1, s_w, sp, s_tot, a.partials, a.bar, met, a.err, a.timeout_ns, &s_bad,
+                          [&] {
+                            s_stop = dbits(s_tot[0]) <= 0 || is_nan(s_tot[0]);
+                            s_alpha = s_stop ? 0.0f : (float)(s_rz / s_tot[0]);
+                          }))
+      return;
+    if (s_stop) break;
+    x = fmaf(s_alpha, p, x);
+    r = fmaf(-s_alpha, w, r);
+    z = d * r;
+    if (it + 1 == a.iters) break;            // the last direction has been taken
+    if (act) __stcg(a.z + v, z);
+    const double v2[1] = {(double)r * (double)z};
+    met += gridDim.x;
+    if (!grid_dots<1, NW>(v2, s_w, sp, s_tot, a.partials + gridDim.x, a.bar, met, a.err,
+                          a.timeout_ns, &s_bad, [&] {
+                            s_stop = dbits(s_tot[0]) <= 0 || is_nan(s_tot[0]);
+                            s_beta = s_stop ? 0.0f : (float)(s_tot[0] / s_rz);
+                            s_rz = s_tot[0];
+                          }))
+      return;
+    float* t = pold;
+    pold = pnew;
+    pnew = t;
+  }
+  if (act) a.x[v] = x;
 }
 
 // L-vector of vertex function v (all elements), FP64
@@ -484,8 +658,14 @@ struct sem_schwarz {
   int Pe = 0;
   SwParams prm{};
   DevBuf<float> tab;                       // FDM tables
+  std::vector<float> tab_h;                // the same on the host
   int64_t nv = 0, nv4 = 0;                 // coarse vertices, padded
   DevBuf<float> K, cdinv, rc, xc, pc, wc;
+  // the one-launch coarse CG (where the vertices fit the resident grid): A_0 as a
+  // stencil, scaled residual, reduction partials, barrier
+  DevBuf<float> stencil, zc;
+  DevBuf<double> cpart;
+  DevBuf<unsigned> cbar;
   DevBuf<float> rg, zg;                    // fine global vectors
   DevBuf<CGState> st;
   DevBuf<double> partials;
@@ -496,16 +676,14 @@ namespace {
 
 template <int PE>
 void launch_local(sem_schwarz* sw, const float* rg, float* zg, cudaStream_t s) {
-  const sem_handle* h = sw->h;
-  auto kern = schwarz_local_kernel<PE>;
-  constexpr int T = SwCfg<PE>::THREADS;
-  static int occ = 0;
-  if (!occ) {
-    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, T, 0));
-    if (occ < 1) occ = 1;
-  }
-  const int grid = (int)std::min<int64_t>(h->E, (int64_t)occ * sem_num_sms());
-  kern<<<grid, T, 0, s>>>(rg, zg, sw->rc.ptr, sw->tab.ptr, sw->prm, (int)h->E);
+  using L = SwLayout<PE>;
+  SwConst<PE> k;
+  for (int d = 0; d < 3; ++d)
+    for (int a = 0; a < PE; ++a)
+      for (int b = 0; b < PE; ++b)
+        k.S[d][a * PE + b] = sw->tab_h[(d * 4) * L::TAB + PE * L::R + a * L::R + b];
+  schwarz_local_kernel<PE><<<(unsigned)sw->h->E, SwCfg<PE>::THREADS, 0, s>>>(
+      rg, zg, sw->rc.ptr, sw->tab.ptr, sw->prm, k);
   SEM_CHECK_LAUNCH();
 }
 
@@ -564,7 +742,15 @@ void build_tables(sem_schwarz* sw, std::vector<float>& out) {
       for (int a = 0; a < Pe; ++a) t[2 * Pe * R + a] = (float)lam[a];
     }
   }
+  auto lam0 = [&](int d, int a) { return out[d * 4 * TAB + 2 * Pe * R + a]; };
+  const float h1 = sw->prm.h1, h2 = sw->prm.h2;
+  for (int c = 0; c < Pe; ++c)
+    for (int b = 0; b < Pe; ++b)
+      for (int a = 0; a < Pe; ++a)
+        out.push_back(1.0f / (h1 * (lam0(0, a) + lam0(2, c) + lam0(1, b)) + h2));
 }
+
+int64_t coarse_cg_threads();
 
 // coarse element matrices from the FP64 element operator
 void build_coarse(sem_schwarz* sw, cudaStream_t s) {
@@ -594,6 +780,15 @@ void build_coarse(sem_schwarz* sw, cudaStream_t s) {
   k_coarse_dinv<<<ew_blocks(sw->nv), 256, 0, s>>>((int)E, dg.ptr, sw->cdinv.ptr, acc.ptr,
                                                  h->nelx, h->nely, h->nelz, h->faces, 1);
   SEM_CHECK_LAUNCH();
+  if (sw->nv <= coarse_cg_threads()) {
+    sw->stencil.alloc((size_t)sw->nv * 27);
+    sw->zc.alloc(sw->nv);
+    sw->cpart.alloc(2 * 2 * kCoarseBlocks);
+    sw->cbar.alloc(1);
+    k_coarse_stencil<<<ew_blocks(sw->nv), 256, 0, s>>>(h->nelx, h->nely, h->nelz, sw->K.ptr,
+                                                       sw->stencil.ptr, (int)sw->nv);
+    SEM_CHECK_LAUNCH();
+  }
   SEM_CUDA(cudaStreamSynchronize(s));      // the scratch buffers are freed on return
 }
 
@@ -603,6 +798,43 @@ sem_handle* schwarz_handle(const sem_schwarz* sw) { return sw->h; }
 
 namespace {
 
+// threads a grid of resident CTAs of the one-launch coarse CG has
+int64_t coarse_cg_threads() {
+  static int occ = 0;
+  if (!occ) {
+    const int smem = kCoarseBlocks * (int)sizeof(longlong2);
+    int o = 0;
+    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_coarse_cg, kCoarseThreads, smem));
+    occ = std::max(1, o);
+  }
+  return (int64_t)std::min(kCoarseBlocks, occ * sem_num_sms()) * kCoarseThreads;
+}
+
+void launch_coarse_cg(sem_schwarz* sw, cudaStream_t s) {
+  const sem_handle* h = sw->h;
+  CoarseArgs a{};
+  a.st = sw->stencil.ptr;
+  a.dinv = sw->cdinv.ptr;
+  a.r = sw->rc.ptr;
+  a.x = sw->xc.ptr;
+  a.p0 = sw->pc.ptr;
+  a.p1 = sw->wc.ptr;
+  a.z = sw->zc.ptr;
+  a.partials = reinterpret_cast<longlong2*>(sw->cpart.ptr);
+  a.bar = sw->cbar.ptr;
+  a.err = h->dev_err.ptr;
+  a.timeout_ns = kWaitTimeoutNs;
+  a.nvx = h->nelx + 1;
+  a.nvy = h->nely + 1;
+  a.nvz = h->nelz + 1;
+  a.iters = sw->coarse_iters;
+  SEM_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
+  const int grid = (int)((sw->nv + kCoarseThreads - 1) / kCoarseThreads);
+  void* args[] = {&a};
+  SEM_CUDA(cudaLaunchCooperativeKernel(k_coarse_cg, dim3(grid), dim3(kCoarseThreads), args,
+                                       grid * sizeof(longlong2), s));
+}
+
 // the local solves of rg added into zg (zeroed here), the coarse restriction
 // and the coarse CG; returns the coarse solution or NULL (no coarse level)
 const float* schwarz_levels(sem_schwarz* sw, const float* rg, float* zg, cudaStream_t s) {
@@ -611,7 +843,9 @@ const float* schwarz_levels(sem_schwarz* sw, const float* rg, float* zg, cudaStr
   const bool coarse = (sw->levels & SEM_SCHWARZ_COARSE) != 0;
   if (coarse) SEM_CUDA(cudaMemsetAsync(sw->rc.ptr, 0, sw->nv4 * 4 * sizeof(float), s));
   launch_local_any(sw, rg, zg, s);
-  if (coarse) {
+  if (coarse && sw->stencil.ptr) {
+    launch_coarse_cg(sw, s);
+  } else if (coarse) {
     CGState* st = sw->st.ptr;
     vcg_init(sw->nv4, sw->rc.ptr, sw->cdinv.ptr, sw->pc.ptr, sw->xc.ptr, sw->wc.ptr, st,
              sw->partials.ptr, 0.0, sw->coarse_iters, s);
@@ -628,43 +862,73 @@ const float* schwarz_levels(sem_schwarz* sw, const float* rg, float* zg, cudaStr
   return coarse ? sw->xc.ptr : nullptr;
 }
 
-// z_g = mask o (z_g + R_0^T c) at every global point, c read in the element
-// that holds the point at (i, j, k) with i, j, k < N where possible
-__global__ void k_sw_combine_global(int64_t nG, float* __restrict__ z, const float* __restrict__ xc,
-                                    SwParams prm, int faces, FastDiv dgx, FastDiv dgy,
-                                    FastDiv dN) {
-  const int N = prm.N;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < nG;
-       g += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t r = dgx.div((uint32_t)g);
-    const int ix = (int)((uint32_t)g - r * dgx.d);
-    const uint32_t izu = dgy.div(r);
-    const int iy = (int)(r - izu * dgy.d), iz = (int)izu;
-    const bool masked = ((faces & SEM_FACE_XMIN) && ix == 0) ||
-                        ((faces & SEM_FACE_XMAX) && ix == prm.gx - 1) ||
-                        ((faces & SEM_FACE_YMIN) && iy == 0) ||
-                        ((faces & SEM_FACE_YMAX) && iy == prm.gy - 1) ||
-                        ((faces & SEM_FACE_ZMIN) && iz == 0) ||
-                        ((faces & SEM_FACE_ZMAX) && iz == N * prm.nelz);
-    if (masked) {
-      z[g] = 0.0f;
-      continue;
+// z_g = mask o (z_g + R_0^T c) at every global point.  A warp takes a row (iy,
+// iz) of the lattice: its lanes blend the four coarse lines around the row with
+// the y- and z-weights into shared memory, then the row's points take two
+// entries each.  (A thread per point spent 33 us on 4.8 M points on index
+// arithmetic and the eight coarse values; the bytes take 6 us.)
+constexpr int kCombineWarps = 8;
+
+__global__ void __launch_bounds__(32 * kCombineWarps, 6)
+k_sw_combine_global(float* __restrict__ z, const float* __restrict__ xc,
+                    const __grid_constant__ SwParams prm, int faces, int rows, int gy, FastDiv dgy,
+                    FastDiv dN, int use_line) {
+  extern __shared__ float s_line[];
+  constexpr int Q = 4;                     // points a lane has on their way
+  const int N = prm.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nvx = prm.nelx + 1;
+  float* line = s_line + warp * nvx;
+  __shared__ float s_phi[2][kMaxP];
+  if (threadIdx.x < 2 * kMaxP)
+    s_phi[threadIdx.x / kMaxP][threadIdx.x % kMaxP] =
+        prm.phi[threadIdx.x / kMaxP][threadIdx.x % kMaxP];
+  __syncthreads();
+  const int row = blockIdx.x * kCombineWarps + warp;
+  if (row >= rows) return;
+  const int iz = (int)dgy.div((uint32_t)row), iy = row - iz * gy;
+  float* zr = z + (long long)row * prm.gx;
+  const bool masked = ((faces & SEM_FACE_YMIN) && iy == 0) ||
+                      ((faces & SEM_FACE_YMAX) && iy == N * prm.nely) ||
+                      ((faces & SEM_FACE_ZMIN) && iz == 0) ||
+                      ((faces & SEM_FACE_ZMAX) && iz == N * prm.nelz);
+  if (masked) {
+    for (int ix = lane; ix < prm.gx; ix += 32) zr[ix] = 0.0f;
+    return;
+  }
+  float t[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) t[q] = lane + 32 * q < prm.gx ? zr[lane + 32 * q] : 0.0f;
+  const int ey = min((int)dN.div((uint32_t)iy), prm.nely - 1);
+  const int ez = min((int)dN.div((uint32_t)iz), prm.nelz - 1);
+  const int sy = nvx, sz = nvx * (prm.nely + 1);
+  const float* c0 = xc + (ey * sy + ez * sz);
+  const float fy0 = s_phi[0][iy - ey * N], fy1 = s_phi[1][iy - ey * N];
+  const float fz0 = s_phi[0][iz - ez * N], fz1 = s_phi[1][iz - ez * N];
+  auto blend = [&](int v) {
+    return fmaf(fz1, fmaf(fy1, c0[v + sz + sy], fy0 * c0[v + sz]),
+                fz0 * fmaf(fy1, c0[v + sy], fy0 * c0[v]));
+  };
+  if (xc && use_line) {
+    for (int v = lane; v < nvx; v += 32) line[v] = blend(v);
+    __syncwarp();
+  }
+  const int last = prm.gx - 1;
+  const bool m0 = (faces & SEM_FACE_XMIN) != 0, m1 = (faces & SEM_FACE_XMAX) != 0;
+  for (int i0 = lane; i0 < prm.gx; i0 += 32 * Q) {
+    if (i0 != lane)
+#pragma unroll
+      for (int q = 0; q < Q; ++q) t[q] = i0 + 32 * q < prm.gx ? zr[i0 + 32 * q] : 0.0f;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int ix = i0 + 32 * q;
+      if (ix >= prm.gx) break;
+      float v = t[q];
+      if (xc) {
+        const int ex = min((int)dN.div((uint32_t)ix), prm.nelx - 1), i = ix - ex * N;
+        const float c1 = use_line ? line[ex + 1] : blend(ex + 1), cl = use_line ? line[ex] : blend(ex);
+        v += fmaf(s_phi[1][i], c1, s_phi[0][i] * cl);
+      }
+      zr[ix] = (m0 && ix == 0) || (m1 && ix == last) ? 0.0f : v;
     }
-    if (!xc) continue;
-    const int ex = min((int)dN.div((uint32_t)ix), prm.nelx - 1);
-    const int ey = min((int)dN.div((uint32_t)iy), prm.nely - 1);
-    const int ez = min((int)dN.div((uint32_t)iz), prm.nelz - 1);
-    const int i = ix - ex * N, j = iy - ey * N, k = iz - ez * N;
-    const int v0 = ex + (prm.nelx + 1) * (ey + (prm.nely + 1) * ez);
-    const int sy = prm.nelx + 1, sz = (prm.nelx + 1) * (prm.nely + 1);
-    const float fx0 = prm.phi[0][i], fx1 = prm.phi[1][i];
-    const float fy0 = prm.phi[0][j], fy1 = prm.phi[1][j];
-    const float fz0 = prm.phi[0][k], fz1 = prm.phi[1][k];
-    const float c00 = fmaf(fx1, xc[v0 + 1], fx0 * xc[v0]);
-    const float c10 = fmaf(fx1, xc[v0 + sy + 1], fx0 * xc[v0 + sy]);
-    const float c01 = fmaf(fx1, xc[v0 + sz + 1], fx0 * xc[v0 + sz]);
-    const float c11 = fmaf(fx1, xc[v0 + sz + sy + 1], fx0 * xc[v0 + sz + sy]);
-    z[g] += fmaf(fz1, fmaf(fy1, c11, fy0 * c01), fz0 * fmaf(fy1, c10, fy0 * c00));
   }
 }
 
@@ -673,9 +937,14 @@ __global__ void k_sw_combine_global(int64_t nG, float* __restrict__ z, const flo
 void schwarz_apply_global(sem_schwarz* sw, const float* r_g, float* z_g, cudaStream_t s) {
   sem_handle* h = sw->h;
   const float* xcp = schwarz_levels(sw, r_g, z_g, s);
-  k_sw_combine_global<<<ew_blocks(h->nG), 256, 0, s>>>(
-      h->nG, z_g, xcp, sw->prm, h->faces, FastDiv((uint32_t)(h->N * h->nelx + 1)),
-      FastDiv((uint32_t)(h->N * h->nely + 1)), FastDiv((uint32_t)h->N));
+  const int gy = h->N * h->nely + 1, rows = gy * (h->N * h->nelz + 1);
+  const int blocks = (rows + kCombineWarps - 1) / kCombineWarps;
+  size_t smem = (size_t)kCombineWarps * (h->nelx + 1) * sizeof(float);
+  const int use_line = smem <= 32 * 1024 ? 1 : 0;      // over 1000 elements along x: no lines
+  if (!use_line) smem = 0;
+  k_sw_combine_global<<<blocks, 32 * kCombineWarps, smem, s>>>(
+      z_g, xcp, sw->prm, h->faces, rows, gy, FastDiv((uint32_t)gy), FastDiv((uint32_t)h->N),
+      use_line);
   SEM_CHECK_LAUNCH();
 }
 
@@ -736,10 +1005,9 @@ extern "C" sem_status sem_schwarz_create(sem_handle* h, double h1, double h2, in
       p.phi[0][i] = (float)(0.5 * (1.0 - h->xi[i]));
       p.phi[1][i] = (float)(0.5 * (1.0 + h->xi[i]));
     }
-    std::vector<float> t;
-    build_tables(sw.get(), t);
-    sw->tab.alloc(t.size());
-    sw->tab.upload(t.data(), t.size(), s);
+    build_tables(sw.get(), sw->tab_h);
+    sw->tab.alloc(sw->tab_h.size());
+    sw->tab.upload(sw->tab_h.data(), sw->tab_h.size(), s);
     sw->rg.alloc(h->nG);
     sw->zg.alloc(h->nG);
     sw->nv = (int64_t)(h->nelx + 1) * (h->nely + 1) * (h->nelz + 1);
