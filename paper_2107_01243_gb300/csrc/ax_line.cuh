@@ -37,8 +37,8 @@ struct LineCfg {
   static constexpr size_t SMEM = (3 * (size_t)K * VOL + TS) * sizeof(T);
   // CTAs per SM the registers are bounded for (FP64, P = 10: two of 320 threads;
   // FP32, P = 8: three instead of two, sem_apply on 16.8 M points 120 against 134 us)
-  static constexpr int MINB =
-      sizeof(T) == 4 ? (P >= 10 ? 512 : P == 8 ? 768 : MOST) / MOST : (P <= 8 ? 4 : P == 10 ? 2 : 3);
+  static constexpr int MINB = sizeof(T) == 8 ? (P <= 8 ? 4 : P == 10 ? 2 : 3)
+                                             : (P >= 10 ? 512 : P == 8 ? 768 : MOST) / MOST;
 };
 
 // y = D x or D^T x for a line in registers
@@ -83,21 +83,22 @@ struct LineThread {
 // out = (h1 D^T G D + h2 B) u at the k-column: uc the column of u, g, b, h1f the
 // element's G, B and h1 at this thread's (i, j, 0) (h1f may be NULL).  All
 // threads of the CTA call it (act: the thread has an element); U is free once
-// the second barrier is behind.
-template <int P, class T, int MOST>
+// the second barrier is behind.  PREG: components of G an FP32 thread fetches
+// before the forward lines (the rest where they are used).
+template <int PREG = 6, int P, class T, int MOST>
 __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bool act,
                                              const DMat<P, T>& D, const T (&uc)[P], const T* g,
                                              const T* b, const T* h1f, T h1, T h2, T (&out)[P]) {
   using C = LineCfg<P, T, MOST>;
   constexpr int P2 = C::P2, P3 = C::P3, RS = C::RS, PL = C::PL;
-  constexpr bool PRE = sizeof(T) == 4;       // G prefetched to registers
+  constexpr bool PRE = sizeof(T) == 4;       // prefetches to registers
   T gr[PRE ? P : 1][6];
   if (act) {
     if constexpr (PRE) {
 #pragma unroll
       for (int k = 0; k < P; ++k)
 #pragma unroll
-        for (int c = 0; c < 6; ++c) gr[k][c] = __ldcs(g + c * P3 + k * P2);
+        for (int c = 0; c < PREG; ++c) gr[k][c] = __ldcs(g + c * P3 + k * P2);
     }
 #pragma unroll
     for (int k = 0; k < P; ++k) t.U[k * PL + t.col] = uc[k];
@@ -121,15 +122,11 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       const T ur = t.R[k * PL + t.col], us = t.S[k * PL + t.col];
-      T g11, g22, g33, g12, g13, g23;
-      if constexpr (PRE) {
-        g11 = gr[k][0]; g22 = gr[k][1]; g33 = gr[k][2];
-        g12 = gr[k][3]; g13 = gr[k][4]; g23 = gr[k][5];
-      } else {
-        g11 = __ldcs(g + k * P2); g22 = __ldcs(g + P3 + k * P2); g33 = __ldcs(g + 2 * P3 + k * P2);
-        g12 = __ldcs(g + 3 * P3 + k * P2); g13 = __ldcs(g + 4 * P3 + k * P2);
-        g23 = __ldcs(g + 5 * P3 + k * P2);
-      }
+      T gq[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c)
+        gq[c] = PRE && c < PREG ? gr[PRE ? k : 0][c] : __ldcs(g + c * P3 + k * P2);
+      const T g11 = gq[0], g22 = gq[1], g33 = gq[2], g12 = gq[3], g13 = gq[4], g23 = gq[5];
       T wr = fma(g13, ut[k], fma(g12, us, g11 * ur));
       T ws = fma(g23, ut[k], fma(g22, us, g12 * ur));
       T wk = fma(g33, ut[k], fma(g23, us, g13 * ur));

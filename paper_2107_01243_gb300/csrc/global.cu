@@ -59,7 +59,7 @@ __device__ __forceinline__ unsigned dirichlet_bits(const GBox& b, int ex, int ey
 // gathers its own k-column of u from the lattice (rows of P consecutive floats;
 // what neighbours share comes from L2) and scatters its column of outputs.
 // With the clearing of w, on 17 M points: N = 3 102 us, N = 5 115, N = 7 101, N = 9
-// 147 (Poisson; with a mass term 112, 131, 106, 150).  The kernel it took the
+// 135 (Poisson; with a mass term 112, 131, 106, 138).  The kernel it took the
 // place of staged G by bulk copies and read a row and a column of shared memory
 // for every point: 149, 146, 113, 150 (154, 150, 128, 153).  w
 // must hold zeros at every unmasked point on element faces.
@@ -68,13 +68,24 @@ __device__ __forceinline__ unsigned dirichlet_bits(const GBox& b, int ex, int ey
 // Dirichlet points), every warp's sum added to one of kPwSlots accumulators (in
 // no fixed order, as the face sums of w).
 // No loop over elements: with one the compiler keeps D in registers.
+// The operator alone at N = 9 fetches three components of G ahead instead of six,
+// so that six CTAs fit an SM instead of four: 138 us (h2 = 0: 135).  With the
+// Kahan sum (PW, and batch_glob.cuh) the registers do not allow it: 16 problems
+// with 17,000 elements of N = 9 187 against 169 us.
 template <int P, bool PW>
-__global__ void __launch_bounds__(LineCfg<P, float, kGlobThreads>::THREADS, LineCfg<P, float, kGlobThreads>::MINB)
+struct GlobCfg : LineCfg<P, float, kGlobThreads> {
+  static constexpr bool LEAN = P >= 10 && !PW;
+  static constexpr int PREG = LEAN ? 3 : 6;
+  static constexpr int CTAS = LEAN ? 6 : LineCfg<P, float, kGlobThreads>::MINB;
+};
+
+template <int P, bool PW>
+__global__ void __launch_bounds__(GlobCfg<P, PW>::THREADS, GlobCfg<P, PW>::CTAS)
 ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* __restrict__ G,
                const float* __restrict__ B, float h1, float h2,
                const __grid_constant__ DMat<P, float> D, int E, GBox bx,
                const CGState* __restrict__ st, double* __restrict__ slots) {
-  using C = LineCfg<P, float, kGlobThreads>;
+  using C = GlobCfg<P, PW>;
   constexpr int P3 = C::P3, K = C::K, N = P - 1;
   if (st && st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -94,8 +105,8 @@ ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* 
     for (int k = 0; k < P; ++k) uc[k] = __ldg(u + (org + sk * k));
   }
   const size_t base = (size_t)(act ? e : 0) * P3 + t.lam;
-  line_element(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
-               (const float*)nullptr, h1, h2, out);
+  line_element<C::PREG>(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam,
+                        B + base, (const float*)nullptr, h1, h2, out);
   float pw = 0.0f;
   if (act) {
     int dst0 = org;                        // the column's addresses are made anew:
@@ -148,7 +159,7 @@ double* pw_slots(const sem_handle* h) {
 template <int P, bool PW>
 static void launch_glob_p(const sem_handle* h, const float* u, float* w, float h1, float h2,
                           const CGState* st, cudaStream_t s) {
-  using C = LineCfg<P, float, kGlobThreads>;
+  using C = GlobCfg<P, PW>;
   auto kern = ax_glob_kernel<P, PW>;
   static bool configured = false;
   if (!configured) {

@@ -265,6 +265,7 @@ struct OpEO {
       if (has(m)) U[qoff[m]] = in[m];
     __syncthreads();
     if (act) eo_line<P, T>(U, my, loff, tab);
+    const bool scale = a.h1f || a.h1 != T(1);
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < NQ; ++m) {
@@ -274,8 +275,8 @@ struct OpEO {
       T wr = fma(gr[m][4], ut, fma(gr[m][3], us, gr[m][0] * ur));
       T ws = fma(gr[m][5], ut, fma(gr[m][1], us, gr[m][3] * ur));
       T wt = fma(gr[m][2], ut, fma(gr[m][5], us, gr[m][4] * ur));
-      const T c = a.h1f ? __ldg(a.h1f + (size_t)e * P3 + tid + m * NT) : a.h1;
-      if (c != T(1)) {
+      if (scale) {
+        const T c = a.h1f ? __ldg(a.h1f + (size_t)e * P3 + tid + m * NT) : a.h1;
         wr *= c;
         ws *= c;
         wt *= c;
