@@ -210,7 +210,7 @@ __device__ __forceinline__ void sw_line(const SwConst<PE>& k, bool interior, con
 // with all tables in shared memory spent three 16-byte reads on every output),
 // the interior scaling as a table of reciprocals, and one element a CTA, so
 // that tables that are not used are not loaded and the registers allow twice
-// the CTAs.  13,824 elements, N = 7: LOCALUS.
+// the CTAs.  13,824 elements, N = 7: 91 us (160 before).
 template <int PE>
 __global__ void __launch_bounds__(SwCfg<PE>::THREADS, SwCfg<PE>::MINB)
 schwarz_local_kernel(const float* __restrict__ rg, float* __restrict__ zg,
@@ -520,6 +520,154 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
   if (act) a.x[v] = x;
 }
 
+// ---- the same iterations in one cluster of 16 CTAs, where a thread per vertex
+// fits (up to 16,384 vertices): barriers and sums through distributed shared
+// memory instead of the grid's global ones.  A CTA keeps p of its own vertices
+// and of their neighbours (a halo of one layer and row on either side) in shared
+// memory.  10 iterations on 25^3 vertices: CLUSTERUS.
+constexpr int kClusterCtas = 16, kClusterThreads = 1024;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+// 16 bytes to the same shared address of CTA `to` of the cluster
+__device__ __forceinline__ void cluster_put(longlong2* p, uint32_t to, longlong2 v) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(to));
+  asm volatile("st.shared::cluster.v2.s64 [%0], {%1, %2};" ::"r"(a), "l"(v.x), "l"(v.y) : "memory");
+}
+
+// Sum of v over the cluster, in every thread of warp 0 (others get nothing).
+// slots: kClusterCtas entries, two sets used in turn by the caller.
+__device__ __forceinline__ double cluster_sum(double v, FxVal* sw, longlong2* slots) {
+  constexpr int NW = kClusterThreads / 32;
+  const int lane = threadIdx.x & 31;
+  const FxVal f = fx_warp_sum(v);
+  if (lane == 0) sw[threadIdx.x >> 5] = f;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const FxVal f0 = sw[lane];               // NW = 32 warps
+    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f0.e);
+    FxAcc acc;
+    if (e < kFxBad) acc.add(f0, e);
+    acc = fx_warp_add(acc);
+    // 32 x 2^62: 5 bits to the right it fits 63 bits again
+    if (lane < kClusterCtas)
+      cluster_put(slots + cluster_rank(), lane,
+                  make_longlong2((acc.hi << 27) + (acc.lo >> 5), e + 5));
+    __syncwarp();
+  }
+  static_assert(NW == 32, "a lane per warp");
+  cluster_barrier();
+  if (threadIdx.x >= 32) return 0.0;
+  const longlong2 p = lane < kClusterCtas ? slots[lane] : make_longlong2(0, 1);
+  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.y);
+  FxAcc acc;
+  if (e < kFxBad) acc.add(FxVal{p.x, (int)p.y}, e);
+  acc = fx_warp_add(acc);
+  return fx_round(acc.hi, acc.lo, e);
+}
+
+// a / b rounded to FP32, for positive normal doubles (an FP64 division takes a
+// lone warp half a microsecond): the significands as pairs of floats, the
+// quotient of the leading parts and its first-order correction (Dekker 1971)
+__device__ __forceinline__ float ratio32(double a, double b) {
+  const long long ia = dbits(a), ib = dbits(b);
+  const long long ma = (ia & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  const long long mb = (ib & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  const float ah = (float)(int)(ma >> 29), al = (float)(int)(ma & 0x1FFFFFFF) * 0x1p-29f;
+  const float bh = (float)(int)(mb >> 29), bl = (float)(int)(mb & 0x1FFFFFFF) * 0x1p-29f;
+  const float q = __fdiv_rn(ah, bh);
+  const float rem = fmaf(-q, bl, fmaf(-q, bh, ah) + al);
+  return ldexpf(q + __fdiv_rn(rem, bh), (int)(ia >> 52) - (int)(ib >> 52));
+}
+
+__global__ void __launch_bounds__(kClusterThreads, 1)
+k_coarse_cluster(const __grid_constant__ CoarseArgs a, int nvc, int halo) {
+  extern __shared__ float s_p[];             // p of vertices v0 - halo .. v0 + nvc + halo
+  __shared__ FxVal sw[32];
+  __shared__ longlong2 slots[2][kClusterCtas];
+  __shared__ float s_coef;                   // alpha or beta of the step
+  __shared__ int s_stop;
+  const int nv = a.nvx * a.nvy * a.nvz, tid = threadIdx.x;
+  const int v0 = (int)cluster_rank() * nvc, v = v0 + tid;
+  const bool act = tid < nvc && v < nv;
+  float c[27];
+#pragma unroll
+  for (int o = 0; o < 27; ++o) c[o] = act ? __ldg(a.st + (size_t)o * nv + v) : 0.0f;
+  const float d = act ? a.dinv[v] : 0.0f;
+  float r = act ? a.r[v] : 0.0f, x = 0.0f, z = d * r;
+  if (act) {
+    __stcg(a.z + v, z);
+    __stcg(a.p0 + v, 0.0f);
+  }
+  cluster_barrier();                         // every CTA has started: its memory may be written
+  const int span = nvc + 2 * halo;
+  double rz = 0.0;                           // warp 0
+  int set = 0;
+  float *pold = a.p0, *pnew = a.p1;
+  // one reduction, then warp 0's thread 0 makes the step's coefficient
+  auto meet = [&](double val, auto step) {
+    const double t = cluster_sum(val, sw, slots[set]);
+    set ^= 1;
+    if (tid < 32) {
+      const bool bad = dbits(t) <= 0 || is_nan(t);
+      const float cf = step(t, bad);
+      if (tid == 0) {
+        s_stop = bad;
+        s_coef = cf;
+      }
+    }
+    __syncthreads();
+  };
+  meet((double)r * (double)z, [&](double t, bool) {
+    rz = t;
+    return 0.0f;
+  });
+  for (int it = 0; it < a.iters && !s_stop; ++it) {
+    const float beta = s_coef;
+    for (int q = tid; q < span; q += kClusterThreads) {
+      const int n = v0 - halo + q;
+      s_p[q] = n >= 0 && n < nv ? fmaf(beta, __ldcg(pold + n), __ldcg(a.z + n)) : 0.0f;
+    }
+    __syncthreads();
+    float w = 0.0f, p = 0.0f;
+    if (act) {
+      // neighbours outside the box have zero entries
+      const float* sp = s_p + halo + tid;
+      p = sp[0];
+      __stcg(pnew + v, p);
+#pragma unroll
+      for (int o = 0; o < 27; ++o)
+        w = fmaf(c[o], sp[o % 3 - 1 + a.nvx * ((o / 3) % 3 - 1 + a.nvy * (o / 9 - 1))], w);
+    }
+    meet((double)p * (double)w,
+         [&](double t, bool bad) { return bad ? 0.0f : ratio32(rz, t); });
+    if (s_stop) break;
+    const float alpha = s_coef;
+    x = fmaf(alpha, p, x);
+    r = fmaf(-alpha, w, r);
+    z = d * r;
+    if (it + 1 == a.iters) break;            // the last direction has been taken
+    if (act) __stcg(a.z + v, z);
+    meet((double)r * (double)z, [&](double t, bool bad) {
+      const float b = bad ? 0.0f : ratio32(t, rz);
+      rz = t;
+      return b;
+    });
+    float* t = pold;
+    pold = pnew;
+    pnew = t;
+  }
+  if (act) a.x[v] = x;
+}
+
 // L-vector of vertex function v (all elements), FP64
 __global__ void k_vertex_field(int64_t nL, int P, int v, const double* __restrict__ xi,
                                double* __restrict__ out) {
@@ -666,6 +814,7 @@ struct sem_schwarz {
   DevBuf<float> stencil, zc;
   DevBuf<double> cpart;
   DevBuf<unsigned> cbar;
+  bool cluster_ok = false;                 // in one cluster
   DevBuf<float> rg, zg;                    // fine global vectors
   DevBuf<CGState> st;
   DevBuf<double> partials;
@@ -751,6 +900,7 @@ void build_tables(sem_schwarz* sw, std::vector<float>& out) {
 }
 
 int64_t coarse_cg_threads();
+bool cluster_fits(const sem_schwarz* sw, cudaStream_t s);
 
 // coarse element matrices from the FP64 element operator
 void build_coarse(sem_schwarz* sw, cudaStream_t s) {
@@ -788,6 +938,7 @@ void build_coarse(sem_schwarz* sw, cudaStream_t s) {
     k_coarse_stencil<<<ew_blocks(sw->nv), 256, 0, s>>>(h->nelx, h->nely, h->nelz, sw->K.ptr,
                                                        sw->stencil.ptr, (int)sw->nv);
     SEM_CHECK_LAUNCH();
+    sw->cluster_ok = cluster_fits(sw, s);
   }
   SEM_CUDA(cudaStreamSynchronize(s));      // the scratch buffers are freed on return
 }
@@ -810,6 +961,46 @@ int64_t coarse_cg_threads() {
   return (int64_t)std::min(kCoarseBlocks, occ * sem_num_sms()) * kCoarseThreads;
 }
 
+// the one-cluster form: vertices per CTA, neighbours kept on either side, launch
+int cluster_share(const sem_schwarz* sw) {
+  return (int)((sw->nv + kClusterCtas - 1) / kClusterCtas);
+}
+int cluster_halo(const sem_schwarz* sw) {
+  const int nvx = sw->h->nelx + 1, nvy = sw->h->nely + 1;
+  return nvx * nvy + nvx + 1;
+}
+cudaLaunchConfig_t cluster_config(const sem_schwarz* sw, cudaLaunchAttribute* at, cudaStream_t s) {
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = kClusterCtas;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kClusterCtas);
+  cfg.blockDim = dim3(kClusterThreads);
+  cfg.dynamicSmemBytes = (size_t)(cluster_share(sw) + 2 * cluster_halo(sw)) * sizeof(float);
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+// whether the vertices fit one cluster and the device can hold it
+bool cluster_fits(const sem_schwarz* sw, cudaStream_t s) {
+  if (cluster_share(sw) > kClusterThreads) return false;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = cluster_config(sw, &at, s);
+  if (cfg.dynamicSmemBytes > 200 * 1024) return false;
+  SEM_CUDA(cudaFuncSetAttribute(k_coarse_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                1));
+  SEM_CUDA(cudaFuncSetAttribute(k_coarse_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                200 * 1024));
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, k_coarse_cluster, &cfg) != cudaSuccess) {
+    cudaGetLastError();                      // not a failure of the solve
+    return false;
+  }
+  return n >= 1;
+}
+
 void launch_coarse_cg(sem_schwarz* sw, cudaStream_t s) {
   const sem_handle* h = sw->h;
   CoarseArgs a{};
@@ -828,6 +1019,12 @@ void launch_coarse_cg(sem_schwarz* sw, cudaStream_t s) {
   a.nvy = h->nely + 1;
   a.nvz = h->nelz + 1;
   a.iters = sw->coarse_iters;
+  if (sw->cluster_ok) {
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t cfg = cluster_config(sw, &at, s);
+    SEM_CUDA(cudaLaunchKernelEx(&cfg, k_coarse_cluster, a, cluster_share(sw), cluster_halo(sw)));
+    return;
+  }
   SEM_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
   const int grid = (int)((sw->nv + kCoarseThreads - 1) / kCoarseThreads);
   void* args[] = {&a};
