@@ -524,7 +524,8 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
 // fits (up to 16,384 vertices): barriers and sums through distributed shared
 // memory instead of the grid's global ones.  A CTA keeps p of its own vertices
 // and of their neighbours (a halo of one layer and row on either side) in shared
-// memory.  10 iterations on 25^3 vertices: CLUSTERUS.
+// memory.  Bound by the latency of its 20 sums, one after another: 10
+// iterations on 25^3 vertices 57 us (97 as a cooperative grid).
 constexpr int kClusterCtas = 16, kClusterThreads = 1024;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
