@@ -97,8 +97,8 @@ def ax_source_digest(root=ROOT):
 # schedulers x the maximum SM clock.
 AX_CAPTURES = {
     "ax_df_kernel<8, 1, 1>": {
-        "source": "337018094dbfaa39",
-        "dram_bytes": 939_699_456 + 78_679_552,
+        "source": "397f10f47f1d106b",
+        "dram_bytes": 939_732_736 + 78_302_464,
         "warp_instructions": 249_740_848,       # profiles/ax_df_kernel_fused_f64_e32768_n7.md
     },
 }

@@ -442,8 +442,8 @@ sem_status sem_gmres_solve(sem_handle* h, const double* b_L, double* x_L,
  * SEM_PREC_F32 and an odd N (even points per direction), into a batch that
  * advances all their solves together: every stage of an FP32 inner CG
  * iteration (the operator, the vector updates with per-problem dot products)
- * is one kernel launch over all problems (the element kernels one persistent
- * launch per order present), and batches of iterations are captured in a
+ * is one kernel launch over all problems (the element kernels one launch per
+ * order present), and batches of iterations are captured in a
  * CUDA graph.  The inner PCG runs on global vectors (as sem_apply_global)
  * unless a handle asks for L-vectors (sem_set_inner_vectors).  Each problem refines in FP64 as
  * in sem_cg_solve with SEM_SOLVE_MIXED (constant h1, h2 per problem).
@@ -460,8 +460,8 @@ sem_status sem_batch_destroy(sem_batch* b);
 /* sem_batch_set_concurrency: concurrent = 1 launches the element kernels of
  * the order classes of an inner iteration as concurrent branches (side
  * streams forked from and joined back into the solve's stream; parallel paths
- * of the iteration graph), so that the persistent grids of the classes can
- * fill one another's tails; 0 (the default) launches them one after another.
+ * of the iteration graph), so that the grids of the classes can fill one
+ * another's tails; 0 (the default) launches them one after another.
  * The classes touch disjoint problems, so either way computes the same
  * iteration.  SEM_ERR_ARG for a NULL batch or a flag other than 0 or 1. */
 sem_status sem_batch_set_concurrency(sem_batch* b, int concurrent);
