@@ -1,5 +1,5 @@
 """Asynchronous calls recorded into a CUDA graph replay to the eager results:
-the Schwarz preconditioner (whose coarse solve is one cooperative launch) and
+the Schwarz preconditioner (whose coarse solve is one cluster or one cooperative launch) and
 the assembled operators."""
 import math
 
@@ -25,7 +25,8 @@ def replayed(call, out):
     return eager, out.clone()
 
 
-@pytest.mark.parametrize("nel,N", [((3, 4, 5), 5), ((9, 8, 7), 7), ((2, 1, 1), 2)])
+@pytest.mark.parametrize("nel,N", [((3, 4, 5), 5), ((9, 8, 7), 7), ((2, 1, 1), 2),
+                                   ((32, 31, 15), 2)])   # 16,896 vertices: a grid
 def test_schwarz_apply_captured(nel, N):
     h = sem.sem_setup(nel, N, length=(2 * math.pi,) * 3, deform=0.1)
     m = sem.sem_schwarz_create(h)
