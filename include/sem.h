@@ -216,8 +216,8 @@ sem_status sem_ax(sem_handle* h, const void* u_L, void* w_L, double h1, double h
  * result.  An element whose u holds an Inf or a NaN gives NaN at all of its
  * points (the native kernel lets them spread through the element's contractions
  * instead, so some of its points stay finite).
- * SEM_F64_KERNEL_NATIVE forces IEEE FP64 arithmetic (except at N = 1 and 3 with
- * the even-odd split of D, about a fifth fewer FP64 operations).  Returns SEM_ERR_ARG
+ * SEM_F64_KERNEL_NATIVE forces IEEE FP64 arithmetic (at N = 7 and 9 with the
+ * even-odd split of D, about 20% fewer FP64 operations).  Returns SEM_ERR_ARG
  * for an unknown kind.
  */
 sem_status sem_set_f64_kernel(sem_handle* h, int kind);
@@ -264,9 +264,10 @@ sem_status sem_set_tuning(sem_handle* h, const sem_tuning* t);
  * finish phase must follow a local phase on the same handle, dtype and
  * vectors; splitting lets a caller time or overlap the two).  Segments hold
  * four elements (double-float, FP32 bulk copies) or as many as the line kernel
- * takes per CTA.  FP64 at N = 1 and 3 runs sem_ax and sem_dssum's kernels
- * instead, the local phase being the element operator and the finish phase
- * the whole gather-scatter.  u_L and w_L are distinct L-vectors of the
+ * takes per CTA.  IEEE FP64 (even N, the native kernel, a per-point h1), except
+ * at N = 7 and 9 on large meshes, runs sem_ax and sem_dssum's kernels instead,
+ * the local phase being the element operator and the finish phase the whole
+ * gather-scatter.  u_L and w_L are distinct L-vectors of the
  * dtype (SEM_F64 or SEM_F32); SEM_ERR_ARG otherwise.
  */
 sem_status sem_apply(sem_handle* h, const void* u_L, void* w_L, double h1, double h2,

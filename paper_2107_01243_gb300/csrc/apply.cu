@@ -320,10 +320,10 @@ void finish_slab(const sem_handle* h, double* w, int z0, int z1, cudaStream_t s)
 // line: the element kernel was the line kernel (its own segment length)
 template <int P, class T>
 void finish_p(const sem_handle* h, T* w, bool line, const CGState* st, cudaStream_t s) {
-  if (line)
-    finish_box<P, line_elems(P, sizeof(T) == 8), T>(w, h->nelx, h->nely, h->nelz, st, s);
-  else if constexpr (P % 2 == 0)
-    finish_box<P, kFuseSeg, T>(w, h->nelx, h->nely, h->nelz, st, s);
+  if constexpr (sizeof(T) == 4 || eo_split(P, true))
+    if (line)
+      return finish_box<P, line_elems(P, sizeof(T) == 8), T>(w, h->nelx, h->nely, h->nelz, st, s);
+  if constexpr (P % 2 == 0) finish_box<P, kFuseSeg, T>(w, h->nelx, h->nely, h->nelz, st, s);
 }
 
 template <class T>

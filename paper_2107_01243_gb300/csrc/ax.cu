@@ -1,10 +1,11 @@
 // Matrix-free element operator w_e = (h1 D^T G_e D + h2 B_e) u_e
 // (arXiv 2107.01243 §2, Eq. 9; the ax_t compute of Listing 1).
 //
-// The dispatch between the kernels, and the column kernel of FP64 at P = 2 and 4
-// (ax_line.cu, ax_df.cu and ax_tma.cu hold the others).
+// The dispatch between the kernels, the column kernel of IEEE FP64 and its
+// even-odd kernel at P = 8 and 10 (ax_line.cu, ax_df.cu and ax_tma.cu hold the
+// others).
 //
-// Layout: one CTA works on EPB elements at a time; inside an element a
+// Column kernel: one CTA works on EPB elements at a time; inside an element a
 // P x P thread plane owns the k-columns (i, j, 0..P-1).  The column of u
 // stays in registers (t-derivative and its transpose in registers), the
 // element is staged in shared memory for the r- and s-derivatives, rows are
@@ -103,6 +104,117 @@ ax_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__ G,
   }
 }
 
+// ------------------------------------------------- IEEE FP64, P = 8 and 10
+// One element per CTA of 3 P^2 threads with the even-odd split of D (eo_tile.cuh):
+// group g runs the lines of direction g (forward derivatives, then transposed
+// contractions, in place), and the geometric factors are applied point by point
+// in between.  GB300's FP64 pipe bounds it; against the column kernel on 32^3-size
+// meshes 2.6% and 17% less time (at P = 6 its 108-thread CTAs idle a fifth of
+// their lanes: 18% more).
+template <int P>
+__global__ void __launch_bounds__(3 * P * P)
+ax_eo_kernel(const double* __restrict__ u, double* __restrict__ w, const double* __restrict__ G,
+             const double* __restrict__ B, const double* __restrict__ h1f, double h1, double h2,
+             const double* __restrict__ tabg, int E, const CGState* __restrict__ st) {
+  using L = EoLayout<P, double>;
+  constexpr int P2 = P * P, P3 = P2 * P, NT = 3 * P2, NQ = (P3 + NT - 1) / NT;
+  constexpr int TS = LineTab<P, double>::SIZE;
+  if (st && st->done) return;
+  __shared__ double sU[L::VOL];
+  __shared__ double sR[3][L::VOL];
+  __shared__ double sTab[TS];
+  const int tid = threadIdx.x;
+  for (int q = tid; q < TS; q += NT) sTab[q] = tabg[q];
+  const int g = tid / P2, lam = tid % P2, c1 = lam % P, c2 = lam / P;
+  int loff[P];
+#pragma unroll
+  for (int l = 0; l < P; ++l)
+    loff[l] = g == 0 ? L::at(l, c1, c2) : (g == 1 ? L::at(c1, l, c2) : L::at(c1, c2, l));
+  int qoff[NQ];
+#pragma unroll
+  for (int m = 0; m < NQ; ++m) {
+    const int q = tid + m * NT;
+    qoff[m] = q < P3 ? L::at(q % P, (q / P) % P, q / P2) : 0;
+  }
+  double* myR = sR[g];
+  const bool helm = h2 != 0.0;
+  for (int e = blockIdx.x; e < E; e += gridDim.x) {
+    const size_t base = (size_t)e * P3;
+#pragma unroll
+    for (int m = 0; m < NQ; ++m) {
+      const int q = tid + m * NT;
+      if (q < P3) sU[qoff[m]] = u[base + q];
+    }
+    __syncthreads();
+    tab_line<P, double, false>(sU, myR, loff, sTab);     // forward derivatives along g
+    __syncthreads();
+    const double* ge = G + (size_t)e * 6 * P3;
+#pragma unroll
+    for (int m = 0; m < NQ; ++m) {
+      const int q = tid + m * NT;
+      if (q >= P3) break;
+      const int at = qoff[m];
+      const double ur = sR[0][at], us = sR[1][at], ut = sR[2][at];
+      const double g11 = ge[q], g22 = ge[P3 + q], g33 = ge[2 * P3 + q];
+      const double g12 = ge[3 * P3 + q], g13 = ge[4 * P3 + q], g23 = ge[5 * P3 + q];
+      double wr = fma(g13, ut, fma(g12, us, g11 * ur));
+      double ws = fma(g23, ut, fma(g22, us, g12 * ur));
+      double wt = fma(g33, ut, fma(g23, us, g13 * ur));
+      const double c = h1f ? h1f[base + q] : h1;
+      if (h1f || c != 1.0) {
+        wr *= c;
+        ws *= c;
+        wt *= c;
+      }
+      sR[0][at] = wr;
+      sR[1][at] = ws;
+      sR[2][at] = wt;
+    }
+    __syncthreads();
+    tab_line<P, double, true>(myR, myR, loff, sTab);     // transposed contractions, in place
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < NQ; ++m) {
+      const int q = tid + m * NT;
+      if (q >= P3) break;
+      const int at = qoff[m];
+      double acc = (sR[0][at] + sR[1][at]) + sR[2][at];
+      if (helm) acc = fma(h2 * B[base + q], sU[at], acc);
+      w[base + q] = acc;
+    }
+    // the next element's first phase rewrites sU (read above for Helmholtz)
+    // and its forward phase sR (read above): all threads finish here first
+    __syncthreads();
+  }
+}
+
+template <int P>
+static int eo_occupancy() {
+  static const int occ = [] {
+    int o = 0;
+    SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, ax_eo_kernel<P>, 3 * P * P, 0));
+    return std::max(1, o);
+  }();
+  return occ;
+}
+
+// once-per-process setup, run by sem_setup outside any stream capture
+void eo_prepare(const sem_handle* h) {
+  if (h->P == 8) eo_occupancy<8>();
+  if (h->P == 10) eo_occupancy<10>();
+}
+
+template <int P>
+static void launch_eo_p(const sem_handle* h, const OpData<double>& op, const double* u, double* w,
+                        double h1, double h2, const double* h1f, const CGState* st,
+                        cudaStream_t s) {
+  const int E = (int)h->E;
+  const int grid = (int)std::min<int64_t>(E, (int64_t)eo_occupancy<P>() * sem_num_sms());
+  ax_eo_kernel<P><<<grid, 3 * P * P, 0, s>>>(u, w, op.G.ptr, op.B.ptr, h1f, h1, h2,
+                                             op.D.ptr + LineTab<P, double>::FROM, E, st);
+  SEM_CHECK_LAUNCH();
+}
+
 // diag(H^e) at every local point: the rr, ss, tt terms run along the line
 // through the point, the mixed terms only see the point (D_ii D_jj ...).
 template <class T>
@@ -164,12 +276,23 @@ void launch_ax(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1,
     if (h->f64_kernel == SEM_F64_KERNEL_DOUBLEFLOAT)
       throw Error(SEM_ERR_STATE, "double-float Ax needs N in {5, 7, 9}, constant h1 and "
                                  "16-byte aligned vectors");
-    if (line_ax_supported<double>(h))
+    if (line_ax_supported<double>(h)) {
       launch_ax_line<double>(h, op, u, w, h1, h2, h1f, false, st, s);
-    else if (h->P == 2)
-      launch_ax_p<2, double>(h, op, u, w, h1, h2, h1f, st, s);
-    else
-      launch_ax_p<4, double>(h, op, u, w, h1, h2, h1f, st, s);
+      return;
+    }
+    switch (h->P) {
+      case 2: launch_ax_p<2, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 3: launch_ax_p<3, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 4: launch_ax_p<4, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 5: launch_ax_p<5, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 6: launch_ax_p<6, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 7: launch_ax_p<7, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 8: launch_eo_p<8>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 9: launch_ax_p<9, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 10: launch_eo_p<10>(h, op, u, w, h1, h2, h1f, st, s); break;
+      case 11: launch_ax_p<11, double>(h, op, u, w, h1, h2, h1f, st, s); break;
+      default: throw Error(SEM_ERR_ARG, "launch_ax: unsupported order");
+    }
   }
 }
 

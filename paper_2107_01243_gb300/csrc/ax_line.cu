@@ -1,8 +1,7 @@
 // Element operator w_e = (h1 D^T G_e D + h2 B_e) u_e (arXiv 2107.01243 §2,
-// Eq. 9) for any number of points P, any alignment and both precisions, from
-// plain coalesced loads: the FP32 kernel of odd P (whose elements are no whole
-// number of 16 bytes, so that bulk copies cannot fetch them) and the IEEE FP64
-// kernel.
+// Eq. 9) from plain coalesced loads at any alignment: the FP32 kernel of every P
+// (elements of odd P are no whole number of 16 bytes, so that bulk copies cannot
+// fetch them) and the IEEE FP64 kernel of large meshes at P = 8 and 10.
 //
 // A CTA takes K consecutive elements, K chosen so that K P^2 threads fill whole
 // warps (P = 7: five elements, 245 of 256 lanes).  Thread (i, j) of an element
@@ -113,19 +112,24 @@ static void launch_line_p(const sem_handle* h, const OpData<T>& op, const T* u, 
 template <class T>
 void launch_ax_line(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2,
                     const T* h1f, bool fuse, const CGState* st, cudaStream_t s) {
-  switch (h->P) {
-    case 2: launch_line_p<2, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 3: launch_line_p<3, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 4: launch_line_p<4, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 5: launch_line_p<5, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 6: launch_line_p<6, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 7: launch_line_p<7, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 8: launch_line_p<8, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 9: launch_line_p<9, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 10: launch_line_p<10, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    case 11: launch_line_p<11, T>(h, op, u, w, h1, h2, h1f, fuse, st, s); break;
-    default: throw Error(SEM_ERR_ARG, "launch_ax_line: unsupported order");
+  if constexpr (sizeof(T) == 8) {
+    if (h->P == 8) return launch_line_p<8, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+    if (h->P == 10) return launch_line_p<10, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+  } else {
+    switch (h->P) {
+      case 2: return launch_line_p<2, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 3: return launch_line_p<3, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 4: return launch_line_p<4, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 5: return launch_line_p<5, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 6: return launch_line_p<6, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 7: return launch_line_p<7, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 8: return launch_line_p<8, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 9: return launch_line_p<9, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 10: return launch_line_p<10, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+      case 11: return launch_line_p<11, T>(h, op, u, w, h1, h2, h1f, fuse, st, s);
+    }
   }
+  throw Error(SEM_ERR_ARG, "launch_ax_line: unsupported order");
 }
 
 template void launch_ax_line<float>(const sem_handle*, const OpData<float>&, const float*, float*,

@@ -33,11 +33,11 @@ struct LineCfg {
   static constexpr int P2 = P * P, P3 = P2 * P, K = line_elems(P, sizeof(T) == 8, MOST);
   static constexpr int THREADS = (K * P2 + 31) / 32 * 32;
   static constexpr int RS = P | 1, PL = P * RS, VOL = P * PL;   // rows of odd length
-  static constexpr int TS = sizeof(T) == 8 ? 2 * EoTab<P>::SIZE : 0;
+  static constexpr int TS = LineTab<P, T>::EO ? LineTab<P, T>::SIZE : 0;
   static constexpr size_t SMEM = (3 * (size_t)K * VOL + TS) * sizeof(T);
-  // CTAs per SM the registers are bounded for (FP64, P = 10: two of 320 threads;
+  // CTAs per SM the registers are bounded for (FP64: P = 8 four of 256, P = 10 two of 320 threads;
   // FP32, P = 8: three instead of two, sem_apply on 16.8 M points 120 against 134 us)
-  static constexpr int MINB = sizeof(T) == 8 ? (P <= 8 ? 4 : P == 10 ? 2 : 3)
+  static constexpr int MINB = sizeof(T) == 8 ? (P == 8 ? 4 : 2)
                                              : (P >= 10 ? 512 : P == 8 ? 768 : MOST) / MOST;
 };
 
@@ -45,7 +45,7 @@ struct LineCfg {
 template <int P, class T, bool TRANS, class PUT>
 __device__ __forceinline__ void line_dots(const T (&x)[P], const DMat<P, T>& D, const T* tab,
                                           PUT put) {
-  if constexpr (sizeof(T) == 8) {
+  if constexpr (LineTab<P, T>::EO) {
     eo_dots<P, T>(x, tab + (TRANS ? EoTab<P>::SIZE : 0), put);
   } else {
 #pragma unroll
@@ -173,14 +173,19 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
 // (8 M points, us, against the kernel it took the place of: N = 2 58 / 79, N = 4
 // 50 / 76, N = 6 49 / 99, N = 8 52 / 91; against the bulk-copy kernel, which
 // stays for large meshes at N = 7 and 9 and for tuned handles: N = 1 58 / 209,
-// N = 3 46 / 52, N = 5 45 / 56, N = 7 42 / 42, N = 9 59 / 61).  FP64: not at P = 2 and 4, where the split saves next to
-// nothing and the column kernel keeps the FP64 pipe busier (N = 1 447 / 367, N = 3
-// 585 / 528; N = 2 431 / 452, N = 4 603 / 637, N = 6 670 / 810, N = 8 805 / 1037,
-// N = 10 814 / 1072, and against the one-element even-odd kernel N = 7 681 / 783,
-// N = 9 818 / 923); nor where a handle insists on the double-float kernel.
+// N = 3 46 / 52, N = 5 45 / 56, N = 7 42 / 42, N = 9 59 / 61; on 27 to 1,000
+// elements sem_apply takes 0.40 to 0.85 of the former kernels' time).  IEEE FP64:
+// the orders of the even-odd split from kLineElems64 elements (8 M points, against
+// the one-element kernel: N = 7 681 / 783, N = 9 818 / 923; sem_apply on 1,728
+// elements 92 / 98 and 200 / 222, on 1,000 65 / 59 and 152 / 129, on 64 34 / 13 and
+// 52 / 23: a CTA's four or three elements are a chain four or three times as long
+// on the FP64 pipe).  Elsewhere the column kernel (N = 6, 8,000 elements 298 against
+// 329 us with plain lines), nor where a handle insists on the double-float kernel.
+constexpr int64_t kLineElems64 = 1536;
 template <class T>
 inline bool line_ax_supported(const sem_handle* h) {
-  return sizeof(T) == 4 || (h->P != 2 && h->P != 4 && h->f64_kernel != SEM_F64_KERNEL_DOUBLEFLOAT);
+  return sizeof(T) == 4 || (eo_split(h->P, true) && h->E >= kLineElems64 &&
+                            h->f64_kernel != SEM_F64_KERNEL_DOUBLEFLOAT);
 }
 
 // w = (h1 A + h2 B) u on L-vectors; fuse: masked points zero, x-pairs inside

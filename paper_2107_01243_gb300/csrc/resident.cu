@@ -53,7 +53,7 @@ struct ResArgs {
   const float* imult;
   const void *G, *B;          // T values, or float pairs (double-float operator)
   const T* h1f;               // per-point h1 or NULL
-  const T* tab;               // even-odd tables of D and D^T
+  const T* tab;               // IEEE operators: LineTab
   const int* esc;             // double-float: exponents of G and B per element
   T h1, h2;
   DFScal df;                  // double-float: h1 and h2
@@ -217,15 +217,15 @@ struct OpDF {
   }
 };
 
-// IEEE arithmetic in T (FP64 or FP32), even-odd lines, optional per-point h1
+// IEEE arithmetic in T (FP64 or FP32), optional per-point h1
 template <int P, class TT>
-struct OpEO {
+struct OpIEEE {
   using T = TT;
   static constexpr bool ONE = true;      // one barrier
   using L = EoLayout<P, T>;
   static constexpr int P2 = P * P, P3 = P2 * P, NT = 3 * P2, NTB = (NT + 31) / 32 * 32;
-  static constexpr int NQ = (P3 + NT - 1) / NT, TS = EoTab<P>::SIZE;
-  static constexpr size_t SMEM = (4 * (size_t)L::VOL + 2 * TS) * sizeof(T);
+  static constexpr int NQ = (P3 + NT - 1) / NT, TS = LineTab<P, T>::SIZE;
+  static constexpr size_t SMEM = (4 * (size_t)L::VOL + TS) * sizeof(T);
   T *U, *R0, *R1, *R2, *my, *tab;
   int loff[P], qoff[NQ];
   bool act;
@@ -236,7 +236,7 @@ struct OpEO {
     R2 = R1 + L::VOL;
     tab = R2 + L::VOL;
     const int tid = threadIdx.x, g = tid / P2, lam = tid % P2, c1 = lam % P, c2 = lam / P;
-    for (int q = tid; q < 2 * TS; q += NTB) tab[q] = a.tab[q];
+    for (int q = tid; q < TS; q += NTB) tab[q] = a.tab[q];
     act = tid < NT;
     my = g == 0 ? R0 : (g == 1 ? R1 : R2);
 #pragma unroll
@@ -264,7 +264,7 @@ struct OpEO {
     for (int m = 0; m < NQ; ++m)
       if (has(m)) U[qoff[m]] = in[m];
     __syncthreads();
-    if (act) eo_line<P, T>(U, my, loff, tab);
+    if (act) tab_line<P, T, false>(U, my, loff, tab);
     const bool scale = a.h1f || a.h1 != T(1);
     __syncthreads();
 #pragma unroll
@@ -286,7 +286,7 @@ struct OpEO {
       R2[at] = wt;
     }
     __syncthreads();
-    if (act) eo_line<P, T>(my, my, loff, tab + TS);
+    if (act) tab_line<P, T, true>(my, my, loff, tab);
     __syncthreads();
     const T* b = static_cast<const T*>(a.B) + (size_t)e * P3;
 #pragma unroll
@@ -704,18 +704,23 @@ static void resident_common(sem_handle* h, const PcgVecs<T>& v, ResArgs<T>& a, i
 }
 
 template <class T>
-static void launch_resident_eo(sem_handle* h, ResArgs<T>& a, cudaStream_t s) {
+static void launch_resident_ieee(sem_handle* h, const T* D, ResArgs<T>& a, cudaStream_t s) {
+  auto go = [&](auto p) {
+    constexpr int P = decltype(p)::value;
+    a.tab = D + LineTab<P, T>::FROM;
+    launch_resident_op<OpIEEE<P, T>>(h, a, s);
+  };
   switch (h->P) {
-    case 2: launch_resident_op<OpEO<2, T>>(h, a, s); break;
-    case 3: launch_resident_op<OpEO<3, T>>(h, a, s); break;
-    case 4: launch_resident_op<OpEO<4, T>>(h, a, s); break;
-    case 5: launch_resident_op<OpEO<5, T>>(h, a, s); break;
-    case 6: launch_resident_op<OpEO<6, T>>(h, a, s); break;
-    case 7: launch_resident_op<OpEO<7, T>>(h, a, s); break;
-    case 8: launch_resident_op<OpEO<8, T>>(h, a, s); break;
-    case 9: launch_resident_op<OpEO<9, T>>(h, a, s); break;
-    case 10: launch_resident_op<OpEO<10, T>>(h, a, s); break;
-    case 11: launch_resident_op<OpEO<11, T>>(h, a, s); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 3: go(std::integral_constant<int, 3>()); break;
+    case 4: go(std::integral_constant<int, 4>()); break;
+    case 5: go(std::integral_constant<int, 5>()); break;
+    case 6: go(std::integral_constant<int, 6>()); break;
+    case 7: go(std::integral_constant<int, 7>()); break;
+    case 8: go(std::integral_constant<int, 8>()); break;
+    case 9: go(std::integral_constant<int, 9>()); break;
+    case 10: go(std::integral_constant<int, 10>()); break;
+    case 11: go(std::integral_constant<int, 11>()); break;
     default: throw Error(SEM_ERR_ARG, "resident CG: unsupported order");
   }
 }
@@ -739,8 +744,7 @@ void launch_resident<double>(sem_handle* h, const PcgVecs<double>& v, int iters,
   }
   a.G = h->f64.G.ptr;
   a.B = h->f64.B.ptr;
-  a.tab = h->f64.D.ptr + h->P * h->P;
-  launch_resident_eo<double>(h, a, s);
+  launch_resident_ieee<double>(h, h->f64.D.ptr, a, s);
 }
 
 template <>
@@ -749,8 +753,7 @@ void launch_resident<float>(sem_handle* h, const PcgVecs<float>& v, int iters, c
   resident_common(h, v, a, iters);
   a.G = h->f32.G.ptr;
   a.B = h->f32.B.ptr;
-  a.tab = h->f32.D.ptr + h->P * h->P;
-  launch_resident_eo<float>(h, a, s);
+  launch_resident_ieee<float>(h, h->f32.D.ptr, a, s);
 }
 
 }  // namespace sem

@@ -447,10 +447,13 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     DevBuf<double> dxi, dwq;
     dxi.alloc(P); dxi.upload(h->xi.data(), P, s);
     dwq.alloc(P); dwq.upload(h->wq.data(), P, s);
-    // D, then the even-odd tables of D and D^T (eo_tile.cuh), in one buffer
-    std::vector<double> D64(h->Dh), eo = eo_tables(P, h->Dh);
-    D64.insert(D64.end(), eo.begin(), eo.end());
-    const std::vector<float> D32(D64.begin(), D64.end());
+    // D; in FP64 the even-odd tables of D and D^T (eo_tile.cuh) behind it
+    std::vector<double> D64(h->Dh);
+    if (eo_split(P, true)) {
+      const std::vector<double> eo = eo_tables(P, h->Dh);
+      D64.insert(D64.end(), eo.begin(), eo.end());
+    }
+    const std::vector<float> D32(h->Dh.begin(), h->Dh.end());
     h->f64.D.alloc(D64.size()); h->f64.D.upload(D64.data(), D64.size(), s);
     h->f32.D.alloc(D32.size()); h->f32.D.upload(D32.data(), D32.size(), s);
 
@@ -500,6 +503,7 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
       SEM_CHECK_LAUNCH();
       df_prepare(h.get());
     }
+    eo_prepare(h.get());
     noalloc_prepare();
     h->dev_err.alloc(1);
     SEM_CUDA(cudaMemsetAsync(h->dev_err.ptr, 0, sizeof(int), s));
