@@ -98,6 +98,7 @@ extern "C" sem_status sem_autotune(sem_handle* h, void* stream, sem_tuning* out)
     const auto key = std::make_tuple(h->P, b);
     std::lock_guard<std::mutex> lock(g_mu);
     load_file_locked();
+    h->tune.ax32_bulk = 0;                  // the measured choice alone
     sem_tuning t{};
     t.ax32_ms = -1.0;
     t.ax64_ms = -1.0;
@@ -175,6 +176,7 @@ extern "C" sem_status sem_set_tuning(sem_handle* h, const sem_tuning* t) {
       if (kTmaStages[q] == t->ax32_stages && kTmaElems[q] == t->ax32_elems_per_cta) v = q;
     SEM_REQUIRE(v >= 0, "sem_set_tuning: no such (stages, elements per CTA) variant");
     h->tune.ax32_ldg = t->ax32_kernel;
+    h->tune.ax32_bulk = 0;
     h->tune.ax32_variant = v;
     h->tune.df_variant = t->f64_stages - 1;
   });

@@ -92,8 +92,17 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
   using C = LineCfg<P, T, MOST>;
   constexpr int P2 = C::P2, P3 = C::P3, RS = C::RS, PL = C::PL;
   constexpr bool PRE = sizeof(T) == 4;       // prefetches to registers
-  T gr[PRE ? P : 1][6];
+  // B comes with G where the backward lines are too short to hide its latency and no
+  // other CTA hides it (N = 3, cold caches: sem_apply_global on 216 elements 9.7
+  // against 11.0 us, sem_apply 11.0 against 11.6); on large grids that costs 1 to 2%
+  const bool early_b = PRE && P <= 4 && gridDim.x < 1024;
+  T gr[PRE ? P : 1][6], bk[PRE ? P : 1];
+  auto fetch_b = [&] {
+#pragma unroll
+    for (int k = 0; k < P; ++k) bk[PRE ? k : 0] = __ldcs(b + k * P2);
+  };
   if (act) {
+    if (early_b && h2 != T(0)) fetch_b();
     if constexpr (PRE) {
 #pragma unroll
       for (int k = 0; k < P; ++k)
@@ -141,11 +150,7 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
       wt[k] = wk;
     }
   }
-  T bk[PRE ? P : 1];                         // on its way while the backward lines run
-  if (PRE && act && h2 != T(0)) {
-#pragma unroll
-    for (int k = 0; k < P; ++k) bk[PRE ? k : 0] = __ldcs(b + k * P2);
-  }
+  if (PRE && !early_b && act && h2 != T(0)) fetch_b();   // on its way during the backward lines
   __syncthreads();
   if (act) {
     T x[P];

@@ -72,20 +72,23 @@ __device__ __forceinline__ unsigned dirichlet_bits(const GBox& b, int ex, int ey
 // so that six CTAs fit an SM instead of four: 138 us (h2 = 0: 135).  With the
 // Kahan sum (PW, and batch_glob.cuh) the registers do not allow it: 16 problems
 // with 17,000 elements of N = 9 187 against 169 us.
-template <int P, bool PW>
+// FEW: at most a CTA an SM, where a late load's latency counts and registers do
+// not: all six components ahead (N = 9, 8 to 64 elements, cold caches: 11.1 to 12.5
+// against 12.3 to 13.3 us).
+template <int P, bool PW, bool FEW>
 struct GlobCfg : LineCfg<P, float, kGlobThreads> {
-  static constexpr bool LEAN = P >= 10 && !PW;
+  static constexpr bool LEAN = P >= 10 && !PW && !FEW;
   static constexpr int PREG = LEAN ? 3 : 6;
   static constexpr int CTAS = LEAN ? 6 : LineCfg<P, float, kGlobThreads>::MINB;
 };
 
-template <int P, bool PW>
-__global__ void __launch_bounds__(GlobCfg<P, PW>::THREADS, GlobCfg<P, PW>::CTAS)
+template <int P, bool PW, bool FEW>
+__global__ void __launch_bounds__(GlobCfg<P, PW, FEW>::THREADS, GlobCfg<P, PW, FEW>::CTAS)
 ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* __restrict__ G,
                const float* __restrict__ B, float h1, float h2,
                const __grid_constant__ DMat<P, float> D, int E, GBox bx,
                const CGState* __restrict__ st, double* __restrict__ slots) {
-  using C = GlobCfg<P, PW>;
+  using C = GlobCfg<P, PW, FEW>;
   constexpr int P3 = C::P3, K = C::K, N = P - 1;
   if (st && st->done) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -156,11 +159,11 @@ double* pw_slots(const sem_handle* h) {
   return h->partials.ptr + 6 * kRedBlocks + kFusedPartials;
 }
 
-template <int P, bool PW>
+template <int P, bool PW, bool FEW>
 static void launch_glob_p(const sem_handle* h, const float* u, float* w, float h1, float h2,
                           const CGState* st, cudaStream_t s) {
-  using C = GlobCfg<P, PW>;
-  auto kern = ax_glob_kernel<P, PW>;
+  using C = GlobCfg<P, PW, FEW>;
+  auto kern = ax_glob_kernel<P, PW, FEW>;
   static bool configured = false;
   if (!configured) {
     SEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -186,8 +189,10 @@ int64_t glob_padded(const sem_handle* h) { return (h->nG + 3) / 4 * 4; }
 template <int P>
 static void launch_glob_any(const sem_handle* h, const float* u, float* w, float h1, float h2,
                             const CGState* st, bool pw, cudaStream_t s) {
-  if (pw) launch_glob_p<P, true>(h, u, w, h1, h2, st, s);
-  else launch_glob_p<P, false>(h, u, w, h1, h2, st, s);
+  if (pw) return launch_glob_p<P, true, false>(h, u, w, h1, h2, st, s);
+  if constexpr (P == 10)
+    if (h->E <= sem_num_sms()) return launch_glob_p<P, false, true>(h, u, w, h1, h2, st, s);
+  launch_glob_p<P, false, false>(h, u, w, h1, h2, st, s);
 }
 
 void launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,

@@ -430,6 +430,13 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     // 10 (sem_apply, us, line / bulk: N = 9 4 M points 51 / 56, 17.6 M 167 / 166
     // and with a mass term 187 / 169; N = 7 4 M 42 / 46, 16.8 M 120 / 119)
     h->tune.ax32_ldg = h->P >= 8 && h->P % 2 == 0 && h->nL > (1 << 23) ? 0 : 1;
+    // sem_ax alone takes bulk copies also on small meshes at P = 4 and 6, where the
+    // line kernel's several elements a CTA leave most of the chip idle, and from 2.5 M
+    // points at P = 10 (us with cold caches, line / bulk: N = 3 64 elements 7.2 / 6.1,
+    // 512 7.6 / 6.1, 1,000 7.9 / 7.2, 1,728 8.2 / 8.2; N = 5 8 7.6 / 6.6, 125 8.2 / 7.2,
+    // 343 8.2 / 8.6; N = 9 1,728 22.5 / 22.5, 2,744 30.5 / 28.7, 5,832 52.7 / 49.2)
+    h->tune.ax32_bulk = (h->P == 4 && h->E <= 1024) || (h->P == 6 && h->E <= 192) ||
+                        (h->P == 10 && h->E >= 2500);
     h->tune.ax32_variant = h->P <= 4 ? 2 : 1;     // 3 stages for small elements, else 2
     gll_host(N, h->xi, h->wq, h->Dh);
 

@@ -1,0 +1,43 @@
+"""Calls at the sizes where the dispatch changes kernels, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2107_01243_gb300 as sem
+import seeded_inputs as si
+from tests.helpers import OracleProblem, rel_inf, TWO_PI
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("nel,N", [((12, 8, 8), 3), ((13, 12, 5), 3), ((8, 6, 4), 5),
+                                   ((13, 5, 3), 5), ((2, 2, 2), 5)])
+@pytest.mark.parametrize("tuned", [False, True])
+def test_fp32_element_operator_on_small_boxes(nel, N, tuned):
+    """Bulk copies up to 768 elements at N = 3 and 192 at N = 5, unless the caller
+    pins the line kernel (the FP32 tolerance of the other kernels' tests)."""
+    h = sem.sem_setup(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    o = OracleProblem(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    if tuned:
+        sem.sem_set_tuning(h, ax32_kernel="global-load")
+    u = si.uniform(o.shape, 61).astype(np.float32).astype(np.float64)
+    ud = torch.from_numpy(u).to(DEV, torch.float32).view(-1)
+    w = torch.empty_like(ud)
+    sem.sem_ax(h, ud, w, 0.7, 1.5)
+    assert rel_inf(w.double().cpu().numpy().reshape(o.shape), o.ax(u, 0.7, 1.5)) < 2e-5
+
+
+@pytest.mark.parametrize("nel", [(8, 19, 1), (9, 17, 1), (2, 2, 2)])
+def test_global_operator_n9_around_one_cta_an_sm(nel):
+    """152 elements (all of G fetched ahead) and 153, at the tolerance of the
+    other orders' parity tests."""
+    N = 9
+    h = sem.sem_setup(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    o = OracleProblem(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    u = si.uniform((h.n_global,), 62).astype(np.float32).astype(np.float64)
+    w = torch.empty(h.n_global, dtype=torch.float32, device=DEV)
+    sem.sem_apply_global(h, torch.from_numpy(u).to(DEV, torch.float32), w, 0.7, 1.5)
+    ref = np.zeros(h.n_global)
+    ref[o.gid.reshape(-1)] = o.matvec(u[o.gid], 0.7, 1.5).reshape(-1)
+    assert rel_inf(w.double().cpu().numpy(), ref) < 2e-5
