@@ -382,9 +382,8 @@ void sem_solve_opts_default(sem_solve_opts* o);
  * relative residual <= tol.  Synchronises the stream once per check_every
  * iterations and at the end.  Problems of at most 2^20 local points iterate
  * inside one cooperative launch (512 iterations between synchronisations;
- * use_graph and check_every have no effect), by recurrences that apply H to
- * the preconditioned residual and agree with standard PCG in exact
- * arithmetic.  Returns SEM_ERR_NOCONV / SEM_ERR_BREAKDOWN
+ * use_graph and check_every have no effect), unless the pipelined variant,
+ * global inner vectors or other multiplicities were asked for.  Returns SEM_ERR_NOCONV / SEM_ERR_BREAKDOWN
  * (with info filled) when the solve fails.
  */
 sem_status sem_cg_solve(sem_handle* h, const double* b_L, double* x_L,

@@ -822,15 +822,7 @@ template <class T>
 static CGState run_pcg(sem_handle* h, const PcgArgs<T>& a, const sem_solve_opts& o,
                        cudaStream_t s) {
   if (resident_ok<T>(h, a.h1f)) {
-    T *vs, *w2;
-    if constexpr (std::is_same<T, double>::value) {
-      ensure(h->res_s, h->nL); ensure(h->res_w2, h->nL);
-      vs = h->res_s.ptr; w2 = h->res_w2.ptr;
-    } else {
-      ensure(h->res_s32, h->nL); ensure(h->res_w232, h->nL);
-      vs = h->res_s32.ptr; w2 = h->res_w232.ptr;
-    }
-    const PcgVecs<T> v{a.x, a.r, a.p, vs, a.w, w2, a.dinv, a.h1f, a.h1, a.h2, a.st};
+    const PcgVecs<T> v{a.x, a.r, a.p, a.w, a.dinv, a.h1f, a.h1, a.h2, a.st};
     CGState hs;
     do {
       launch_resident<T>(h, v, kResidentIters, s);

@@ -4,8 +4,7 @@
 // What bounds small solves is latency: with one kernel per stage an iteration
 // on 4^3 elements (N = 7, FP64) took 38 us in six launches, for about 3 us of
 // arithmetic.  Here the whole grid stays on the GPU (a cooperative launch of
-// at most the resident CTAs).  An iteration of the double-float operator takes
-// two grid barriers:
+// at most the resident CTAs).  An iteration takes two grid barriers:
 //   - p = z + beta p; the element operator; the local products (masked, not
 //     assembled) go to w, and <p, H p> = sum_L p (H_L p) (p is continuous and
 //     zero on Dirichlet points, so the sum over local points is the unique-dof
@@ -13,16 +12,11 @@
 //   - every point gathers the copies of its w (at most eight, summed pair by
 //     pair along x, y, z as sem_apply does), x += alpha p, r -= alpha w,
 //     z = dinv r, <r, z> and <r, r>; barrier, beta
-// The IEEE operators (FP64 and FP32) need only one, by the recurrences of
-// Chronopoulos and Gear (J. Comput. Appl. Math. 25, 1989), in exact arithmetic
-// the same: the operator is applied to z, s = H z + beta s stands for H p, and
-// <p, H p> follows from <z, H z>, so that all three sums meet at the barrier
-// that also publishes w.  Their s accumulates the operator's errors, which is
-// harmless while those are of the size of the vectors' roundings; with the
-// double-float operator (1e-13) it left true residuals 5 to 10 times those of
-// the standard recurrences at tolerances below 1e-11, so that operator keeps
-// two barriers.
-// x, r, p and s of an element are only touched by its own CTA's threads; w
+// (One barrier would do with the recurrences of Chronopoulos and Gear, which
+// form <p, H p> from <z, H z> and s = H p by a recurrence; but they lose digits:
+// FP32 inner solves took 5 to 20% more iterations, and the residual that FP64
+// solves end at was 1% larger, 5 to 10 times with the double-float operator.)
+// x, r and p of an element are only touched by its own CTA's threads; w
 // alone crosses CTAs, and is read past L1.  Every CTA adds the CTAs' sums the
 // same way and steps its own copy of the CGState.  The barrier's wait is
 // bounded: a CTA that gives up records SEM_ERR_TIMEOUT and leaves, and the
@@ -48,7 +42,7 @@ namespace sem {
 
 template <class T>
 struct ResArgs {
-  T *x, *r, *p, *s, *w, *w2;  // L-vectors
+  T *x, *r, *p, *w;           // L-vectors
   const T* dinv;
   const float* imult;
   const void *G, *B;          // T values, or float pairs (double-float operator)
@@ -60,7 +54,7 @@ struct ResArgs {
   FuseBox fb;
   FastDiv dnx, dny;
   CGState* st;
-  longlong2* partials;        // 2 x 3 gridDim.x values
+  longlong2* partials;        // 2 x 2 gridDim.x values
   unsigned* bar;              // zero at launch
   int* err;
   uint64_t timeout_ns;
@@ -76,7 +70,6 @@ struct ResArgs {
 template <int P>
 struct OpDF {
   using T = double;
-  static constexpr bool ONE = false;     // two barriers, the standard recurrences
   using L = DFLayout<P>;
   static constexpr int P2 = P * P, P3 = P2 * P, NT = 3 * P2, NTB = (NT + 31) / 32 * 32;
   static constexpr int NQ = (P3 + NT - 1) / NT, NW = NTB / 32;
@@ -221,7 +214,6 @@ struct OpDF {
 template <int P, class TT>
 struct OpIEEE {
   using T = TT;
-  static constexpr bool ONE = true;      // one barrier
   using L = EoLayout<P, T>;
   static constexpr int P2 = P * P, P3 = P2 * P, NT = 3 * P2, NTB = (NT + 31) / 32 * 32;
   static constexpr int NQ = (P3 + NT - 1) / NT, TS = LineTab<P, T>::SIZE;
@@ -339,7 +331,7 @@ __device__ __forceinline__ T res_widen(float f) {
 // State transitions with the comparisons on the bits of the doubles (an FP64
 // comparison costs as much as an addition); tol2 and <r, r> are not negative.
 
-// standard recurrences (cg_state.cuh): after <p, H p>
+// the recurrences of cg_state.cuh: after <p, H p>
 __device__ __forceinline__ void res_after_pw(CGState* st, double pw) {
   st->pw = pw;
   if (dbits(pw) <= 0 || is_nan(pw)) {
@@ -368,36 +360,6 @@ __device__ __forceinline__ void res_after_update(CGState* st, const double* tot)
   }
 }
 
-// one-barrier recurrences: after <r, z>, <z, H z> and <r, r> (tot) of the
-// current residual, the stop tests, then beta = rz / rz_old, <p, H p> =
-// <z, H z> - beta^2 <p, H p>_old and alpha = rz / <p, H p> of the next update
-__device__ __forceinline__ void res_step(CGState* st, const double* tot) {
-  const bool first = st->iter == 0;
-  st->rr = tot[2];
-  if (is_nan(tot[0]) || is_nan(tot[1]) || is_nan(tot[2])) {
-    st->status = SEM_ERR_BREAKDOWN;
-    st->done = 1;
-  } else if (dbits(tot[2]) <= dbits(st->tol2)) {
-    st->done = 1;
-  } else if (st->iter >= st->maxit) {
-    st->status = SEM_ERR_NOCONV;
-    st->done = 1;
-  } else {
-    const double beta = first ? 0.0 : tot[0] / st->rz;
-    const double pw = fma(-beta * beta, st->pw, tot[1]);
-    st->pw = pw;
-    if (dbits(pw) <= 0) {
-      st->status = SEM_ERR_BREAKDOWN;
-      st->done = 1;
-    } else {
-      st->beta = beta;
-      st->alpha = tot[0] / pw;
-      st->rz = tot[0];
-      st->iter += 1;
-    }
-  }
-}
-
 // RES: every CTA has one element, whose vectors stay in registers.
 template <class OP, bool RES>
 __global__ void __launch_bounds__(OP::NTB)
@@ -408,8 +370,8 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   longlong2* sp = reinterpret_cast<longlong2*>(smem + (OP::SMEM + 15) / 16 * 16);
   __shared__ CGState s_st;
-  __shared__ FxVal s_w[3][16];
-  __shared__ double s_tot[3];
+  __shared__ FxVal s_w[2][16];
+  __shared__ double s_tot[2];
   __shared__ int s_bad;
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -422,27 +384,24 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
   __syncthreads();
   if (s_st.done) return;                 // the same in every CTA
   const int i = tid % P, j = (tid / P) % P, k0 = tid / P2;
-  T x[NQ], r[NQ], p[NQ], s[NQ], d[NQ];   // this thread's points of one element
+  T x[NQ], r[NQ], p[NQ], d[NQ];          // this thread's points of one element
   T z[NQ] = {};                          // dinv r
   float im[NQ];
-  ResAcc<T> rz, zh, rr;
+  ResAcc<T> rz, pw, rr;
 
-  auto load = [&](int e, bool all) {
+  auto load = [&](int e) {
     const size_t base = (size_t)e * P3 + tid;
 #pragma unroll
     for (int m = 0; m < NQ; ++m) {
-      x[m] = r[m] = p[m] = s[m] = d[m] = T(0);
+      x[m] = r[m] = p[m] = d[m] = T(0);
       im[m] = 1.0f;
       if (op.has(m)) {
         const size_t q = base + m * NT;
         r[m] = a.r[q];
         d[m] = __ldg(a.dinv + q);
         im[m] = __ldg(a.imult + q);
-        if (all) {
-          x[m] = a.x[q];
-          p[m] = a.p[q];
-          if (OP::ONE) s[m] = a.s[q];
-        }
+        x[m] = a.x[q];
+        p[m] = a.p[q];
       }
     }
   };
@@ -455,7 +414,6 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
         a.x[q] = x[m];
         a.r[q] = r[m];
         a.p[q] = p[m];
-        if (OP::ONE) a.s[q] = s[m];
       }
   };
   auto dots = [&](int m) {
@@ -463,17 +421,15 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
     rr.add2(rm, r[m]);
     rz.add2(rm, z[m]);
   };
-  // z = dinv r and (ONE) w = H_L z with the dots of this element, else p = z +
-  // beta p and w = H_L p with <p, H p>; w is masked, not assembled
-  auto front = [&](int e, T* w, T beta, bool first) {
-    T hz[NQ];
+  // p = z + beta p and w = H_L p with <p, H p>; w is masked, not assembled
+  auto front = [&](int e, T beta, bool first) {
+    T hp[NQ];
 #pragma unroll
     for (int m = 0; m < NQ; ++m) {
-      if (OP::ONE || !RES) z[m] = d[m] * r[m];   // else left by the last update
-      if (!OP::ONE) p[m] = first ? z[m] : fma(beta, p[m], z[m]);
+      if (!RES) z[m] = d[m] * r[m];              // else left by the last update
+      p[m] = first ? z[m] : fma(beta, p[m], z[m]);
     }
-    T (&v)[NQ] = OP::ONE ? z : p;
-    op.apply(a, e, v, hz);
+    op.apply(a, e, p, hp);
     const uint32_t re = a.dnx.div((uint32_t)e), ez = a.dny.div(re);
     const int ex = e - (int)re * a.fb.nelx, ey = (int)(re - ez * (uint32_t)a.fb.nely);
     const int f = a.fb.faces;
@@ -488,18 +444,18 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
       if (!op.has(m)) break;
       const int k = k0 + 3 * m;
       const bool masked = mij || (mz0 && k == 0) || (mz1 && k == N);
-      w[(size_t)e * P3 + tid + m * NT] = masked ? T(0) : hz[m];
+      a.w[(size_t)e * P3 + tid + m * NT] = masked ? T(0) : hp[m];
     }
 #pragma unroll
     for (int m = 0; m < NQ; ++m) {
       if (!op.has(m)) break;
-      if (OP::ONE) dots(m);
-      zh.add2(v[m], hz[m]);
+      pw.add2(p[m], hp[m]);
     }
   };
-  // gathers the copies of w = H z (summed pair by pair along x, y, z), then
-  // p = z + beta p, s = w + beta s (= H p), x += alpha p, r -= alpha s
-  auto update = [&](int e, const T* w, T alpha, T beta, bool first) {
+  // gathers the copies of w (summed pair by pair along x, y, z), then
+  // x += alpha p, r -= alpha w, z = dinv r and the dots
+  auto update = [&](int e, T alpha) {
+    const T* w = a.w;
     const size_t base = (size_t)e * P3 + tid;
     const uint32_t re = a.dnx.div((uint32_t)e), ez = a.dny.div(re);
     const int ex = e - (int)re * a.fb.nelx, ey = (int)(re - ez * (uint32_t)a.fb.nely);
@@ -544,99 +500,53 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
         }
         v += v4;
       }
-      if constexpr (OP::ONE) {
-        if (!RES) z[m] = d[m] * r[m];    // RES: still there
-        p[m] = first ? z[m] : fma(beta, p[m], z[m]);
-        s[m] = first ? v : fma(beta, s[m], v);
-        x[m] = fma(alpha, p[m], x[m]);
-        r[m] = fma(-alpha, s[m], r[m]);
-      } else {
-        x[m] = fma(alpha, p[m], x[m]);
-        r[m] = fma(-alpha, v, r[m]);
-        z[m] = d[m] * r[m];
-        if (op.has(m)) dots(m);
-      }
+      x[m] = fma(alpha, p[m], x[m]);
+      r[m] = fma(-alpha, v, r[m]);
+      z[m] = d[m] * r[m];
+      if (op.has(m)) dots(m);
     }
   };
 
   const int e0 = blockIdx.x;
   unsigned met = 0;
-  // sums over the grid at the n-th set of partials (at most 3 gridDim.x each)
+  // sums over the grid at the n-th set of partials (at most 2 gridDim.x each)
   auto meet = [&](auto nv, const double* v, int n, auto step) {
     constexpr int NV = decltype(nv)::value;
     double vv[NV];
 #pragma unroll
     for (int q = 0; q < NV; ++q) vv[q] = v[q];
     met += NV * gridDim.x;
-    return grid_dots<NV, NW>(vv, s_w, sp, s_tot, a.partials + n * 3 * gridDim.x, a.bar, met, a.err,
+    return grid_dots<NV, NW>(vv, s_w, sp, s_tot, a.partials + n * 2 * gridDim.x, a.bar, met, a.err,
                              a.timeout_ns, &s_bad, step);
   };
   using One = std::integral_constant<int, 1>;
   using Two = std::integral_constant<int, 2>;
-  using Three = std::integral_constant<int, 3>;
-  if (RES) load(e0, true);
-  if constexpr (OP::ONE) {
-    T *wcur = a.w, *wnext = a.w2;
-    if (RES) {
-      front(e0, wcur, T(0), false);
-    } else {
-      for (int e = e0; e < a.E; e += gridDim.x) {
-        load(e, false);
-        front(e, wcur, T(0), false);
-      }
-    }
-    for (int it = 0; it < a.iters; ++it) {
-      const double v[3] = {rz.value(), zh.value(), rr.value()};
-      rz = ResAcc<T>();
-      zh = ResAcc<T>();
-      rr = ResAcc<T>();
-      // partials alternate: a fast CTA may arrive twice while a slow one reads
-      if (!meet(Three(), v, it & 1, [&] { res_step(&s_st, s_tot); })) break;
-      if (s_st.done) break;
-      const T alpha = (T)s_st.alpha, beta = (T)s_st.beta;
-      const bool first = s_st.iter == 1;
-      if (RES) {
-        update(e0, wcur, alpha, beta, first);
-        front(e0, wnext, T(0), false);
-      } else {
-        for (int e = e0; e < a.E; e += gridDim.x) {
-          load(e, true);
-          update(e, wcur, alpha, beta, first);
-          store(e);
-          front(e, wnext, T(0), false);
-        }
-      }
-      T* t = wcur;                       // w alternates: its copies are read until
-      wcur = wnext;                      // every CTA has arrived once more
-      wnext = t;
-    }
-  } else {
-    for (int it = 0; it < a.iters; ++it) {
-      const T beta = (T)s_st.beta;
-      zh = ResAcc<T>();
-      for (int e = e0; e < a.E; e += gridDim.x) {
-        if (!RES) load(e, true);
-        if (it == 0)                     // a new launch: z of the stored r
+  if (RES) load(e0);
+  for (int it = 0; it < a.iters; ++it) {
+    const T beta = (T)s_st.beta;
+    pw = ResAcc<T>();
+    for (int e = e0; e < a.E; e += gridDim.x) {
+      if (!RES) load(e);
+      if (it == 0)                       // a new launch: z of the stored r
 #pragma unroll
-          for (int m = 0; m < NQ; ++m) z[m] = d[m] * r[m];
-        front(e, a.w, beta, s_st.iter == 0);
-        if (!RES) store(e);
-      }
-      const double v1[1] = {zh.value()};
-      if (!meet(One(), v1, 0, [&] { res_after_pw(&s_st, s_tot[0]); })) break;
-      if (s_st.done) break;
-      const T alpha = (T)s_st.alpha;
-      rz = ResAcc<T>();
-      rr = ResAcc<T>();
-      for (int e = e0; e < a.E; e += gridDim.x) {
-        if (!RES) load(e, true);
-        update(e, a.w, alpha, T(0), false);
-        if (!RES) store(e);
-      }
-      const double v2[2] = {rz.value(), rr.value()};
-      if (!meet(Two(), v2, 1, [&] { res_after_update(&s_st, s_tot); })) break;
-      if (s_st.done) break;
+        for (int m = 0; m < NQ; ++m) z[m] = d[m] * r[m];
+      front(e, beta, s_st.iter == 0);
+      if (!RES) store(e);
     }
+    const double v1[1] = {pw.value()};
+    if (!meet(One(), v1, 0, [&] { res_after_pw(&s_st, s_tot[0]); })) break;
+    if (s_st.done) break;
+    const T alpha = (T)s_st.alpha;
+    rz = ResAcc<T>();
+    rr = ResAcc<T>();
+    for (int e = e0; e < a.E; e += gridDim.x) {
+      if (!RES) load(e);
+      update(e, alpha);
+      if (!RES) store(e);
+    }
+    const double v2[2] = {rz.value(), rr.value()};
+    if (!meet(Two(), v2, 1, [&] { res_after_update(&s_st, s_tot); })) break;
+    if (s_st.done) break;
   }
   if (RES) store(e0);
   if (blockIdx.x == 0 && tid == 0) *a.st = s_st;
@@ -645,7 +555,7 @@ pcg_resident_kernel(const __grid_constant__ ResArgs<typename OP::T> a) {
 // ------------------------------------------------------------ launch
 template <class OP>
 constexpr int resident_smem() {
-  return (int)((OP::SMEM + 15) / 16 * 16 + 3 * kRedBlocks * sizeof(longlong2));
+  return (int)((OP::SMEM + 15) / 16 * 16 + 2 * kRedBlocks * sizeof(longlong2));
 }
 
 template <class OP, bool RES>
@@ -665,10 +575,8 @@ static int resident_occupancy() {
 
 template <class OP>
 static void launch_resident_op(sem_handle* h, ResArgs<typename OP::T>& a, cudaStream_t s) {
-  if (!h->res_bar.ptr) {
-    h->res_bar.alloc(1);
-    h->res_part.alloc(6 * 2 * kRedBlocks);
-  }
+  if (!h->res_bar.ptr) h->res_bar.alloc(1);
+  if (!h->res_part.ptr) h->res_part.alloc(4 * 2 * kRedBlocks);
   a.bar = h->res_bar.ptr;
   a.partials = reinterpret_cast<longlong2*>(h->res_part.ptr);
   SEM_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
@@ -687,7 +595,7 @@ static void launch_resident_op(sem_handle* h, ResArgs<typename OP::T>& a, cudaSt
 
 template <class T>
 static void resident_common(sem_handle* h, const PcgVecs<T>& v, ResArgs<T>& a, int iters) {
-  a.x = v.x; a.r = v.r; a.p = v.p; a.s = v.s; a.w = v.w; a.w2 = v.w2;
+  a.x = v.x; a.r = v.r; a.p = v.p; a.w = v.w;
   a.dinv = v.dinv;
   a.imult = h->imult.ptr;
   a.h1f = v.h1f;

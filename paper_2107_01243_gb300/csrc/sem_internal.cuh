@@ -221,8 +221,6 @@ struct sem_handle {
   // grid-resident CG (resident.cu): its grid barrier and reduction partials
   sem::DevBuf<unsigned> res_bar;
   sem::DevBuf<double> res_part;
-  sem::DevBuf<double> res_s, res_w2;        // its vectors beside r, p, w
-  sem::DevBuf<float> res_s32, res_w232;
   int mult_replaced = 0;                    // sem_set_multiplicity was called
   // host staging for sem_apply_host
   sem::DevBuf<double> stage_in, stage_out;
@@ -288,10 +286,10 @@ void launch_dssum_box(const sem_handle* h, T* w, bool apply_mask, const CGState*
                       cudaStream_t s);
 
 // ---- resident.cu: up to iters PCG iterations of a small problem in one launch
-// (x, r and the state as k_init leaves them; p, s, w, w2 scratch)
+// (x, r and the state as k_init leaves them; p, w scratch)
 template <class T>
 struct PcgVecs {
-  T *x, *r, *p, *s, *w, *w2;
+  T *x, *r, *p, *w;
   const T* dinv;
   const T* h1f;
   T h1, h2;
