@@ -321,19 +321,25 @@ k_pw_v64(int64_t nv, const double2* __restrict__ p, const double2* __restrict__ 
   if (grid_sum<1>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_pw(st, tot[0]);
 }
 
+// x is advanced here, not with the direction as in FP32: the FP64 pipe bounds
+// this kernel, whose loads of x and p are hidden, and HBM the other one (24^3
+// elements, N = 7, us, update and direction: 76 + 35; with the direction 65 + 51).
 __global__ void __launch_bounds__(kRedThreads)
-k_update_v64(int64_t nv, double2* __restrict__ r, const double2* __restrict__ w,
+k_update_v64(int64_t nv, double2* __restrict__ x, double2* __restrict__ r,
+             const double2* __restrict__ p, const double2* __restrict__ w,
              const double2* __restrict__ dmi, const float2* __restrict__ imult,
              CGState* __restrict__ st, double* __restrict__ partials) {
-  if (st_update_skips(st)) return;
+  if (st->done) return;
   const double alpha = st->alpha;
   double rz = 0.0, rr = 0.0;
 #pragma unroll 2
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
        q += (int64_t)gridDim.x * blockDim.x) {
-    double2 rq = r[q];
-    const double2 wq = w[q], dq = dmi[q];
+    double2 xq = x[q], rq = r[q];
+    const double2 pq = p[q], wq = w[q], dq = dmi[q];
     const float2 mq = imult[q];
+    xq.x = fma(alpha, pq.x, xq.x);
+    xq.y = fma(alpha, pq.y, xq.y);
     rq.x = fma(-alpha, wq.x, rq.x);
     rq.y = fma(-alpha, wq.y, rq.y);
     const double sx = rq.x * rq.x, sy = rq.y * rq.y;
@@ -341,12 +347,28 @@ k_update_v64(int64_t nv, double2* __restrict__ r, const double2* __restrict__ w,
     rz = fma(sy, dq.y, rz);
     rr = fma(sx, pow2_widen(mq.x), rr);
     rr = fma(sy, pow2_widen(mq.y), rr);
+    x[q] = xq;
     r[q] = rq;
   }
   double v[2] = {rz, rr};
   double tot[2];
-  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0)
-    st_after_update(st, tot, kXPending);
+  if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_update(st, tot);
+}
+
+__global__ void __launch_bounds__(kRedThreads)
+k_pupd_v64(int64_t nv, double2* __restrict__ p, const double2* __restrict__ r,
+           const double2* __restrict__ dinv, const CGState* __restrict__ st) {
+  if (st->done) return;
+  const double beta = st->beta;
+#pragma unroll 4
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < nv;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    double2 pq = p[q];
+    const double2 rq = r[q], dq = dinv[q];
+    pq.x = dq.x * rq.x + beta * pq.x;
+    pq.y = dq.y * rq.y + beta * pq.y;
+    p[q] = pq;
+  }
 }
 
 template <class T>
@@ -386,16 +408,24 @@ k_pw(int64_t n, const T* __restrict__ p, const T* __restrict__ w, const float* _
   if (grid_sum<1>(v, partials, &st->counter, tot) && threadIdx.x == 0) st_after_pw(st, tot[0]);
 }
 
+// whether x is advanced by the direction's kernel (which reads p anyway): FP32,
+// whose vector kernels HBM bounds; FP64's update kernel has that time to spare
+// (k_update_v64)
+template <class T>
+constexpr bool x_with_direction = sizeof(T) == 4;
+
 template <class T>
 __global__ void __launch_bounds__(kRedThreads)
-k_update(int64_t n, T* __restrict__ r, const T* __restrict__ w, const T* __restrict__ dinv,
-         const float* __restrict__ imult, CGState* __restrict__ st,
-         double* __restrict__ partials) {
-  if (st_update_skips(st)) return;
+k_update(int64_t n, T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
+         const T* __restrict__ w, const T* __restrict__ dinv, const float* __restrict__ imult,
+         CGState* __restrict__ st, double* __restrict__ partials) {
+  constexpr bool XD = x_with_direction<T>;
+  if (XD ? st_update_skips(st) : st->done != 0) return;
   const T alpha = (T)st->alpha;
   Acc<T> a0, a1;
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
+    if (!XD) x[q] += alpha * p[q];
     T rq = r[q] - alpha * w[q];
     r[q] = rq;
     T z = dinv[q] * rq;
@@ -406,7 +436,7 @@ k_update(int64_t n, T* __restrict__ r, const T* __restrict__ w, const T* __restr
   double v[2] = {a0.value(), a1.value()};
   double tot[2];
   if (grid_sum<2>(v, partials, &st->counter, tot) && threadIdx.x == 0)
-    st_after_update(st, tot, kXPending);
+    st_after_update(st, tot, XD ? kXPending : 1);
 }
 
 template <class T>
@@ -419,7 +449,7 @@ k_pupd(int64_t n, T* __restrict__ p, T* __restrict__ x, const T* __restrict__ r,
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n;
        q += (int64_t)gridDim.x * blockDim.x) {
     const T pq = p[q];
-    x[q] += alpha * pq;
+    if (x_with_direction<T>) x[q] += alpha * pq;
     if (done == 0) p[q] = dinv[q] * r[q] + beta * pq;
   }
 }
@@ -687,12 +717,11 @@ static void launch_vec64(sem_handle* h, const PcgArgs<double>& a, bool pw_done, 
     SEM_CHECK_LAUNCH();
   }
   k_update_v64<<<kRedBlocks, kRedThreads, 0, s>>>(
-      nv, (double2*)a.r, (const double2*)a.w, (const double2*)a.dmi,
-      (const float2*)h->imult.ptr, a.st, h->partials.ptr);
+      nv, (double2*)a.x, (double2*)a.r, (const double2*)a.p, (const double2*)a.w,
+      (const double2*)a.dmi, (const float2*)h->imult.ptr, a.st, h->partials.ptr);
   SEM_CHECK_LAUNCH();
-  k_pupd_v<double><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (double2*)a.p, (double2*)a.x,
-                                                      (const double2*)a.r,
-                                                      (const double2*)a.dinv, a.st);
+  k_pupd_v64<<<kRedBlocks, kRedThreads, 0, s>>>(nv, (double2*)a.p, (const double2*)a.r,
+                                                (const double2*)a.dinv, a.st);
   SEM_CHECK_LAUNCH();
 }
 
@@ -704,40 +733,32 @@ static void pcg_iterations(sem_handle* h, const PcgArgs<T>& a, int count, cudaSt
     // the element kernel may take <p, w> and alpha itself (FP32, P = 8)
     const bool pw_done =
         launch_apply<T>(h, *a.op, a.p, a.w, a.h1, a.h2, a.h1f, a.st, SEM_APPLY_FULL, s, a.st);
-    bool done64 = false;
-    if constexpr (std::is_same<T, double>::value) {
-      if (vec && a.dmi) {
-        launch_vec64(h, a, pw_done, s);
-        done64 = true;
-      }
-    }
-    if (done64) continue;
     if (vec) {
-      using V = typename Vec<T>::V;
-      using M = typename Vec<T>::M;
-      const int64_t nv = n / Vec<T>::L;
-      if (!pw_done) {
-        k_pw_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (const V*)a.p, (const V*)a.w,
-                                                     (const M*)h->imult.ptr, a.st,
-                                                     h->partials.ptr);
+      if constexpr (std::is_same<T, double>::value) {
+        launch_vec64(h, a, pw_done, s);
+      } else {
+        const int64_t nv = n / 4;
+        const float4 *p4 = (const float4*)a.p, *w4 = (const float4*)a.w,
+                     *d4 = (const float4*)a.dinv, *m4 = (const float4*)h->imult.ptr;
+        if (!pw_done) {
+          k_pw_v<float><<<kRedBlocks, kRedThreads, 0, s>>>(nv, p4, w4, m4, a.st, h->partials.ptr);
+          SEM_CHECK_LAUNCH();
+        }
+        k_update_v<float><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (float4*)a.r, w4, d4, m4, a.st,
+                                                             h->partials.ptr);
+        SEM_CHECK_LAUNCH();
+        k_pupd_v<float><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (float4*)a.p, (float4*)a.x,
+                                                           (const float4*)a.r, d4, a.st);
         SEM_CHECK_LAUNCH();
       }
-      k_update_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.r, (const V*)a.w,
-                                                       (const V*)a.dinv,
-                                                       (const M*)h->imult.ptr, a.st,
-                                                       h->partials.ptr);
-      SEM_CHECK_LAUNCH();
-      k_pupd_v<T><<<kRedBlocks, kRedThreads, 0, s>>>(nv, (V*)a.p, (V*)a.x, (const V*)a.r,
-                                                     (const V*)a.dinv, a.st);
-      SEM_CHECK_LAUNCH();
     } else {
       if (!pw_done) {
         k_pw<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.p, a.w, h->imult.ptr, a.st,
                                                    h->partials.ptr);
         SEM_CHECK_LAUNCH();
       }
-      k_update<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.r, a.w, a.dinv, h->imult.ptr, a.st,
-                                                     h->partials.ptr);
+      k_update<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.x, a.r, a.p, a.w, a.dinv,
+                                                     h->imult.ptr, a.st, h->partials.ptr);
       SEM_CHECK_LAUNCH();
       k_pupd<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, a.p, a.x, a.r, a.dinv, a.st);
       SEM_CHECK_LAUNCH();
