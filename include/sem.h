@@ -316,8 +316,8 @@ sem_status sem_set_cg_variant(sem_handle* h, int kind);
  * operator; SEM_INNER_GLOBAL on global vectors with sem_apply_global's
  * (a third fewer bytes per vector pass at N = 7, no gather-scatter passes);
  * SEM_INNER_AUTO (the default) takes the global form where it is supported
- * (constant h1, odd N) and the problem has more than 2^20 local points, and
- * the local one elsewhere (small problems iterate inside one launch).  SEM_INNER_GLOBAL on an
+ * (constant h1, odd N) and the problem is too large to iterate inside one
+ * launch (sem_cg_solve), and the local one elsewhere.  SEM_INNER_GLOBAL on an
  * unsupported problem falls back to the local form.  The FP64 outer
  * refinement is the same in all cases.
  */
@@ -380,8 +380,8 @@ void sem_solve_opts_default(sem_solve_opts* o);
  * (FP32 G, B and vectors) inside an FP64 iterative-refinement loop whose
  * residual r = b - Hx and update x += d are FP64.  Stops when the FP64
  * relative residual <= tol.  Synchronises the stream once per check_every
- * iterations and at the end.  Problems of at most 2^20 local points iterate
- * inside one cooperative launch (512 iterations between synchronisations;
+ * iterations and at the end.  Problems of at most 2^20 local points (fewer at low
+ * order: the lines are in csrc/cg.cu) iterate inside one cooperative launch (512 iterations between synchronisations;
  * use_graph and check_every have no effect), unless the pipelined variant,
  * global inner vectors or other multiplicities were asked for.  Returns SEM_ERR_NOCONV / SEM_ERR_BREAKDOWN
  * (with info filled) when the solve fails.

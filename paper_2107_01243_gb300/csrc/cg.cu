@@ -821,17 +821,39 @@ static CGState run_pcg_loop(sem_handle* h, CGState* st, const sem_solve_opts& o,
 static void ensure(DevBuf<double>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
 static void ensure(DevBuf<float>& b, int64_t n) { if (b.n < (size_t)n) b.alloc(n); }
 
-// Whether the grid-resident iterations (resident.cu) run this solve: below
-// about a million local points they win at every order and precision, above
-// it the streaming kernels do (microseconds an iteration, resident / one kernel
-// per stage: 12^3 elements, N = 7, FP64 54.5 / 65.5 and FP32 19.6 / 34.4; 10^3,
-// N = 9, FP64 76.6 / 89.7; 12^3, N = 9, FP64 134.8 / 125.9; 16^3, N = 7, FP64
-// 129.0 / 107.1 and FP32 55.4 / 43.4).
+// Whether the grid-resident iterations (resident.cu) run this solve: up to
+// kResidentPoints local points, and at low order up to so many elements, since a
+// CTA of the resident grid walks its elements one after another, each with the
+// barriers and latencies of its phases.  Microseconds an iteration, resident /
+// staged kernels (FP32 also / staged on global vectors, which SEM_INNER_AUTO takes
+// instead), just below the line and above it:
+//   FP64 double-float  N = 5 4,608 elements 67 / 79, N = 7 2,016 64 / 68, N = 9
+//       1,000 78 / 92 (16^3, N = 7: 129 / 107)
+//   FP64 IEEE  N = 1 2,016 26 / 33, 4,096 34 / 33; N = 2 4,608 41 / 44, 6,480 51 / 48;
+//       N = 3 2,744 46 / 51, 4,096 58 / 55; N = 4 2,016 56 / 62, 2,744 68 / 65; N = 5
+//       2,366 84 / 97, 4,608 153 / 150; N = 6 1,000 76 / 88, 1,452 98 / 89; N = 7
+//       2,016 138 / 165, N = 8 1,331 165 / 176, N = 9 1,000 162 / 175, N = 10 729
+//       186 / 201
+//   FP32  N = 1 2,016 22 / 36 / 24, 4,096 26 / 34 / 22, 8,000 34 / 33 / 21; N = 2
+//       6,480 33 / 34, 9,702 41 / 38; N = 3 1,331 17 / 31 / 20, 2,016 20 / 31 / 20,
+//       8,000 36 / 37 / 24, 11,132 44 / 42 / 30; N = 4 8,000 44 / 48; N = 5 3,332
+//       30 / 42 / 30, 4,608 35 / 45 / 34; N = 6 2,940 36 / 47; N = 7 2,016
+//       31 / 47 / 35; N = 8 1,331 32 / 48; N = 9 704 32 / 43 / 34, 1,000 41 / 47 / 38;
+//       N = 10 729 34 / 51
 constexpr int64_t kResidentPoints = 1 << 20;
+constexpr int kAny = 1 << 30;
+constexpr int kResIeee[kMaxN + 1] = {0, 3000, 4800, 3000, 2200, 2800, 1100, kAny, kAny, kAny, kAny};
+constexpr int kResFp32[kMaxN + 1] = {0, 7000, 7500, 9000, kAny, kAny, kAny, kAny, kAny, kAny, kAny};
+constexpr int kResGlob[kMaxN + 1] = {0, 2400, kAny, 1900, kAny, 3600, kAny, kAny, kAny, 800, kAny};
 
+// or_glob: the alternative is the staged form on global vectors
 template <class T>
-static bool resident_ok(const sem_handle* h, const T* h1f) {
+static bool resident_ok(const sem_handle* h, const T* h1f, bool or_glob = false) {
   if (h->nL > kResidentPoints) return false;
+  const bool df = sizeof(T) == 8 && h->f64_kernel != SEM_F64_KERNEL_NATIVE &&
+                  df_ax_supported(h, nullptr, nullptr, h1f);
+  const int* most = sizeof(T) == 8 ? kResIeee : or_glob ? kResGlob : kResFp32;
+  if (!df && h->E > most[h->N]) return false;
   if (h->mult_replaced) return false;       // its dots count the handle's own copies
   if (sizeof(T) == 8 && h->f64_kernel == SEM_F64_KERNEL_DOUBLEFLOAT &&
       !df_ax_supported(h, nullptr, nullptr, h1f))
@@ -1004,7 +1026,7 @@ static void solve_mixed(sem_handle* h, const double* b, double* x, const sem_sol
   if (!h->f32.G.ptr) throw Error(SEM_ERR_STATE, "mixed solve needs FP32 geometry (SEM_PREC_F32)");
   // AUTO: small problems iterate grid-resident on L-vectors
   const bool glob = h->inner_vectors != SEM_INNER_LOCAL && !o.h1_field && glob_supported(h) &&
-                    !(h->inner_vectors == SEM_INNER_AUTO && resident_ok<float>(h, nullptr));
+                    !(h->inner_vectors == SEM_INNER_AUTO && resident_ok<float>(h, nullptr, true));
   ensure(h->r, n); ensure(h->w, n);
   if (!glob) {
     ensure(h->r32, n); ensure(h->p32, n); ensure(h->w32, n); ensure(h->x32, n);

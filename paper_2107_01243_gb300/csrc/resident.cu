@@ -23,8 +23,8 @@
 // others follow.
 //
 // Microseconds an iteration, resident against one kernel per stage, on 4^3 / 8^3
-// elements: FP64 N = 7 11.3 (38.5) / 23.6 (46.2), N = 6 (IEEE) 13.0 (53.7) /
-// 34.2 (55.3), FP32 N = 7 7.2 (21.6) / 10.8 (25.6).  On 4^3, N = 7, FP64 the
+// elements: FP64 N = 7 11.6 (35.3) / 24.6 (45.2), N = 6 (IEEE) 16.0 (54.7) /
+// 39.2 (57.7), FP32 N = 7 9.7 (20.0 on global vectors) / 15.5 (22.5).  On 4^3, N = 7, FP64 the
 // operator takes 2.3 us, each barrier with its sums 2.5 us (0.45 of them an FP64
 // division), updates and dots on the FP64 pipe 2 us, the copies' reads 1 us.
 // FP64 shuffle trees for the sums (fixsum.cuh says why not) took 3 to 5 us each.

@@ -41,3 +41,22 @@ def test_global_operator_n9_around_one_cta_an_sm(nel):
     ref = np.zeros(h.n_global)
     ref[o.gid.reshape(-1)] = o.matvec(u[o.gid], 0.7, 1.5).reshape(-1)
     assert rel_inf(w.double().cpu().numpy(), ref) < 2e-5
+
+
+@pytest.mark.parametrize("nel,N", [((15, 20, 8), 1), ((15, 20, 11), 1), ((25, 20, 16), 1),
+                                   ((20, 20, 12), 2), ((20, 20, 13), 2), ((25, 20, 16), 2),
+                                   ((19, 10, 10), 3), ((16, 15, 13), 3), ((13, 13, 13), 4),
+                                   ((14, 14, 15), 5), ((11, 10, 10), 6), ((12, 10, 10), 6),
+                                   ((10, 9, 9), 9)])
+@pytest.mark.parametrize("precision", [sem.SEM_SOLVE_F64, sem.SEM_SOLVE_MIXED])
+def test_solves_around_the_resident_limits(nel, N, precision):
+    """Both sides of the element counts where solves stop iterating inside one
+    launch, by order and arithmetic."""
+    h = sem.sem_setup(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    o = OracleProblem(nel, N, length=(TWO_PI,) * 3, deform=0.1)
+    b = o.rhs(si.eval_fourier(si.fourier_modes(31), o.x, o.y, o.z))
+    bd = torch.from_numpy(b).to(DEV).view(-1)
+    x = torch.full_like(bd, float("nan"))
+    info = sem.sem_cg_solve(h, bd, x, h2=0.5, tol=1e-9, precision=precision)
+    res = o.residual(x.cpu().numpy().reshape(o.shape), b, h1=1.0, h2=0.5)
+    assert info["status"] == "SEM_OK" and res <= 1.05e-9
