@@ -266,13 +266,15 @@ k_finish(T* __restrict__ w, int nelx, int nely, int nelz, uint32_t nZ, uint32_t 
   }
 }
 
-// Below this many bytes of w one pass over the shared points takes the place of
+// Up to this many bytes of w one pass over the shared points takes the place of
 // the three: it saves two launches, but its copies across an x-face are
 // scattered writes that cost more than the launches once w no longer sits in
-// the caches (finish alone, us, one pass / three: FP32 N = 7, 0.9 M points 11 / 14,
-// 4.1 M 11 / 15, 16.8 M 30 / 24; FP64 N = 7, 0.9 M 9.5 / 14, 4.1 M 19 / 15, 16.8 M
-// 67 / 38).
-constexpr long long kOnePassBytes = 1 << 24;
+// the caches.  FP32 (finish alone, us, one pass / three): N = 7, 0.9 M points 11 / 14,
+// 4.1 M 11 / 15, 16.8 M 30 / 24.  FP64, whose pass also pays for the adds on the FP64
+// pipe (sem_apply): N = 7, 7.1 MB 31.4 / 32.0, 11.2 MB 44.3 / 43.3, 16.8 MB
+// 61.8 / 59.1; N = 5, 4.7 MB 26.5 / 27.1, 7.1 MB 37.0 / 36.7, 13.8 MB 62.1 / 59.0.
+template <class T>
+constexpr long long kOnePassBytes = sizeof(T) == 8 ? 7 << 20 : 1 << 24;
 
 // the finishing passes on a box of nelx x nely x nelz elements starting at w,
 // after an element kernel with segments of SEG elements
@@ -280,7 +282,7 @@ template <int P, int SEG, class T>
 void finish_box(T* w, int nelx, int nely, int nelz, const CGState* st, cudaStream_t s) {
   const long long layer = (long long)nelx * nely, E = layer * nelz, P2 = P * P;
   const long long nX = nelx > 1 ? ((E + SEG - 1) / SEG - 1) * P2 : 0;
-  if (E * P2 * P * (long long)sizeof(T) <= kOnePassBytes) {
+  if (E * P2 * P * (long long)sizeof(T) <= kOnePassBytes<T>) {
     const long long nZ = layer * (nelz - 1) * P2, nY = (long long)nelx * (nely - 1) * nelz * P2;
     if (nZ + nY + nX == 0) return;
     const int blocks = (int)std::min<long long>((nZ + nY + nX + 255) / 256, 64LL * sem_num_sms());

@@ -60,3 +60,19 @@ def test_solves_around_the_resident_limits(nel, N, precision):
     info = sem.sem_cg_solve(h, bd, x, h2=0.5, tol=1e-9, precision=precision)
     res = o.residual(x.cpu().numpy().reshape(o.shape), b, h1=1.0, h2=0.5)
     assert info["status"] == "SEM_OK" and res <= 1.05e-9
+
+
+@pytest.mark.parametrize("nel,N", [((16, 14, 8), 7), ((17, 14, 8), 7), ((16, 16, 16), 5),
+                                   ((17, 16, 16), 5)])
+def test_fp64_finishing_passes_around_seven_megabytes(nel, N):
+    """One pass up to 7 MB of FP64, three beyond: the sums of sem_ax followed by
+    sem_dssum to their rounding (eight copies: 4e-15 of the largest value)."""
+    h = sem.sem_setup(nel, N, length=(TWO_PI,) * 3, deform=0.1,
+                      faces=sem.SEM_FACE_XMIN | sem.SEM_FACE_ZMAX)
+    u = torch.from_numpy(si.uniform(h.n_local, 63)).to(DEV)
+    w, v = torch.empty_like(u), torch.empty_like(u)
+    sem.sem_apply(h, u, w, 1.0, 0.5)
+    sem.sem_ax(h, u, v, 1.0, 0.5)
+    scale = v.abs().max()
+    sem.sem_dssum(h, v)
+    assert float((w - v).abs().max() / scale) < 4e-15
