@@ -45,7 +45,7 @@ bglob_kernel(const BProb* __restrict__ probs, const int2* __restrict__ groups,
   const size_t base = (size_t)ee * P3 + t.lam;
   line_element(t, act, D, uc, b.G + (size_t)ee * 6 * P3 + t.lam, b.B + base, (const float*)nullptr,
                b.h1, b.h2, out);
-  float pw = 0.0f;
+  float pw = 0.0f, pw_c = 0.0f;            // Kahan-compensated <p, H p>
   if (act) {
     int dst0 = org;                        // the column's addresses are made anew:
     asm volatile("" : "+r"(dst0));         // kept since the gather they would spill
@@ -60,7 +60,6 @@ bglob_kernel(const BProb* __restrict__ probs, const int2* __restrict__ groups,
     const unsigned pij = (t.i == 0 ? 4u : 0u) | (t.i == N ? 8u : 0u) | (t.j == 0 ? 16u : 0u) |
                          (t.j == N ? 32u : 0u);
     float* w = b.wg;
-    float pw_c = 0.0f;                     // Kahan-compensated <p, H p>
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       const float y = __fsub_rn(__fmul_rn(uc[k], out[k]), pw_c);
@@ -76,7 +75,7 @@ bglob_kernel(const BProb* __restrict__ probs, const int2* __restrict__ groups,
         *dst = out[k];
     }
   }
-  const FxVal f = fx_warp_sum((double)pw);
+  const FxVal f = fx_warp_sum(pw, pw_c);
   if ((threadIdx.x & 31) == 0)
     atomicAdd(b.pwacc + (blockIdx.x * NW + (threadIdx.x >> 5)) % kBatchSlots,
               fx_round(f.m >> 32, (long long)(unsigned)f.m, f.e));

@@ -36,6 +36,20 @@ __host__ __device__ inline long long fx_mant(unsigned long long bits, int e) {
   return (bits >> 63) ? -(long long)m : (long long)m;
 }
 
+// a float's biased FP32 exponent (1 for zero and subnormals), and the float on the
+// scale e >= it, truncated: m 2^(e - 183), the same m as fx_mant's of (double)f
+// on the scale e + 896
+__host__ __device__ inline int fx_expf(unsigned f) {
+  const int ex = (int)((f >> 23) & 0xFFu);
+  return ex ? ex : 1;
+}
+__host__ __device__ inline long long fx_mantf(unsigned f, int e) {
+  const int ex = (int)((f >> 23) & 0xFFu), sh = e - (ex ? ex : 1);
+  const unsigned long long w = (unsigned long long)((f & 0x7FFFFFu) | (ex ? 0x800000u : 0u)) << 33;
+  const long long m = sh < 64 ? (long long)(w >> sh) : 0;
+  return (f >> 31) ? -m : m;
+}
+
 // (hi 2^32 + lo) 2^(e - 1079) as a double, lo >= 0: rounded to nearest from its
 // leading 64 bits
 __host__ __device__ inline double fx_round(long long hi, long long lo, int e) {
@@ -113,6 +127,19 @@ __device__ __forceinline__ FxVal fx_warp_sum(double v) {
   FxVal r;
   r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(b));
   r.m = r.e == kFxBad ? 0 : fx_warp_add(fx_mant(b, r.e));
+  return r;
+}
+
+// the same of compensated FP32 sums s - c (the FP64 pipe takes 64 cycles for every
+// conversion)
+__device__ __forceinline__ FxVal fx_warp_sum(float s, float c) {
+  const unsigned us = __float_as_uint(s), uc = __float_as_uint(c);
+  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(fx_expf(us), fx_expf(uc)));
+  FxVal r{0, kFxBad};
+  if (e < 255) {
+    r.e = e + 897;                        // one bit up: both mantissas are below 2^56
+    r.m = fx_warp_add(fx_mantf(us, e + 1) - fx_mantf(uc, e + 1));
+  }
   return r;
 }
 

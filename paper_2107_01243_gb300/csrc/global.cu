@@ -110,12 +110,11 @@ ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* 
   const size_t base = (size_t)(act ? e : 0) * P3 + t.lam;
   line_element<C::PREG>(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam,
                         B + base, (const float*)nullptr, h1, h2, out);
-  float pw = 0.0f;
+  float pw = 0.0f, pw_c = 0.0f;            // Kahan-compensated <p, H p>
   if (act) {
     int dst0 = org;                        // the column's addresses are made anew:
     asm volatile("" : "+r"(dst0));         // kept since the gather they would spill
     const unsigned fl = dirichlet_bits(bx, ex, ey, ez);
-    float pw_c = 0.0f;                     // Kahan-compensated <p, H p>
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       if (PW) {
@@ -135,7 +134,7 @@ ax_glob_kernel(const float* __restrict__ u, float* __restrict__ w, const float* 
   }
   if constexpr (PW) {
     constexpr int NW = C::THREADS / 32;
-    const FxVal f = fx_warp_sum((double)pw);
+    const FxVal f = fx_warp_sum(pw, pw_c);
     if ((threadIdx.x & 31) == 0)
       atomicAdd(slots + (blockIdx.x * NW + (threadIdx.x >> 5)) % kPwSlots,
                 fx_round(f.m >> 32, (long long)(unsigned)f.m, f.e));
