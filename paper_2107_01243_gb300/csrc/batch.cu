@@ -371,25 +371,14 @@ struct KahanF {
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
-// Sums of v over a CTA of 256 threads, in thread 0: in integers (fixsum.cuh; the
-// FP64 shuffle trees of block_sum took 3 to 5 us at the end of every item:
-// bgupdate on 17 M unique points 66 us against 70), or by block_sum where a value is not finite, so that infinities stay infinities.
+// Sums of v over a CTA of 256 threads, in every thread, in integers (fixsum.cuh; the
+// FP64 shuffle trees of block_sum took 3 to 5 us at the end of every item: bgupdate
+// on 17 M unique points 66 us against 70)
 template <int NV>
 __device__ __forceinline__ void item_block_sum(double (&v)[NV]) {
   __shared__ FxVal sw[8];
-  double t[NV];
-  bool bad = false;
 #pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    t[q] = fx_block_total<8>(v[q], sw);
-    bad = bad || __double_as_longlong(t[q]) == 0x7FF8000000000000ll;
-  }
-  if (bad) {                               // the same in every thread
-    block_sum<NV>(v);
-    return;
-  }
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = t[q];
+  for (int q = 0; q < NV; ++q) v[q] = fx_block_total<8>(v[q], sw);
 }
 
 // Stores this item's partial sums; the last item block of the problem returns

@@ -13,16 +13,20 @@ namespace sem {
 
 __host__ __device__ inline int min_int(int a, int b) { return a < b ? a : b; }
 
-// m 2^(e - 1079), e the biased FP64 exponent of the scale; e = kFxBad: Inf or NaN
+// m 2^(e - 1079), e the biased FP64 exponent of the scale (a sum's may exceed
+// 0x7FE: its value need not); e >= kFxInf: not finite
 struct FxVal {
   long long m;
   int e;
 };
-constexpr int kFxBad = 0x7FF;
+// the exponents of values that are not finite, so that the largest of a sum's tells
+// what it is: +Inf, or NaN (-Inf counts as NaN: no sum here survives either)
+constexpr int kFxInf = 0xFFF, kFxBad = 0x1000;
 
 // biased exponent of a double (1 for zero and subnormals)
 __host__ __device__ inline int fx_exp(unsigned long long bits) {
   const int ex = (int)((bits >> 52) & 0x7FF);
+  if (ex == 0x7FF) return bits == 0x7FF0000000000000ull ? kFxInf : kFxBad;
   return ex ? ex : 1;
 }
 
@@ -61,8 +65,8 @@ __host__ __device__ inline double fx_round(long long hi, long long lo, int e) {
     hi = ~hi + (l == 0u ? 1 : 0);
   }
   unsigned long long m = (unsigned long long)hi, bits = neg ? 1ull << 63 : 0ull;
-  if (e >= kFxBad) {
-    bits = 0x7FF8000000000000ull;
+  if (e >= kFxInf) {
+    bits = e == kFxInf ? 0x7FF0000000000000ull : 0x7FF8000000000000ull;
   } else if (m | l) {
     // the leading 64 bits, bit 63 set; ex: the biased exponent of bit 63
 #ifdef __CUDA_ARCH__
@@ -81,7 +85,7 @@ __host__ __device__ inline double fx_round(long long hi, long long lo, int e) {
     const unsigned long long half = (m >> (sh - 1)) & 1ull;
     m = (sh < 64 ? m >> sh : 0ull) + half;   // up to 2^53: the carry moves the exponent
     if (ex == 0) bits |= m;                  // 2^52: the smallest normal number
-    else if (ex >= kFxBad) bits |= 0x7FF0000000000000ull;
+    else if (ex >= 0x7FF) bits |= 0x7FF0000000000000ull;
     else bits |= ((unsigned long long)(ex - 1) << 52) + m;
   }
 #ifdef __CUDA_ARCH__
@@ -126,7 +130,7 @@ __device__ __forceinline__ FxVal fx_warp_sum(double v) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(v);
   FxVal r;
   r.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)fx_exp(b));
-  r.m = r.e == kFxBad ? 0 : fx_warp_add(fx_mant(b, r.e));
+  r.m = r.e >= kFxInf ? 0 : fx_warp_add(fx_mant(b, r.e));
   return r;
 }
 
@@ -135,12 +139,9 @@ __device__ __forceinline__ FxVal fx_warp_sum(double v) {
 __device__ __forceinline__ FxVal fx_warp_sum(float s, float c) {
   const unsigned us = __float_as_uint(s), uc = __float_as_uint(c);
   const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(fx_expf(us), fx_expf(uc)));
-  FxVal r{0, kFxBad};
-  if (e < 255) {
-    r.e = e + 897;                        // one bit up: both mantissas are below 2^56
-    r.m = fx_warp_add(fx_mantf(us, e + 1) - fx_mantf(uc, e + 1));
-  }
-  return r;
+  if (e == 255) return fx_warp_sum((double)s - (double)c);
+  // one bit up: both mantissas are below 2^56
+  return FxVal{fx_warp_add(fx_mantf(us, e + 1) - fx_mantf(uc, e + 1)), e + 897};
 }
 
 // running sum of FxVals by one lane, on a common scale e fixed beforehand:
@@ -166,6 +167,25 @@ __device__ __forceinline__ FxAcc fx_warp_add(const FxAcc& a) {
   t.hi = ((long long)h1 << 27) + (long long)h0;
   return t;
 }
+
+// Sum of the lanes' FxVals, in every lane
+struct FxTot {
+  FxAcc acc;
+  int e;
+};
+__device__ __forceinline__ FxTot fx_lane_sum(FxVal f) {
+  FxTot t;
+  t.e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f.e);
+  if (t.e < kFxInf) t.acc.add(f, t.e);
+  t.acc = fx_warp_add(t.acc);
+  return t;
+}
+// the sum as one FxVal, sh bits to the right so that it fits
+__device__ __forceinline__ longlong2 fx_pack(const FxTot& t, int sh) {
+  return make_longlong2((t.acc.hi << (32 - sh)) + (t.acc.lo >> sh),
+                        t.e < kFxInf ? t.e + sh : t.e);
+}
+
 // sum of v over a CTA of NW warps, in every thread (two barriers; sw: NW entries
 // of shared memory)
 template <int NW>
@@ -175,12 +195,8 @@ __device__ __forceinline__ double fx_block_total(double v, FxVal* sw) {
   __syncthreads();
   if (lane == 0) sw[threadIdx.x >> 5] = f;
   __syncthreads();
-  const FxVal f0 = lane < NW ? sw[lane] : FxVal{0, 1};
-  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f0.e);
-  FxAcc acc;
-  if (e < kFxBad) acc.add(f0, e);
-  acc = fx_warp_add(acc);
-  return fx_round(acc.hi, acc.lo, e);
+  const FxTot t = fx_lane_sum(lane < NW ? sw[lane] : FxVal{0, 1});
+  return fx_round(t.acc.hi, t.acc.lo, t.e);
 }
 #endif
 

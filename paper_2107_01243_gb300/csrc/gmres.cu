@@ -213,13 +213,9 @@ __device__ __forceinline__ void grid_sum_fx(const double (&v)[NV], int cnt, doub
   }
   __syncthreads();
   for (int q = warp; q < cnt; q += NW) {
-    const FxVal f = lane < NW ? sw[q][lane] : FxVal{0, 1};
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f.e);
-    FxAcc acc;
-    if (e < kFxBad) acc.add(f, e);
-    acc = fx_warp_add(acc);
-    if (lane == 0) {
-      __stcg(partials + q * nb + blockIdx.x, make_longlong2((acc.hi << 28) + (acc.lo >> 4), e + 4));
+    const FxTot t = fx_lane_sum(lane < NW ? sw[q][lane] : FxVal{0, 1});
+    if (lane == 0) {                       // at most 8 x 2^62
+      __stcg(partials + q * nb + blockIdx.x, fx_pack(t, 4));
       __threadfence();
     }
   }
@@ -236,7 +232,7 @@ __device__ __forceinline__ void grid_sum_fx(const double (&v)[NV], int cnt, doub
     for (int l = lane; l < nb; l += 32) e = max(e, (unsigned)__ldcg(partials + q * nb + l).y);
     e = __reduce_max_sync(0xffffffffu, e);
     FxAcc acc;
-    if (e < kFxBad)
+    if (e < kFxInf)
       for (int l = lane; l < nb; l += 32) {
         const longlong2 t = __ldcg(partials + q * nb + l);
         acc.add(FxVal{t.x, (int)t.y}, (int)e);

@@ -27,15 +27,9 @@ __device__ __forceinline__ bool grid_dots(const double (&v)[NV], FxVal (*sw)[16]
   }
   __syncthreads();
   for (int q = warp; q < NV; q += NW) {
-    const FxVal f = lane < NW ? sw[q][lane] : FxVal{0, 1};
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f.e);
-    FxAcc acc;
-    if (e < kFxBad) acc.add(f, e);
-    acc = fx_warp_add(acc);
-    // at most 16 x 2^62: 4 bits to the right it fits 63 bits again
-    const long long m = (acc.hi << 28) + (acc.lo >> 4);
-    if (lane == 0) {
-      __stcg(partials + q * nb + blockIdx.x, make_longlong2(m, e + 4));
+    const FxTot t = fx_lane_sum(lane < NW ? sw[q][lane] : FxVal{0, 1});
+    if (lane == 0) {                     // at most 16 x 2^62
+      __stcg(partials + q * nb + blockIdx.x, fx_pack(t, 4));
       asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     }
   }
@@ -67,7 +61,7 @@ __device__ __forceinline__ bool grid_dots(const double (&v)[NV], FxVal (*sw)[16]
     }
     e = __reduce_max_sync(0xffffffffu, e);
     FxAcc acc;
-    if (e < kFxBad)                       // an Inf or NaN was stored as >= kFxBad
+    if (e < kFxInf)
       for (int l = lane; l < nb; l += 32) acc.add(FxVal{mine[l].x, (int)mine[l].y}, (int)e);
     acc = fx_warp_add(acc);
     if (lane == 0) tot[q] = fx_round(acc.hi, acc.lo, (int)e);

@@ -554,33 +554,24 @@ __device__ __forceinline__ double cluster_sum(double v, FxVal* sw, longlong2* sl
   if (lane == 0) sw[threadIdx.x >> 5] = f;
   __syncthreads();
   if (threadIdx.x < 32) {
-    const FxVal f0 = sw[lane];               // NW = 32 warps
-    const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)f0.e);
-    FxAcc acc;
-    if (e < kFxBad) acc.add(f0, e);
-    acc = fx_warp_add(acc);
-    // 32 x 2^62: 5 bits to the right it fits 63 bits again
-    if (lane < kClusterCtas)
-      cluster_put(slots + cluster_rank(), lane,
-                  make_longlong2((acc.hi << 27) + (acc.lo >> 5), e + 5));
+    const FxTot t = fx_lane_sum(sw[lane]);   // NW = 32 warps: at most 32 x 2^62
+    if (lane < kClusterCtas) cluster_put(slots + cluster_rank(), lane, fx_pack(t, 5));
     __syncwarp();
   }
   static_assert(NW == 32, "a lane per warp");
   cluster_barrier();
   if (threadIdx.x >= 32) return 0.0;
   const longlong2 p = lane < kClusterCtas ? slots[lane] : make_longlong2(0, 1);
-  const int e = (int)__reduce_max_sync(0xffffffffu, (unsigned)p.y);
-  FxAcc acc;
-  if (e < kFxBad) acc.add(FxVal{p.x, (int)p.y}, e);
-  acc = fx_warp_add(acc);
-  return fx_round(acc.hi, acc.lo, e);
+  const FxTot t = fx_lane_sum(FxVal{p.x, (int)p.y});
+  return fx_round(t.acc.hi, t.acc.lo, t.e);
 }
 
-// a / b rounded to FP32, for positive normal doubles (an FP64 division takes a
+// a / b rounded to FP32, for positive normal doubles and infinities (an FP64 division takes a
 // lone warp half a microsecond): the significands as pairs of floats, the
 // quotient of the leading parts and its first-order correction (Dekker 1971)
 __device__ __forceinline__ float ratio32(double a, double b) {
   const long long ia = dbits(a), ib = dbits(b);
+  if (max(ia, ib) >= 0x7FF0000000000000ll) return (float)(a / b);
   const long long ma = (ia & 0xFFFFFFFFFFFFFll) | (1ll << 52);
   const long long mb = (ib & 0xFFFFFFFFFFFFFll) | (1ll << 52);
   const float ah = (float)(int)(ma >> 29), al = (float)(int)(ma & 0x1FFFFFFF) * 0x1p-29f;

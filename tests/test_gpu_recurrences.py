@@ -82,3 +82,24 @@ def test_iterations_across_launches(kind):
         assert abs(info["iters"] - ref.iters) <= ref.iters // 50
         info = sem.sem_cg_solve(h, to_dev(b), x, tol=1e-9, maxit=515, raise_on_fail=False, **kw)
         assert info["status"] == "SEM_ERR_NOCONV" and info["iters"] == 515
+
+
+@pytest.mark.parametrize("N", [3, 2])
+def test_right_hand_sides_near_the_largest_double(N):
+    """b whose squares reach 2^1020 and more but whose norm is finite: the solution of
+    a power of two times b, to the bit pattern's scale (products by powers of two are
+    exact).  Few unknowns, so that one square makes up much of the norm."""
+    h = sem.sem_setup((1, 1, 1), N)
+    f = to_dev(si.uniform(h.n_local, 4) + 1.5)
+    b = sem.sem_rhs(h, f, torch.empty_like(f))
+    bb = torch.zeros(1, dtype=torch.float64, device=DEV)
+    sem.sem_dot(h, b, b, bb)
+    k = 511 - int(np.floor(np.log2(float(b.abs().max()))))      # max |b| 2^k in [2^511, 2^512)
+    while float(bb) * 2.0 ** (2 * k - 1000) >= 2.0 ** 24:       # <b, b> stays finite
+        k -= 1
+    assert float(b.abs().max()) ** 2 * 2.0 ** (2 * k - 1000) >= 2.0 ** 20
+    x, y = torch.empty_like(b), torch.empty_like(b)
+    a = sem.sem_cg_solve(h, b, x, tol=1e-9)
+    c = sem.sem_cg_solve(h, b * 2.0 ** k, y, tol=1e-9)
+    assert (a["status"], a["iters"]) == (c["status"], c["iters"]) == ("SEM_OK", a["iters"])
+    assert float((y * 2.0 ** -k - x).abs().max()) <= 1e-12 * float(x.abs().max())
