@@ -89,17 +89,24 @@ ax_line_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__
   }
 }
 
+// once-per-process kernel attributes, set by sem_setup outside any stream capture
+template <int P, class T>
+static void configure_line() {
+  using C = LineCfg<P, T>;
+  static const bool done = [] {
+    for (auto k : {ax_line_kernel<P, T, true>, ax_line_kernel<P, T, false>})
+      SEM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
+    return true;
+  }();
+  (void)done;
+}
+
 template <int P, class T>
 static void launch_line_p(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2,
                           const T* h1f, bool fuse, const CGState* st, cudaStream_t s) {
   using C = LineCfg<P, T>;
   auto kern = fuse ? ax_line_kernel<P, T, true> : ax_line_kernel<P, T, false>;
-  static bool configured = false;
-  if (!configured) {
-    for (auto k : {ax_line_kernel<P, T, true>, ax_line_kernel<P, T, false>})
-      SEM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-    configured = true;
-  }
+  configure_line<P, T>();
   DMat<P, T> D;
   for (int a = 0; a < P * P; ++a) D.d[a] = (T)h->Dh[a];
   const int E = (int)h->E;
@@ -130,6 +137,24 @@ void launch_ax_line(const sem_handle* h, const OpData<T>& op, const T* u, T* w, 
     }
   }
   throw Error(SEM_ERR_ARG, "launch_ax_line: unsupported order");
+}
+
+void line_prepare(const sem_handle* h) {
+  if (h->P == 8) configure_line<8, double>();
+  if (h->P == 10) configure_line<10, double>();
+  if (!h->f32.G.ptr) return;
+  switch (h->P) {
+    case 2: return configure_line<2, float>();
+    case 3: return configure_line<3, float>();
+    case 4: return configure_line<4, float>();
+    case 5: return configure_line<5, float>();
+    case 6: return configure_line<6, float>();
+    case 7: return configure_line<7, float>();
+    case 8: return configure_line<8, float>();
+    case 9: return configure_line<9, float>();
+    case 10: return configure_line<10, float>();
+    case 11: return configure_line<11, float>();
+  }
 }
 
 template void launch_ax_line<float>(const sem_handle*, const OpData<float>&, const float*, float*,

@@ -659,15 +659,16 @@ static int bapply_occupancy(int ncls) {
   return occ;
 }
 
+// (set by sem_batch_create, outside any stream capture)
+template <int P>
+static void bglob_configure() {
+  SEM_CUDA(cudaFuncSetAttribute(bglob_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)LineCfg<P, float, kGlobThreads>::SMEM));
+}
+
 template <int P>
 static void launch_bglob(sem_batch* bt, cudaStream_t s) {
   using C = LineCfg<P, float, kGlobThreads>;
-  static bool configured = false;
-  if (!configured) {
-    SEM_CUDA(cudaFuncSetAttribute(bglob_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)C::SMEM));
-    configured = true;
-  }
   DMat<P, float> D;
   for (const sem_handle* h : bt->hs)
     if (h->P == P) {
@@ -947,6 +948,13 @@ extern "C" sem_status sem_batch_create(sem_handle* const* handles, int n, sem_ba
       bt->gitem_prob.upload(gitem_prob.data(), gitem_prob.size(), nullptr);
       for (int P = 2; P <= kMaxP; P += 2) {
         if (!bt->ncls[P]) continue;
+        switch (P) {
+          case 2: bglob_configure<2>(); break;
+          case 4: bglob_configure<4>(); break;
+          case 6: bglob_configure<6>(); break;
+          case 8: bglob_configure<8>(); break;
+          default: bglob_configure<10>(); break;
+        }
         const int K = line_elems(P, false, kGlobThreads);
         std::vector<int2> groups;
         for (int p = 0; p < n; ++p)

@@ -159,16 +159,22 @@ double* pw_slots(const sem_handle* h) {
 }
 
 template <int P, bool PW, bool FEW>
+static void configure_glob() {
+  static const bool done = [] {
+    SEM_CUDA(cudaFuncSetAttribute(ax_glob_kernel<P, PW, FEW>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)GlobCfg<P, PW, FEW>::SMEM));
+    return true;
+  }();
+  (void)done;
+}
+
+template <int P, bool PW, bool FEW>
 static void launch_glob_p(const sem_handle* h, const float* u, float* w, float h1, float h2,
                           const CGState* st, cudaStream_t s) {
   using C = GlobCfg<P, PW, FEW>;
   auto kern = ax_glob_kernel<P, PW, FEW>;
-  static bool configured = false;
-  if (!configured) {
-    SEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)C::SMEM));
-    configured = true;
-  }
+  configure_glob<P, PW, FEW>();
   DMat<P, float> D;
   for (int a = 0; a < P * P; ++a) D.d[a] = (float)h->Dh[a];
   const int E = (int)h->E;
@@ -192,6 +198,25 @@ static void launch_glob_any(const sem_handle* h, const float* u, float* w, float
   if constexpr (P == 10)
     if (h->E <= sem_num_sms()) return launch_glob_p<P, false, true>(h, u, w, h1, h2, st, s);
   launch_glob_p<P, false, false>(h, u, w, h1, h2, st, s);
+}
+
+template <int P>
+static void configure_glob_any() {
+  configure_glob<P, true, false>();
+  configure_glob<P, false, false>();
+  if constexpr (P == 10) configure_glob<P, false, true>();
+}
+
+// once-per-process kernel attributes, set by sem_setup outside any stream capture
+void glob_kernel_prepare(const sem_handle* h) {
+  if (!h->f32.G.ptr) return;
+  switch (h->P) {
+    case 2: return configure_glob_any<2>();
+    case 4: return configure_glob_any<4>();
+    case 6: return configure_glob_any<6>();
+    case 8: return configure_glob_any<8>();
+    case 10: return configure_glob_any<10>();
+  }
 }
 
 void launch_apply_global(const sem_handle* h, const float* u, float* w, float h1, float h2,

@@ -560,16 +560,15 @@ constexpr int resident_smem() {
 
 template <class OP, bool RES>
 static int resident_occupancy() {
-  static int occ = 0;
-  if (!occ) {
+  static const int occ = [] {
     auto kern = pcg_resident_kernel<OP, RES>;
     SEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   resident_smem<OP>()));
     int o = 0;
     SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, OP::NTB,
                                                            resident_smem<OP>()));
-    occ = std::max(1, std::min(o, kRedBlocks / sem_num_sms()));
-  }
+    return std::max(1, std::min(o, kRedBlocks / sem_num_sms()));
+  }();
   return occ;
 }
 

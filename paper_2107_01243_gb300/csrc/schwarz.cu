@@ -944,13 +944,12 @@ namespace {
 
 // threads a grid of resident CTAs of the one-launch coarse CG has
 int64_t coarse_cg_threads() {
-  static int occ = 0;
-  if (!occ) {
+  static const int occ = [] {
     const int smem = kCoarseBlocks * (int)sizeof(longlong2);
     int o = 0;
     SEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_coarse_cg, kCoarseThreads, smem));
-    occ = std::max(1, o);
-  }
+    return std::max(1, o);
+  }();
   return (int64_t)std::min(kCoarseBlocks, occ * sem_num_sms()) * kCoarseThreads;
 }
 

@@ -511,6 +511,8 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
       df_prepare(h.get());
     }
     eo_prepare(h.get());
+    line_prepare(h.get());
+    glob_kernel_prepare(h.get());
     noalloc_prepare();
     h->dev_err.alloc(1);
     SEM_CUDA(cudaMemsetAsync(h->dev_err.ptr, 0, sizeof(int), s));
