@@ -166,10 +166,11 @@ sem_status sem_sync(sem_handle* h, void* stream);
 /*
  * sem_selftest_timeout -- diagnostic: launches the bulk-copy Ax kernel with
  * an mbarrier that expects 16 bytes more than its copies deliver, so its
- * wait can never complete, with the given limit (0 < timeout_ms <= 2000).
- * Returns SEM_ERR_TIMEOUT when the kernel gave up, recorded the failure and
- * returned (the GPU context stays usable); SEM_OK would mean the wait was
- * not bounded.  Needs FP32 geometry and even N+1.
+ * wait can never complete, then the coarse solve's cooperative kernel with a
+ * grid barrier one arrival short, each with the given limit
+ * (0 < timeout_ms <= 2000).  Returns SEM_ERR_TIMEOUT when both gave up,
+ * recorded the failure and returned (the second with NaN for its solution;
+ * the GPU context stays usable); SEM_OK would mean a wait was not bounded.  Needs FP32 geometry and even N+1.
  */
 sem_status sem_selftest_timeout(sem_handle* h, double timeout_ms, void* stream);
 

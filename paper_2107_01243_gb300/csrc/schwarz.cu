@@ -459,6 +459,10 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
     s_bad = 0;
     s_stop = 0;
   }
+  // a wait ran out (recorded in err): no earlier call's solution is left in x
+  auto give_up = [&] {
+    if (act) a.x[v] = __int_as_float(0x7FC00000);
+  };
   unsigned met = 0;
   float *pold = a.p0, *pnew = a.p1;
   {
@@ -470,7 +474,7 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
                             s_beta = 0.0f;
                             s_stop = dbits(s_tot[0]) <= 0 || is_nan(s_tot[0]);
                           }))
-      return;
+      return give_up();
   }
   for (int it = 0; it < a.iters && !s_stop; ++it) {
     const float beta = s_beta;
@@ -497,7 +501,7 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
                             s_stop = dbits(s_tot[0]) <= 0 || is_nan(s_tot[0]);
                             s_alpha = s_stop ? 0.0f : (float)(s_rz / s_tot[0]);
                           }))
-      return;
+      return give_up();
     if (s_stop) break;
     x = fmaf(s_alpha, p, x);
     r = fmaf(-s_alpha, w, r);
@@ -512,7 +516,7 @@ k_coarse_cg(const __grid_constant__ CoarseArgs a) {
                             s_beta = s_stop ? 0.0f : (float)(s_tot[0] / s_rz);
                             s_rz = s_tot[0];
                           }))
-      return;
+      return give_up();
     float* t = pold;
     pold = pnew;
     pnew = t;
@@ -1023,6 +1027,51 @@ void launch_coarse_cg(sem_schwarz* sw, cudaStream_t s) {
   SEM_CUDA(cudaLaunchCooperativeKernel(k_coarse_cg, dim3(grid), dim3(kCoarseThreads), args,
                                        grid * sizeof(longlong2), s));
 }
+
+}  // namespace
+
+// the one-launch coarse CG of 2^3 vertices with a grid barrier that starts one
+// arrival short, so that its first wait runs out; whether it gave up, recorded
+// SEM_ERR_TIMEOUT in the handle's word and left NaN in its solution
+bool selftest_coarse_timeout(const sem_handle* h, uint64_t timeout_ns, cudaStream_t s) {
+  constexpr int nv = 8;
+  DevBuf<float> f;                         // stencil, then dinv, r, x, p0, p1, z
+  DevBuf<double> part;
+  DevBuf<unsigned> bar;
+  f.alloc(27 * nv + 6 * nv);
+  part.alloc(4);
+  bar.alloc(1);
+  SEM_CUDA(cudaMemsetAsync(f.ptr, 0, f.n * sizeof(float), s));
+  SEM_CUDA(cudaMemsetAsync(bar.ptr, 0xFF, sizeof(unsigned), s));
+  CoarseArgs a{};
+  float* v = f.ptr + 27 * nv;
+  a.st = f.ptr;
+  a.dinv = v;
+  a.r = v + nv;
+  a.x = v + 2 * nv;
+  a.p0 = v + 3 * nv;
+  a.p1 = v + 4 * nv;
+  a.z = v + 5 * nv;
+  a.partials = reinterpret_cast<longlong2*>(part.ptr);
+  a.bar = bar.ptr;
+  a.err = h->dev_err.ptr;
+  a.timeout_ns = timeout_ns;
+  a.nvx = a.nvy = a.nvz = 2;
+  a.iters = 10;
+  void* args[] = {&a};
+  SEM_CUDA(cudaLaunchCooperativeKernel(k_coarse_cg, dim3(1), dim3(kCoarseThreads), args,
+                                       sizeof(longlong2), s));
+  float x[nv];
+  int err = 0;
+  SEM_CUDA(cudaMemcpyAsync(x, a.x, sizeof(x), cudaMemcpyDeviceToHost, s));
+  SEM_CUDA(cudaMemcpyAsync(&err, h->dev_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
+  SEM_CUDA(cudaStreamSynchronize(s));
+  bool nan = true;
+  for (float q : x) nan = nan && std::isnan(q);
+  return err == (int)SEM_ERR_TIMEOUT && nan;
+}
+
+namespace {
 
 // the local solves of rg added into zg (zeroed here), the coarse restriction
 // and the coarse CG; returns the coarse solution or NULL (no coarse level)

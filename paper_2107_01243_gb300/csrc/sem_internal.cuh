@@ -364,6 +364,7 @@ void schwarz_apply(sem_schwarz* sw, const double* r, double* z, cudaStream_t s);
 // z_g = M^-1 r_g on FP32 global vectors (z_g padded like r_g; padding stays zero)
 void schwarz_apply_global(sem_schwarz* sw, const float* r_g, float* z_g, cudaStream_t s);
 sem_handle* schwarz_handle(const sem_schwarz* sw);
+bool selftest_coarse_timeout(const sem_handle* h, uint64_t timeout_ns, cudaStream_t s);
 
 // ---- grad.cu
 void launch_grad(const sem_handle* h, const double* u, const double* lam, double* g,

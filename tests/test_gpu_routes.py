@@ -76,3 +76,24 @@ def test_fp64_finishing_passes_around_seven_megabytes(nel, N):
     scale = v.abs().max()
     sem.sem_dssum(h, v)
     assert float((w - v).abs().max() / scale) < 4e-15
+
+
+def test_bounded_waits_run_out_and_later_solves_are_clean():
+    """The self-test's grid barrier is one arrival short: the coarse solve's kernel
+    gives up after 20 ms, records it and leaves NaN in its solution (the self-test
+    says SEM_OK otherwise).  Solves on the handle, in one launch and with the
+    preconditioner, go on as before."""
+    h = sem.sem_setup((4, 3, 3), 7, length=(TWO_PI,) * 3, deform=0.1)
+    f = torch.from_numpy(si.uniform(h.n_local, 64)).to(DEV)
+    b = sem.sem_rhs(h, f, torch.empty_like(f))
+    m = sem.sem_schwarz_create(h)
+    before = torch.empty_like(b)
+    sem.sem_cg_solve(h, b, before, tol=1e-9)
+    assert sem.sem_selftest_timeout(h, 20.0) == "SEM_ERR_TIMEOUT"
+    sem.sem_sync(h)
+    after = torch.empty_like(b)
+    assert sem.sem_cg_solve(h, b, after, tol=1e-9)["status"] == "SEM_OK"
+    assert torch.equal(before, after)
+    info = sem.sem_gmres_solve(h, b, after, tol=1e-9, restart=10, precond=m,
+                               precision=sem.SEM_SOLVE_MIXED)
+    assert info["status"] == "SEM_OK" and info["rel_res"] <= 1e-9
