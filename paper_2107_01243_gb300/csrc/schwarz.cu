@@ -138,8 +138,8 @@ template <int PE>
 struct SwLayout {
   static constexpr int R = (PE + 3) / 4 * 4;
   static constexpr int TAB = 2 * PE * R + R;         // one (d, v) table
-  static constexpr int ALL = 12 * TAB;               // then 1 / (h1 (lx + ly + lz) + h2) of
-                                                     // the interior element, [c][b][a]
+  static constexpr int ALL = 12 * TAB;               // then h1 (lx + ly + lz) + h2 of the
+                                                     // interior element, [c][b][a]
 };
 
 struct SwParams {
@@ -208,7 +208,7 @@ __device__ __forceinline__ void sw_line(const SwConst<PE>& k, bool interior, con
 // The kernel is bound by issue and by the latency of its line phases: S as
 // constant operands (an interior direction reads no table: the persistent form
 // with all tables in shared memory spent three 16-byte reads on every output),
-// the interior scaling as a table of reciprocals, and one element a CTA, so
+// the interior scaling's divisors as a table, and one element a CTA, so
 // that tables that are not used are not loaded and the registers allow twice
 // the CTAs.  13,824 elements, N = 7: 91 us (160 before).
 template <int PE>
@@ -243,7 +243,7 @@ schwarz_local_kernel(const float* __restrict__ rg, float* __restrict__ zg,
   for (int c = 0; c < R; ++c)
     col[c] = (c < PE && colkeep && ((kz >> c) & 1u)) ? __ldg(rg + cbase + prm.sk * c) : 0.0f;
   // the tables of the directions that are not interior; the eigenvalues unless
-  // the whole element is interior (then the reciprocals serve)
+  // the whole element is interior (then the divisors serve)
   const bool inner = (vk[0] | vk[1] | vk[2]) == 0;
   if (!inner) {
 #pragma unroll
@@ -330,9 +330,9 @@ schwarz_local_kernel(const float* __restrict__ rg, float* __restrict__ zg,
     for (int b = 0; b < R; ++b) x[b] = b < PE ? yl[b * R] : 0.0f;
     sw_line<PE, 1, true>(kst, vk[1] == 0, tab[1], x, [&](int b, float v) { y[b] = v; });
     if (inner) {
-      const float* inv = tab_g + L::ALL + cb * PE2 + ca;     // 1 / (h1 (lx + ly + lz) + h2)
+      const float* den = tab_g + L::ALL + cb * PE2 + ca;     // h1 (lx + ly + lz) + h2
 #pragma unroll
-      for (int b = 0; b < PE; ++b) y[b] *= __ldg(inv + b * PE);
+      for (int b = 0; b < PE; ++b) y[b] /= __ldg(den + b * PE);
     } else {
       const float lac = tab[0][2 * PE * R + ca] + tab[2][2 * PE * R + cb];
 #pragma unroll
@@ -893,7 +893,7 @@ void build_tables(sem_schwarz* sw, std::vector<float>& out) {
   for (int c = 0; c < Pe; ++c)
     for (int b = 0; b < Pe; ++b)
       for (int a = 0; a < Pe; ++a)
-        out.push_back(1.0f / (h1 * (lam0(0, a) + lam0(2, c) + lam0(1, b)) + h2));
+        out.push_back(std::fma(h1, lam0(0, a) + lam0(2, c) + lam0(1, b), h2));
 }
 
 int64_t coarse_cg_threads();
