@@ -594,7 +594,9 @@ struct sem_batch {
   // inner solves on global vectors (every handle allows it): per class the
   // element offsets of its problems, the global vector items
   bool glob = false;
-  DevBuf<int2> cls_groups[kMaxP + 1];       // (problem, first element) of every CTA
+  DevBuf<int2> cls_groups[kMaxP + 1];       // (problem, first element) of every CTA: of
+  long long ngroups[kMaxP + 1] = {};        // all problems at first, later (set_groups) of
+                                            // those still running
   DevBuf<int> gitem_prob;
   DevBuf<double> pwacc;                  // per problem
   int ngitems = 0;
@@ -666,6 +668,32 @@ static void bglob_configure() {
                                 (int)LineCfg<P, float, kGlobThreads>::SMEM));
 }
 
+// CTAs of problem p's elements in its class's launch
+static long long group_count(const BProb& b) {
+  const int K = line_elems(b.P, false, kGlobThreads);
+  return (b.E + K - 1) / K;
+}
+
+// the element launches' CTAs: those of the problems that run(p) names
+template <class F>
+static long long set_groups(sem_batch* bt, cudaStream_t s, F run) {
+  long long total = 0;
+  for (int P = 2; P <= kMaxP; P += 2) {
+    if (!bt->ncls[P]) continue;
+    const int K = line_elems(P, false, kGlobThreads);
+    std::vector<int2> groups;
+    for (int p = 0; p < (int)bt->hs.size(); ++p)
+      if (bt->hp[p].P == P && run(p))
+        for (int e = 0; e < bt->hp[p].E; e += K) groups.push_back(make_int2(p, e));
+    if (bt->cls_groups[P].n < groups.size()) bt->cls_groups[P].alloc(groups.size());
+    if (!groups.empty()) bt->cls_groups[P].upload(groups.data(), groups.size(), s);
+    bt->ngroups[P] = (long long)groups.size();
+    total += bt->ngroups[P];
+    SEM_CUDA(cudaStreamSynchronize(s));      // the host copy goes
+  }
+  return total;
+}
+
 template <int P>
 static void launch_bglob(sem_batch* bt, cudaStream_t s) {
   using C = LineCfg<P, float, kGlobThreads>;
@@ -675,7 +703,8 @@ static void launch_bglob(sem_batch* bt, cudaStream_t s) {
       for (int a = 0; a < P * P; ++a) D.d[a] = (float)h->Dh[a];
       break;
     }
-  bglob_kernel<P><<<(unsigned)bt->cls_groups[P].n, C::THREADS, C::SMEM, s>>>(
+  if (bt->ngroups[P] == 0) return;
+  bglob_kernel<P><<<(unsigned)bt->ngroups[P], C::THREADS, C::SMEM, s>>>(
       bt->probs.ptr, bt->cls_groups[P].ptr, D);
   SEM_CHECK_LAUNCH();
 }
@@ -955,14 +984,8 @@ extern "C" sem_status sem_batch_create(sem_handle* const* handles, int n, sem_ba
           case 8: bglob_configure<8>(); break;
           default: bglob_configure<10>(); break;
         }
-        const int K = line_elems(P, false, kGlobThreads);
-        std::vector<int2> groups;
-        for (int p = 0; p < n; ++p)
-          if (bt->hp[p].P == P)
-            for (int e = 0; e < bt->hp[p].E; e += K) groups.push_back(make_int2(p, e));
-        bt->cls_groups[P].alloc(groups.size());
-        bt->cls_groups[P].upload(groups.data(), groups.size(), nullptr);
       }
+      set_groups(bt.get(), nullptr, [](int) { return true; });
     }
     bt->d_off.alloc(n);
     bt->d_off.upload(d_off.data(), n, nullptr);
@@ -1058,8 +1081,13 @@ extern "C" sem_status sem_batch_solve(sem_batch* bt, const double* const* b_L,
     std::vector<int> phase(n, RUNNING), iters(n, 0), outer(n, 0), status(n, SEM_ERR_NOCONV);
     std::vector<double> rel(n, 0.0);
     const int batch_it = std::max(1, o.check_every);
-    cudaGraphExec_t exec = nullptr;
-    if (o.use_graph) {
+    auto running = [&](int p) { return phase[p] == RUNNING; };
+    long long launched = bt->glob ? set_groups(bt, own, running) : 0;
+    cudaGraphExec_t& exec = cleanup.ex;
+    auto capture = [&] {
+      if (!o.use_graph) return;
+      if (exec) SEM_CUDA(cudaGraphExecDestroy(exec));
+      exec = nullptr;
       cudaGraph_t graph = nullptr;
       SEM_CUDA(cudaStreamBeginCapture(own, cudaStreamCaptureModeThreadLocal));
       try {
@@ -1073,8 +1101,7 @@ extern "C" sem_status sem_batch_solve(sem_batch* bt, const double* const* b_L,
       cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
       cudaGraphDestroy(graph);
       SEM_CUDA(e);
-      cleanup.ex = exec;
-    }
+    };
     SEM_CUDA(cudaMemsetAsync(bt->tickets.ptr, 0, n * sizeof(unsigned), own));
     // FP64 residual of problem p; starts its next inner solve unless it is finished
     auto refine = [&](int p) {
@@ -1110,10 +1137,25 @@ extern "C" sem_status sem_batch_solve(sem_batch* bt, const double* const* b_L,
     };
     for (int p = 0; p < n; ++p) refine(p);
     std::vector<CGState> st(n);
+    bool captured = false;
     for (long guard = 0;; ++guard) {
+      long long live = 0;
       bool any = false;
-      for (int p = 0; p < n; ++p) any = any || phase[p] == RUNNING;
+      for (int p = 0; p < n; ++p)
+        if (running(p)) {
+          any = true;
+          if (bt->glob) live += group_count(bt->hp[p]);
+        }
       if (!any) break;
+      // CTAs of finished problems only start and leave, but 116,000 of them took as
+      // long (55 us) as all else of an iteration on 216 running elements: they are
+      // left out of the launches whenever they are half of them or more
+      if (bt->glob && 2 * live <= launched) {
+        launched = set_groups(bt, own, running);
+        captured = false;
+      }
+      if (!captured) capture();
+      captured = true;
       if (guard > 10000000L) throw Error(SEM_ERR_NOCONV, "sem_batch_solve: iteration guard");
       if (exec) SEM_CUDA(cudaGraphLaunch(exec, own));
       else
