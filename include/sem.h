@@ -225,8 +225,9 @@ sem_status sem_set_f64_kernel(sem_handle* h, int kind);
 
 /* Tile chosen by sem_autotune (times in ms per Ax launch, -1 if not timed). */
 typedef struct {
-  int ax32_kernel;          /* FP32 Ax: 0 bulk-copy (TMA) pipeline, 1 global-load (line) kernel,
-                               the default */
+  int ax32_kernel;          /* FP32 Ax: 0 bulk-copy (TMA) pipeline, 1 global-load (line) kernel;
+                               without tuning 1, but 0 at N = 7 and 9 above 2^23 points
+                               and, for sem_ax alone, on some smaller meshes (setup.cu) */
   int ax32_stages;          /* bulk-copy stages in flight per CTA (1..3) */
   int ax32_elems_per_cta;   /* elements per CTA of the bulk-copy kernel (1 or 2) */
   int f64_stages;           /* double-float FP64 Ax: bulk-copy stages (1 or 2) */

@@ -6,14 +6,19 @@
 // (e + nelx nely).  Summing the x-pairs, then the y-pairs, then the z-pairs
 // gives every copy the sum of all its copies (2, 4 or 8).
 //
-//   local   the element kernel walks segments of kFuseSeg consecutive elements
-//           per CTA and sums the x-pairs inside a segment itself (the upper
-//           element reads back the copy the lower one stored just before);
-//           masked points are written as zero
-//   finish  k_sx_cut: x-pairs between segments;
+//   local   the element kernel sums the x-pairs inside a segment of consecutive
+//           elements itself (streaming kernels: kFuseSeg elements a CTA walks, the
+//           upper one reading back the copy the lower one stored just before; the
+//           line kernel: the elements of a CTA, through shared memory); masked
+//           points are written as zero
+//   finish  small vectors: k_finish, all remaining pairs in one pass; else
+//           k_sx_cut: x-pairs between segments;
 //           k_sy, k_sz: the y- and z-pairs, each a coalesced sweep over the
 //           j = N / k = N planes of the elements and their neighbours' j = 0 /
 //           k = 0 planes
+//
+// IEEE FP64 but for large meshes at N = 7 and 9: the element kernel of sem_ax, then
+// the gather-scatter of sem_dssum.
 //
 // The x-face copies are 8-byte values 64 bytes apart (P = 8), so a separate
 // gather-scatter spends a 32-byte sector on each; here they never leave the

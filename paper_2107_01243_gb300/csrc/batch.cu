@@ -21,7 +21,8 @@
 //   bpw, bupdate, bpupd  vector updates over fixed-size chunks; the chunk
 //           partial sums of one problem are reduced by the last chunk block to
 //           finish (a ticket per problem)
-// Converged problems are skipped by every stage.  A batch of iterations is
+// Converged problems are skipped by every stage (and leave the element launches
+// on global vectors altogether, set_groups).  A batch of iterations is
 // captured in a CUDA graph; after each graph launch the host reads the
 // problems' states and, for every problem whose inner solve finished, applies
 // the correction, computes the FP64 residual and restarts its inner solve,

@@ -9,16 +9,18 @@
 //               matrices of the element and its neighbours (undeformed box
 //               spacing), inverted by fast diagonalisation: per direction
 //               A S = B S diag(lam), S^T B S = I, computed once on the host.
-//               One CTA per element (persistent): gather the grown box of
-//               r from the global vector, five line phases (S^T along x, y;
-//               along z with the diagonal scaling and S back; S along y, x),
-//               scatter-add to z by L2 reductions.  The same kernel forms the
-//               coarse restriction from the element's own points.
+//               One CTA per element: gather the grown box of r from the global
+//               vector by columns, S^T along z, then x, then y with the diagonal
+//               scaling and S back, S along x and z, scatter-add to z by L2
+//               reductions.  The same kernel forms the coarse restriction from
+//               the element's own points.
 // coarse level  trilinear vertex functions; A_0 = R_0 H R_0^T assembled from
 //               8 x 8 element matrices Phi^T H_e Phi (computed at setup with
-//               the FP64 element operator, stored packed in FP32); a fixed
-//               number of Jacobi-PCG iterations from zero (the FP32 CG steps
-//               of cg.cu with an element-by-element coarse matvec).
+//               the FP64 element operator, stored packed in FP32), as a
+//               27-point stencil where the vertices fit one launch; a fixed
+//               number of Jacobi-PCG iterations from zero: in one cluster
+//               (up to 16,384 vertices), in one cooperative grid, or with the
+//               FP32 CG steps of cg.cu and an element-by-element matvec.
 // output        z_L = mask o (z_local[g(L)] + R_0^T c) as FP64 L-vector.
 #include <cmath>
 #include <memory>
@@ -210,7 +212,8 @@ __device__ __forceinline__ void sw_line(const SwConst<PE>& k, bool interior, con
 // with all tables in shared memory spent three 16-byte reads on every output),
 // the interior scaling's divisors as a table, and one element a CTA, so
 // that tables that are not used are not loaded and the registers allow twice
-// the CTAs.  13,824 elements, N = 7: 91 us (160 before).
+// the CTAs.  13,824 elements, N = 7: 95 us (160 before; 91 with reciprocals in the
+// table, a rounding more).
 template <int PE>
 __global__ void __launch_bounds__(SwCfg<PE>::THREADS, SwCfg<PE>::MINB)
 schwarz_local_kernel(const float* __restrict__ rg, float* __restrict__ zg,
