@@ -26,8 +26,11 @@
 
 namespace sem {
 
-template <int P, class T, bool FUSE>
-__global__ void __launch_bounds__(LineCfg<P, T>::THREADS, LineCfg<P, T>::MINB)
+// FIELD: a per-point h1 is given (FP32: its column is fetched with G, so that two
+// CTAs fit an SM; one, with more registers, takes up to 38% longer at N = 9, 10)
+template <int P, class T, bool FUSE, bool FIELD>
+__global__ void __launch_bounds__(LineCfg<P, T>::THREADS,
+                                  sizeof(T) == 4 && FIELD ? 2 : LineCfg<P, T>::MINB)
 ax_line_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__ G,
                const T* __restrict__ B, const T* __restrict__ h1f, T h1, T h2,
                const __grid_constant__ DMat<P, T> D, const T* __restrict__ tabg, int E, FuseBox fb,
@@ -48,8 +51,8 @@ ax_line_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__
 #pragma unroll
     for (int k = 0; k < P; ++k) uc[k] = u[base + k * P2];
   }
-  line_element(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
-                     h1f ? h1f + base : nullptr, h1, h2, out);
+  line_element<6, FIELD>(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
+                         h1f + base, h1, h2, out);
   if constexpr (FUSE) {
     // masked points, then the x-pairs of neighbours in this CTA: the faces
     // i = 0 and i = N of every element go through U
@@ -94,7 +97,8 @@ template <int P, class T>
 static void configure_line() {
   using C = LineCfg<P, T>;
   static const bool done = [] {
-    for (auto k : {ax_line_kernel<P, T, true>, ax_line_kernel<P, T, false>})
+    for (auto k : {ax_line_kernel<P, T, true, false>, ax_line_kernel<P, T, false, false>,
+                   ax_line_kernel<P, T, true, true>, ax_line_kernel<P, T, false, true>})
       SEM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
     return true;
   }();
@@ -105,7 +109,8 @@ template <int P, class T>
 static void launch_line_p(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2,
                           const T* h1f, bool fuse, const CGState* st, cudaStream_t s) {
   using C = LineCfg<P, T>;
-  auto kern = fuse ? ax_line_kernel<P, T, true> : ax_line_kernel<P, T, false>;
+  auto kern = h1f ? (fuse ? ax_line_kernel<P, T, true, true> : ax_line_kernel<P, T, false, true>)
+                  : (fuse ? ax_line_kernel<P, T, true, false> : ax_line_kernel<P, T, false, false>);
   configure_line<P, T>();
   DMat<P, T> D;
   for (int a = 0; a < P * P; ++a) D.d[a] = (T)h->Dh[a];

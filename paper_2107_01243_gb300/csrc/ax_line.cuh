@@ -81,11 +81,15 @@ struct LineThread {
 };
 
 // out = (h1 D^T G D + h2 B) u at the k-column: uc the column of u, g, b, h1f the
-// element's G, B and h1 at this thread's (i, j, 0) (h1f may be NULL).  All
+// element's G, B and (FIELD) h1 at this thread's (i, j, 0).  All
 // threads of the CTA call it (act: the thread has an element); U is free once
 // the second barrier is behind.  PREG: components of G an FP32 thread fetches
 // before the forward lines (the rest where they are used).
-template <int PREG = 6, int P, class T, int MOST>
+// FIELD: h1f is given; an FP32 thread fetches its column with G (where it is used its
+// latency shows: FP32 sem_ax / sem_apply, us, late / with G / the kernels this one
+// took the place of: N = 5, 13,824 elements 26 / 19.6 / 23 and 40 / 31 / 37, N = 7, 4,096
+// 22.5 / 15.9 / 16.3 and 28 / 22.5 / 27, N = 9, 5,832 82 / 44 / 45 and 94 / 59 / 64).
+template <int PREG = 6, bool FIELD = false, int P, class T, int MOST>
 __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bool act,
                                              const DMat<P, T>& D, const T (&uc)[P], const T* g,
                                              const T* b, const T* h1f, T h1, T h2, T (&out)[P]) {
@@ -96,7 +100,7 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
   // other CTA hides it (N = 3, cold caches: sem_apply_global on 216 elements 9.7
   // against 11.0 us, sem_apply 11.0 against 11.6); on large grids that costs 1 to 2%
   const bool early_b = PRE && P <= 4 && gridDim.x < 1024;
-  T gr[PRE ? P : 1][6], bk[PRE ? P : 1];
+  T gr[PRE ? P : 1][6], bk[PRE ? P : 1], hk[PRE && FIELD ? P : 1];
   auto fetch_b = [&] {
 #pragma unroll
     for (int k = 0; k < P; ++k) bk[PRE ? k : 0] = __ldcs(b + k * P2);
@@ -108,6 +112,10 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
       for (int k = 0; k < P; ++k)
 #pragma unroll
         for (int c = 0; c < PREG; ++c) gr[k][c] = __ldcs(g + c * P3 + k * P2);
+    }
+    if constexpr (PRE && FIELD) {
+#pragma unroll
+      for (int k = 0; k < P; ++k) hk[k] = __ldcs(h1f + k * P2);
     }
 #pragma unroll
     for (int k = 0; k < P; ++k) t.U[k * PL + t.col] = uc[k];
@@ -127,7 +135,7 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
   if (act) {
     T ut[P];
     line_dots<P, T, false>(uc, D, t.tab, [&](int a, T y) { ut[a] = y; });
-    const bool scale = h1f || h1 != T(1);
+    const bool scale = FIELD || h1 != T(1);
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       const T ur = t.R[k * PL + t.col], us = t.S[k * PL + t.col];
@@ -140,7 +148,7 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
       T ws = fma(g23, ut[k], fma(g22, us, g12 * ur));
       T wk = fma(g33, ut[k], fma(g23, us, g13 * ur));
       if (scale) {
-        const T c = h1f ? __ldcs(h1f + k * P2) : h1;
+        const T c = !FIELD ? h1 : PRE ? hk[PRE && FIELD ? k : 0] : __ldcs(h1f + k * P2);
         wr *= c;
         ws *= c;
         wk *= c;

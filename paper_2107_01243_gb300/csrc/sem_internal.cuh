@@ -186,7 +186,8 @@ struct sem_handle {
   int f64_kernel = SEM_F64_KERNEL_AUTO;     // which FP64 Ax kernel runs
   struct Tune {
     int ax32_ldg = 1;          // 1: FP32 Ax by the line kernel (global loads), 0: bulk copies
-    int ax32_bulk = 0;         // 1: sem_ax takes bulk copies all the same (setup.cu; untuned)
+    int ax32_bulk = 0;         // sem_ax takes bulk copies all the same (setup.cu; untuned):
+                               // 1 always, 2 with a per-point h1
     int ax32_variant = 1;      // bulk-copy variant: (stages, elements per CTA), see ax_tma.cu
     int df_variant = 0;        // double-float Ax: 0 = one stage, 1 = two stages
     int tuned = 0;

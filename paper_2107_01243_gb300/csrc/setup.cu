@@ -437,6 +437,8 @@ extern "C" sem_status sem_setup(const sem_mesh_desc* mesh, int N, int precision_
     // 343 8.2 / 8.6; N = 9 1,728 22.5 / 22.5, 2,744 30.5 / 28.7, 5,832 52.7 / 49.2)
     h->tune.ax32_bulk = (h->P == 4 && h->E <= 1024) || (h->P == 6 && h->E <= 192) ||
                         (h->P == 10 && h->E >= 2500);
+    // with a per-point h1 at N = 7 from 4 M points (13,824 elements 44 / 41 us)
+    if (h->P == 8 && h->nL > (1 << 22)) h->tune.ax32_bulk = 2;
     h->tune.ax32_variant = h->P <= 4 ? 2 : 1;     // 3 stages for small elements, else 2
     gll_host(N, h->xi, h->wq, h->Dh);
 
