@@ -26,8 +26,8 @@
 
 namespace sem {
 
-// FIELD: a per-point h1 is given (FP32: its column is fetched with G, so that two
-// CTAs fit an SM; one, with more registers, takes up to 38% longer at N = 9, 10)
+// FIELD (FP32; FP64 looks at h1f): a per-point h1 is given, its column fetched with G
+// and two CTAs made to fit an SM (one takes up to 38% longer at N = 9, 10)
 template <int P, class T, bool FUSE, bool FIELD>
 __global__ void __launch_bounds__(LineCfg<P, T>::THREADS,
                                   sizeof(T) == 4 && FIELD ? 2 : LineCfg<P, T>::MINB)
@@ -52,7 +52,7 @@ ax_line_kernel(const T* __restrict__ u, T* __restrict__ w, const T* __restrict__
     for (int k = 0; k < P; ++k) uc[k] = u[base + k * P2];
   }
   line_element<6, FIELD>(t, act, D, uc, G + (size_t)(act ? e : 0) * 6 * P3 + t.lam, B + base,
-                         h1f + base, h1, h2, out);
+                         h1f ? h1f + base : nullptr, h1, h2, out);
   if constexpr (FUSE) {
     // masked points, then the x-pairs of neighbours in this CTA: the faces
     // i = 0 and i = N of every element go through U
@@ -97,8 +97,9 @@ template <int P, class T>
 static void configure_line() {
   using C = LineCfg<P, T>;
   static const bool done = [] {
+    constexpr bool F = sizeof(T) == 4;
     for (auto k : {ax_line_kernel<P, T, true, false>, ax_line_kernel<P, T, false, false>,
-                   ax_line_kernel<P, T, true, true>, ax_line_kernel<P, T, false, true>})
+                   ax_line_kernel<P, T, true, F>, ax_line_kernel<P, T, false, F>})
       SEM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
     return true;
   }();
@@ -109,7 +110,8 @@ template <int P, class T>
 static void launch_line_p(const sem_handle* h, const OpData<T>& op, const T* u, T* w, T h1, T h2,
                           const T* h1f, bool fuse, const CGState* st, cudaStream_t s) {
   using C = LineCfg<P, T>;
-  auto kern = h1f ? (fuse ? ax_line_kernel<P, T, true, true> : ax_line_kernel<P, T, false, true>)
+  constexpr bool F = sizeof(T) == 4;
+  auto kern = h1f ? (fuse ? ax_line_kernel<P, T, true, F> : ax_line_kernel<P, T, false, F>)
                   : (fuse ? ax_line_kernel<P, T, true, false> : ax_line_kernel<P, T, false, false>);
   configure_line<P, T>();
   DMat<P, T> D;

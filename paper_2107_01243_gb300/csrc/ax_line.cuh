@@ -81,7 +81,7 @@ struct LineThread {
 };
 
 // out = (h1 D^T G D + h2 B) u at the k-column: uc the column of u, g, b, h1f the
-// element's G, B and (FIELD) h1 at this thread's (i, j, 0).  All
+// element's G, B and h1 at this thread's (i, j, 0) (h1f NULL without; FP32: FIELD tells).  All
 // threads of the CTA call it (act: the thread has an element); U is free once
 // the second barrier is behind.  PREG: components of G an FP32 thread fetches
 // before the forward lines (the rest where they are used).
@@ -135,7 +135,8 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
   if (act) {
     T ut[P];
     line_dots<P, T, false>(uc, D, t.tab, [&](int a, T y) { ut[a] = y; });
-    const bool scale = FIELD || h1 != T(1);
+    const bool field = PRE ? FIELD : h1f != nullptr;
+    const bool scale = field || h1 != T(1);
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       const T ur = t.R[k * PL + t.col], us = t.S[k * PL + t.col];
@@ -148,7 +149,7 @@ __device__ __forceinline__ void line_element(const LineThread<P, T, MOST>& t, bo
       T ws = fma(g23, ut[k], fma(g22, us, g12 * ur));
       T wk = fma(g33, ut[k], fma(g23, us, g13 * ur));
       if (scale) {
-        const T c = !FIELD ? h1 : PRE ? hk[PRE && FIELD ? k : 0] : __ldcs(h1f + k * P2);
+        const T c = !field ? h1 : PRE ? hk[PRE && FIELD ? k : 0] : __ldcs(h1f + k * P2);
         wr *= c;
         ws *= c;
         wk *= c;
