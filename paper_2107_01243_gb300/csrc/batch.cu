@@ -1083,7 +1083,13 @@ extern "C" sem_status sem_batch_solve(sem_batch* bt, const double* const* b_L,
     std::vector<double> rel(n, 0.0);
     const int batch_it = std::max(1, o.check_every);
     auto running = [&](int p) { return phase[p] == RUNNING; };
-    long long launched = bt->glob ? set_groups(bt, own, running) : 0;
+    // every problem runs (an earlier solve may have left some out)
+    long long launched = 0, all = 0;
+    if (bt->glob) {
+      for (int p = 0; p < n; ++p) all += group_count(bt->hp[p]);
+      for (int P = 2; P <= kMaxP; P += 2) launched += bt->ngroups[P];
+      if (launched < all) launched = set_groups(bt, own, running);
+    }
     cudaGraphExec_t& exec = cleanup.ex;
     auto capture = [&] {
       if (!o.use_graph) return;
